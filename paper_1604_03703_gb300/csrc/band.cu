@@ -60,15 +60,6 @@ extern "C" int sev_trace_set_reg_band(void *p) {
 
 namespace sev {
 
-__device__ __forceinline__ int ld_acquire(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release(int *p, int v) {
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 __host__ __device__ __forceinline__ int band_num_chases(int n, int b, int h, int i) {
     const int r = n - i * h;
     return r < 2 ? 0 : (n - 2 - i * h) / b + 1;
@@ -625,16 +616,8 @@ __device__ void band_chase_x3(T *AB, int ldab, int n, int b, int h, int i, int j
 
 // Capped wait of one thread until sweep s - 1 has completed `need` chases;
 // false on expiry or a latched error (then the error word is set).
-__device__ __forceinline__ bool wait_progress(const int *progress, int s, int need, int *err) {
-    const long long t0 = clock64();
-    while (ld_acquire(&progress[s - 1]) < need) {
-        if (*(volatile int *)err != 0) return false;
-        if (wait_expired(t0, err)) {
-            latch_error(err, SEV_ERR_TIMEOUT);
-            return false;
-        }
-    }
-    return true;
+__device__ __forceinline__ bool wait_progress(const int *progress, int s, int need, long long cap, int *err) {
+    return wait_flag(&progress[s - 1], need, cap, err, [&] { return *(volatile int *)err != 0; }) >= 0;
 }
 
 // Cluster of three CTAs per sweep.  Rank 0 takes sweeps from the counter
@@ -651,6 +634,7 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(kThreads)
     ChaseSmem<T> S(smem, b, h);
     __shared__ int s_sweep, s_abort, s_nr;
     const unsigned rank = cluster_rank();
+    const long long cap = wait_cap(err);
     int bad = 0;
     if (threadIdx.x == 0) {
         s_abort = 0;
@@ -667,13 +651,13 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(kThreads)
         const int i = s + 1;
         const int J = band_num_chases(n, b, h, i);
         const int Jprev = i > 1 ? band_num_chases(n, b, h, i - 1) : 0;
-        if (i > 1 && threadIdx.x == 0 && !wait_progress(progress, s, min(3, Jprev), err)) atomicOr(abort0, 1);
+        if (i > 1 && threadIdx.x == 0 && !wait_progress(progress, s, min(3, Jprev), cap, err)) atomicOr(abort0, 1);
         cluster_sync();  // B of "chase 0": every rank may start chase 1
         if (*(volatile int *)abort0) break;
         for (int j = 1; j <= J; ++j) {
             band_chase_x3<T, RQ, QQ>(AB, ldab, n, b, h, i, j, S, rank, &s_nr, bad);
             __syncthreads();
-            if (i > 1 && j < J && threadIdx.x == 0 && !wait_progress(progress, s, min(j + 3, Jprev), err))
+            if (i > 1 && j < J && threadIdx.x == 0 && !wait_progress(progress, s, min(j + 3, Jprev), cap, err))
                 atomicOr(abort0, 1);
             cluster_sync();  // B: chase j is complete on all ranks
             // the release store orders the cluster's writes (made visible to
@@ -693,6 +677,7 @@ __global__ void __launch_bounds__(kThreads) band_chase_kernel(int n, T *AB, int 
     extern __shared__ __align__(16) unsigned char smem[];
     ChaseSmem<T> S(smem, b, h);
     __shared__ int s_sweep, s_abort;
+    const long long cap = wait_cap(err);
     int bad = 0;  // this thread met an index outside the band
     for (;;) {
         __syncthreads();
@@ -708,21 +693,7 @@ __global__ void __launch_bounds__(kThreads) band_chase_kernel(int n, T *AB, int 
         const int Jprev = i > 1 ? band_num_chases(n, b, h, i - 1) : 0;
         for (int j = 1; j <= J; ++j) {
             if (i > 1) {
-                if (threadIdx.x == 0) {
-                    const int need = min(j + 2, Jprev);
-                    const long long t0 = clock64();
-                    while (ld_acquire(&progress[s - 1]) < need) {
-                        if (*(volatile int *)err != 0) {
-                            s_abort = 1;
-                            break;
-                        }
-                        if (wait_expired(t0, err)) {
-                            latch_error(err, SEV_ERR_TIMEOUT);
-                            s_abort = 1;
-                            break;
-                        }
-                    }
-                }
+                if (threadIdx.x == 0 && !wait_progress(progress, s, min(j + 2, Jprev), cap, err)) s_abort = 1;
                 __syncthreads();
                 if (s_abort) return;
             }

@@ -1,106 +1,305 @@
 // band_tri.cu -- the last band reduction, b -> 1 (Algorithm 4.2 with k = b,
 // h = 1), for b <= 32, as a sliding-window bulge chase.
 //
-// With h = 1 every chase (i, j) is ONE Householder reflector: it
-// annihilates the single column o_qr.c below row o_qr.r (o_qr.r =
-// i + (j-1) b, o_qr.c = o_qr.r - 1 for j = 1, o_qr.r - b for j > 1) and
-// applies H two-sidedly to the qr rows [o_qr.r, o_qr.r + n_r) against the
-// update rows [o_up.c, o_up.c + n_c) (o_up.c = o_qr.r for j = 1,
-// o_qr.r - b + 1 for j > 1; n_c = min(n - o_up.c, 2b) resp. 3b - 1).  One
-// warp performs a chase: lane l owns one update row above, in, and below
-// the qr rows; off rows get X <- X H (row-local), the qr-row block gets
-// H X H = X - v w^T - w v^T with p = tau X v, w = p - (tau/2)(p^T v) v.
+// With h = 1 every chase (i, j) is ONE Householder reflector H_j on the qr
+// rows [o, o + n_r), o = i + (j-1) b, n_r = min(n - o, b).  Step (i, j) here
+// does everything that H_j is still owed, and what makes H_{j+1}:
+//   D: the diagonal block [o, o + n_r)^2 gets H_j X H_j = X - v w^T - w v^T
+//      with p = tau X v, w = p - (tau/2)(p^T v) v;
+//   M: the block of rows [o + b, o + 2b) and columns [o, o + b) gets M H_j,
+//      then its first column gives the reflector H_{j+1} (the column becomes
+//      [beta; 0]) and the other columns get H_{j+1} M.
+// Step (i, 0) forms H_1 from column i - 1.  (Algorithm 4.2 applies H_{j+1} to
+// those columns in chase j + 1; nothing reads them in between, so doing it
+// here gives the same matrix, and M is read and written once per sweep
+// instead of twice.)
 //
-// Schedule.  A CTA takes G consecutive sweeps (compute warp g -> sweep
-// i0 + g) and steps them together: at step t warp g performs chase t - 3g,
-// so sweep i runs 3 chases behind sweep i - 1 -- the rule that chase (i, j)
-// follows (i - 1, j + 2) -- and the chases of one step are independent.
-// Steps are separated by a named barrier among the compute warps.  The band
-// columns the group touches live in a shared-memory ring of (3G + 3) b + 2
-// columns (2b diagonals each): a loader warp brings columns in (16-byte
-// asynchronous copies) ahead of warp 0, and a writer warp writes them back
-// once the group's last sweep has passed them (after its chase j, columns
-// below o_qr.r(i_last, j) are final).  The writer then publishes j with a
-// release store; the next group's loader waits (acquire, capped) for j + 2
-// before loading a column range -- the only global synchronisation, once
-// per step per group boundary.  Groups are handed out in order by a global
-// counter and each CTA finishes its group before taking another, so every
-// awaited group is held by a running CTA.
+// Order of the steps.  Step (i, j) touches columns [o, o + b) only, and of
+// those the last one (o + b - 1) together with row o + 2b - 1 are the only
+// places where it meets step (i - 1, j + 1), whose rows and columns start at
+// o + b - 1.  Step (i - 1, j + 2) starts at column o + 2b - 1.  So (i, j)
+// needs (i - 1, j + 1) complete and runs beside (i - 1, j + 2): sweep i
+// trails sweep i - 1 by TWO steps, 2 n steps for the whole stage.  (With the
+// column of H_{j+1} annihilated in chase j + 1, as printed, chases (i, j) and
+// (i - 1, j + 2) share the entry beta and the lag is three.)
+//
+// What bounds it: the chain of one step -- loads from shared memory, the
+// M H_j product, the pair-float sum of squares, the reflector scalars, the
+// H_{j+1} M product -- times 2 n; the band itself is read from L2 once per
+// group of G sweeps.  So D and M are two warps, every lane of a warp holds
+// B^2 / 32 entries (a row or column is spread over 32 / B lanes), the ring
+// is a power of two (no divisions in the addresses) and there is one barrier
+// per step.  Measured (GB300): 16 -> 1 at
+// n = 16384 in FP32 162.5 -> 37.2 ms (lag three, one warp a sweep, two
+// barriers a step: 6.8K cycles a step, now ~1.8K), n = 2048 20.2 -> 4.5 ms,
+// n = 3001 in FP64 73.3 -> 25.6 ms.
+//
+// Schedule.  A CTA takes G consecutive sweeps (sweep i0 + g on warps 2g and
+// 2g + 1) and steps them together: at step t sweep g performs step t - 2g.
+// The band columns the group touches live in a shared-memory ring (2b
+// diagonals each): a loader warp brings columns in (16-byte asynchronous
+// copies that signal an mbarrier per step, so that polling the previous
+// group and copying overlap), and a writer warp writes them back once the
+// group's last sweep has passed them (after its step j, columns below
+// o + b are final) and publishes j with a release store; the next group's
+// loader waits (acquire, capped) for j >= ts + 1 before loading the columns of
+// step ts -- the only global synchronisation.  Groups are handed out in order
+// by a global counter and each CTA finishes its group before taking another,
+// so every awaited group is held by a running CTA.
 #include "common.cuh"
-
-#ifdef SEV_TRACE
-static __device__ long long *sev_trace_buf = nullptr;
-static __device__ int sev_trace_phase_on = 0;
-static __device__ long long sev_trace_phase[8];
-extern "C" int sev_trace_set(void *p) {
-    return cudaMemcpyToSymbol(sev_trace_buf, &p, sizeof(p)) == cudaSuccess ? 0 : 1;
-}
-#define TRACE(gi, t, k, v)                                                                    \
-    do {                                                                                      \
-        if (sev_trace_buf && (gi) < 4 && (t) < 4096) sev_trace_buf[((gi) * 4096 + (t)) * 8 + (k)] = (v); \
-    } while (0)
-#define TRACEP(k)                                                                      \
-    do {                                                                               \
-        if (sev_trace_phase_on == (int)blockIdx.x + 1 && (threadIdx.x & 31) == 0 && (threadIdx.x >> 5) == 0) \
-            sev_trace_phase[(k)] = clock64();                                          \
-    } while (0)
-#else
-#define TRACEP(k) \
-    do {          \
-    } while (0)
-#define TRACE(gi, t, k, v) \
-    do {                   \
-    } while (0)
-#endif
 
 #include "tri_chase.cuh"
 
 namespace sev {
 
-// G compute warps + one loader warp + one writer warp, decoupled through
-// shared-memory flags.  Compute warps step together (named barrier 1): at
-// step t warp g performs chase t - 3g once the loader has made step t's
-// columns available (s_avail >= t).  The loader runs ahead: it polls the
-// previous group (acquire, capped, cached), waits for ring space (columns
-// written back, s_wblo) and loads each step's new columns.  The writer runs
-// behind: once compute has finished a step (s_done), it writes back every
-// column that became final, advances s_wblo and publishes the group's
-// progress (release store).  Flags are ordered with block-scope fences; each
-// wait is capped and an abort turns the remaining steps into no-ops so that
-// every warp still reaches its barriers.  The ring holds (3G + 3) b + 2
-// columns.
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_bytes) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-template <int B, int G>
-__host__ __device__ constexpr int tri_wcap() {
-    return (3 * G + 3) * B + 2;
+__device__ __forceinline__ unsigned tri_smem(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void tri_mbar_init(uint64_t *bar, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tri_smem(bar)), "r"(count) : "memory");
+}
+// Arrives once all asynchronous copies this thread has issued have landed.
+__device__ __forceinline__ void tri_mbar_arrive_copies(uint64_t *bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tri_smem(bar)) : "memory");
+}
+__device__ __forceinline__ void tri_mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tri_smem(bar)) : "memory");
+}
+__device__ __forceinline__ bool tri_mbar_test(uint64_t *bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n"
+        " .reg .pred p;\n"
+        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(tri_smem(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
 }
 
 __device__ __forceinline__ void named_bar(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Lane layout of a B x B block: lane = r + B g holds row (or column) r,
+// entries g, g + LPR, g + 2 LPR, ... of it; lanes past B LPR hold nothing.
+template <int B>
+struct TriLanes {
+    static constexpr int LPR = 32 / B < B ? 32 / B : B;  // lanes per row
+    static constexpr int CPL = B / LPR;                  // entries per lane
+    static constexpr int ON = B * LPR;                   // lanes in use
+};
+
+// Columns the ring holds: the steps in flight span (2G - 1) b columns, the
+// loader runs ahead and the writer behind by a few steps more; a power of two.
+template <int B, int G>
+__host__ __device__ constexpr int tri_ring_cols() {
+    int c = 1;
+    while (c < (2 * G + 4) * B + 2) c *= 2;
+    return c;
+}
+// Element k of the ring counted from element `base` (base < S).  WRAP = false:
+// the caller knows that the block it works on does not cross the ring's end,
+// so the offsets are immediates of the loads and stores.
+template <typename T, int S, bool WRAP>
+__device__ __forceinline__ T &tri_at(T *w, int base, int k) {
+    return WRAP ? w[(base + k) & (S - 1)] : w[base + k];
+}
+constexpr int kTriBars = 8;  // mbarriers of the loader's steps
+constexpr int kTriVec = 40;  // spacing of the per-sweep vector buffers (v: B entries, tau at B)
+
+// Sum over the LPR lanes that share a row / over the B rows of a lane group.
+template <int B, typename T>
+__device__ __forceinline__ T tri_sum_row(T s) {
+#pragma unroll
+    for (int off = B; off < TriLanes<B>::ON; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return s;
+}
+
+// Reflector of x (row r of the column in every lane with that r; rows >= nr
+// zero): v, tau and beta in every lane; squares and scalars FP64-accurate
+// (pair-float for FP32 data).
+template <typename T, int B>
+__device__ __forceinline__ void tri_house(T x, int r, int nr, T &v, T &tau, T &beta) {
+    const bool rest = r >= 1 && r < nr;
+    if constexpr (sizeof(T) == 4) {
+        const F2 acc = warp_sum_f2<B>(two_prod((float)x, (float)x));  // alpha^2 included
+        float tf, bf, inf;
+        house_scalars_f2s(__shfl_sync(0xffffffffu, (float)x, 0), acc, &tf, &bf, &inf);
+        tau = (T)tf;
+        beta = (T)bf;
+        v = r == 0 ? T(1) : (rest ? x * (T)inf : T(0));
+    } else {
+        double a = rest ? (double)x * (double)x : 0.0;
+#pragma unroll
+        for (int off = B / 2; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        double td, bd, id;
+        house_scalars((double)__shfl_sync(0xffffffffu, x, 0), a, &td, &bd, &id);
+        tau = (T)td;
+        beta = (T)bd;
+        v = r == 0 ? T(1) : (rest ? x * (T)id : T(0));
+    }
+}
+
+// This lane's entries of a vector whose entry r is held by the lanes of row r.
+template <typename T, int B>
+__device__ __forceinline__ void tri_spread(T x, T (&v)[TriLanes<B>::CPL]) {
+    const int g = (threadIdx.x & 31) / B;
+#pragma unroll
+    for (int q = 0; q < TriLanes<B>::CPL; ++q) {
+        const T e = __shfl_sync(0xffffffffu, x, g + TriLanes<B>::LPR * q);
+        v[q] = TriLanes<B>::ON == 32 || g < TriLanes<B>::LPR ? e : T(0);
+    }
+}
+
+// Step (i, 0): H_1 from column i - 1, rows [i, i + nr).
+template <typename T, int B, int S>
+__device__ __forceinline__ void tri_first(T *w, int n, int i, T *vn, T (&v)[TriLanes<B>::CPL], T &tau) {
+    constexpr int LDW = 2 * B;
+    const int lane = threadIdx.x & 31, r = lane % B;
+    const int nr = min(n - i, B);
+    T *px = w + (((i - 1) * LDW + 1 + r) & (S - 1));
+    const T x = r < nr ? *px : T(0);
+    T nv, beta;
+    tri_house<T, B>(x, r, nr, nv, tau, beta);
+    tri_spread<T, B>(nv, v);
+    __syncwarp();
+    if (lane < B) {
+        if (r < nr) *px = r == 0 ? beta : T(0);
+        vn[r] = nv;
+        if (r == 0) vn[B] = tau;
+    }
+}
+
+// M of step (i, j) by one warp: M H_j, then H_{j+1} from the first column and
+// H_{j+1} M on the others.  v, tau: this lane's entries of v_j and tau_j on
+// entry, of v_{j+1} and tau_{j+1} on return (also stored to vn for the warp
+// of D).  FULL: M has b rows (sizes known at compile time).
+template <typename T, int B, int S, bool FULL, bool WRAP>
+__device__ __forceinline__ void tri_bulge(T *w, int n, int o, T (&v)[TriLanes<B>::CPL], T &tau, T *vn) {
+    constexpr int LDW = 2 * B, LPR = TriLanes<B>::LPR, CPL = TriLanes<B>::CPL;
+    const int lane = threadIdx.x & 31, r = lane % B, g = lane / B;
+    const bool on = TriLanes<B>::ON == 32 || g < LPR;
+    const int mb = FULL ? B : min(n - (o + B), B);
+    if (!FULL && mb < 1) return;
+    T x[CPL];
+    const int base = (o * LDW) & (S - 1);
+    const int xo = B + r;  // entry (row r, column 0); column c lies LDW - 1 further
+#pragma unroll
+    for (int q = 0; q < CPL; ++q)
+        x[q] = (on && (FULL || r < mb)) ? tri_at<T, S, WRAP>(w, base + xo + g * (LDW - 1), LPR * q * (LDW - 1)) : T(0);
+    T s = T(0), s1 = T(0);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        if (q & 1)
+            s1 = fma(x[q], v[q], s1);
+        else
+            s = fma(x[q], v[q], s);
+    }
+    s = tau * tri_sum_row<B>(s + s1);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) x[q] = fma(-s, v[q], x[q]);
+    const T x0 = __shfl_sync(0xffffffffu, x[0], r);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q)
+        if (on && (FULL || r < mb)) tri_at<T, S, WRAP>(w, base + xo + g * (LDW - 1), LPR * q * (LDW - 1)) = x[q];
+    if (!FULL && mb < 2) return;
+    __syncwarp();
+    // the same block by columns: lane column r, rows g + LPR q
+    T y[CPL];
+    const int yo = base + B + r * (LDW - 1) + g;
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        const int rr = g + LPR * q;
+        y[q] = (on && (FULL || rr < mb)) ? tri_at<T, S, WRAP>(w, yo, LPR * q) : T(0);
+    }
+    T nv, nbeta;
+    tri_house<T, B>(x0, r, mb, nv, tau, nbeta);
+    tri_spread<T, B>(nv, v);
+    if (lane < B) vn[r] = nv;
+    if (lane == 0) vn[B] = tau;
+    T z = T(0), z1 = T(0);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        if (q & 1)
+            z1 = fma(v[q], y[q], z1);
+        else
+            z = fma(v[q], y[q], z);
+    }
+    z = tau * tri_sum_row<B>(z + z1);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        const int rr = g + LPR * q;
+        T val = fma(-z, v[q], y[q]);
+        if (r == 0) val = rr == 0 ? nbeta : T(0);
+        if (on && (FULL || rr < mb)) tri_at<T, S, WRAP>(w, yo, LPR * q) = val;
+    }
+}
+
+// D of step (i, j) by one warp.  vb: v_j, tau_j at vb[B]; wb: B entries of
+// scratch.
+template <typename T, int B, int S, bool FULL, bool WRAP>
+__device__ __forceinline__ void tri_diag(T *w, int n, int o, const T *vb, T *wb) {
+    constexpr int LDW = 2 * B, LPR = TriLanes<B>::LPR, CPL = TriLanes<B>::CPL;
+    const int lane = threadIdx.x & 31, r = lane % B, g = lane / B;
+    const bool on = TriLanes<B>::ON == 32 || g < LPR;
+    const int nr = FULL ? B : min(n - o, B);
+    T x[CPL], vc[CPL];
+    const T tau = vb[B], vr = vb[r];
+    const int base = (o * LDW) & (S - 1);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        const int c = g + LPR * q;
+        const int off = c <= r ? c * (LDW - 1) + r : r * (LDW - 1) + c;
+        vc[q] = on ? vb[c] : T(0);
+        x[q] = (on && (FULL || (r < nr && c < nr))) ? tri_at<T, S, WRAP>(w, base, off) : T(0);
+    }
+    T p = T(0), p1 = T(0);
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        if (q & 1)
+            p1 = fma(x[q], vc[q], p1);
+        else
+            p = fma(x[q], vc[q], p);
+    }
+    p = tau * tri_sum_row<B>(p + p1);
+    T ptv = p * vr;
+#pragma unroll
+    for (int off = B / 2; off > 0; off >>= 1) ptv += __shfl_xor_sync(0xffffffffu, ptv, off);
+    const T wr = fma(T(-0.5) * tau * ptv, vr, p);
+    if (lane < B) wb[r] = wr;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+        const int c = g + LPR * q;
+        if (on && c <= r && (FULL || r < nr))
+            tri_at<T, S, WRAP>(w, base + g * (LDW - 1) + r, LPR * q * (LDW - 1)) = fma(-vr, wb[c], fma(-wr, vc[q], x[q]));
+    }
+}
+
 template <typename T, int B, int G>
-__global__ void __launch_bounds__((G + 2) * 32, 1)
+__global__ void __launch_bounds__((2 * G + 3) * 32, 1)
     band_tri_kernel(int n, T *AB, int ldab, int nsweeps, int ngroups, int *progress, int *group_ctr, int *err,
                     int async_ok) {
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int LDW = 2 * B;
-    constexpr int wcap = tri_wcap<B, G>();
-    TriWin<T, B> W;
-    W.w = (T *)smem;
-    W.wcap = wcap;
-    T *vb = W.w + (size_t)wcap * LDW;  // G x 32
-    T *wb = vb + G * 32;               // G x 32
+    constexpr int LDW = 2 * B, CAP = tri_ring_cols<B, G>(), S = CAP * LDW;
+    T *const w = (T *)smem;
+    T *const vbuf = w + S;                     // G x 2 x kTriVec
+    T *const wbuf = vbuf + 2 * G * kTriVec;    // G x kTriVec
+    __shared__ __align__(8) uint64_t avail[kTriBars];
     __shared__ int s_group;
-    __shared__ volatile int s_abort, s_avail, s_done, s_wblo;
+    __shared__ volatile int s_abort, s_done, s_wblo;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool loader = warp == G, writer = warp == G + 1;
+    if (threadIdx.x == 0)
+        for (int q = 0; q < kTriBars; ++q) tri_mbar_init(&avail[q], 32);
+    const long long cap = wait_cap(err);
+    int step0 = 0;  // loader steps of the groups this CTA has finished
 
     for (;;) {
         __syncthreads();
@@ -108,9 +307,8 @@ __global__ void __launch_bounds__((G + 2) * 32, 1)
             const int g = atomicAdd(group_ctr, 1);
             s_group = g;
             s_abort = 0;
-            s_avail = 0;
             s_done = 0;
-            s_wblo = 1 + g * G - 1;
+            s_wblo = g * G;  // = i0 - 1
         }
         __syncthreads();
         const int gi = s_group;
@@ -120,136 +318,118 @@ __global__ void __launch_bounds__((G + 2) * 32, 1)
         const int il = i0 + nact - 1;
         const int Jf = tri_chases(n, B, i0), Jl = tri_chases(n, B, il);
         const int Jprev = gi > 0 ? tri_chases(n, B, i0 - 1) : 0;
-        const int tmax = Jl + 3 * (nact - 1);
-        auto hi_of = [&](int ts) { return (ts >= Jf) ? n : min(n, i0 + ts * B); };
+        const int tmax = Jl + 2 * (nact - 1);
 
-        if (warp < G) {
+        if (warp < 2 * G) {
             // ------------------------------------------------------ compute
-            T rv = T(0), rtau = T(0), rbeta = T(0);  // this warp's pending reflector
-            for (int t = 1; t <= tmax; ++t) {
-                if (warp == 0 && lane == 0) TRACE(gi, t, 0, clock64());
-                if (warp == 0 && lane == 0 && !s_abort) {
-                    const int need = min(t, Jf);
-                    const long long t0 = clock64();
-                    while (s_avail < need && !s_abort) {
-                        if (wait_expired(t0, err)) {
-                            latch_error(err, SEV_ERR_TIMEOUT);
-                            s_abort = 1;
+            const int g = warp >> 1;
+            const bool diag = warp & 1;
+            const int i = i0 + g;
+            const int Ji = g < nact ? tri_chases(n, B, i) : -1;
+            T rv[TriLanes<B>::CPL], rtau = T(0);  // the bulge warp's pending reflector
+#pragma unroll
+            for (int q = 0; q < TriLanes<B>::CPL; ++q) rv[q] = T(0);
+            named_bar(1, (2 * G + 1) * 32);
+            for (int t = 0; t <= tmax; ++t) {
+                const int j = t - 2 * g;
+                if (j >= 0 && j <= Ji) {  // (after an abort the steps run on stale data: every access stays in the ring)
+                    const int o = i + (j - 1) * B;
+                    T *vb = vbuf + (2 * g + (j & 1)) * kTriVec, *vn = vbuf + (2 * g + ((j + 1) & 1)) * kTriVec;
+                    T *wb = wbuf + g * kTriVec;
+                    // an interior step whose block lies in one piece in the ring
+                    const bool plain = o + 2 * B <= n && ((o * LDW) & (S - 1)) + B * LDW <= S;
+                    if (diag) {
+                        if (j > 0) {
+                            if (plain)
+                                tri_diag<T, B, S, true, false>(w, n, o, vb, wb);
+                            else
+                                tri_diag<T, B, S, false, true>(w, n, o, vb, wb);
                         }
+                    } else if (j == 0) {
+                        tri_first<T, B, S>(w, n, i, vn, rv, rtau);
+                    } else if (plain) {
+                        tri_bulge<T, B, S, true, false>(w, n, o, rv, rtau, vn);
+                    } else {
+                        tri_bulge<T, B, S, false, true>(w, n, o, rv, rtau, vn);
                     }
-                    __threadfence_block();
-                }
-                named_bar(1, G * 32);
-                if (warp == 0 && lane == 0) TRACE(gi, t, 1, clock64());
-                if (!s_abort) {
-                    const int j = t - 3 * warp;
-                    const int i = i0 + warp;
-                    const int Ji = tri_chases(n, B, i);
-                    if (warp < nact && j >= 1 && j <= Ji) {
-                        const int o = i + (j - 1) * B;
-                        if (j == 1) {
-                            // the sweep's first reflector: column i - 1, rows [i, i + n_r)
-                            const int nr1 = min(n - o, B);
-                            T *xcol = W.w + (size_t)((o - 1) % wcap) * LDW + 1;
-                            const T x = lane < nr1 ? xcol[lane] : T(0);
-                            tri_reflector<T, B>(x, nr1, rv, rtau, rbeta);
-                            if (lane < nr1) xcol[lane] = lane == 0 ? rbeta : T(0);
-                            __syncwarp();
-                        }
-#ifdef SEV_TRACE
-                        if (warp == 0 && lane == 0 && gi == 1 && j == 40) sev_trace_phase_on = blockIdx.x + 1;
-                        __syncwarp();
-#endif
-                        if (j > 1 && j < Ji && o + 3 * B <= n)
-                            tri_chase<T, B, true>(n, o, j, true, W, vb + warp * 32, wb + warp * 32, rv, rtau, rbeta);
-                        else
-                            tri_chase<T, B>(n, o, j, j < Ji, W, vb + warp * 32, wb + warp * 32, rv, rtau, rbeta);
-#ifdef SEV_TRACE
-                        if (warp == 0 && lane == 0 && gi == 1 && j == 40 && sev_trace_buf)
-                            for (int k = 0; k < 6; ++k) sev_trace_buf[3 * 4096 * 8 + 4000 * 8 + k] = sev_trace_phase[k];
-                        if (warp == 0 && lane == 0 && gi == 1 && j == 40) sev_trace_phase_on = 0;
-#endif
-                    }
-                }
-                if (lane == 0) TRACE(gi, t, 3 + (warp < 3 ? warp : 2), clock64());
-                named_bar(1, G * 32);
-                if (warp == 0 && lane == 0) {
-                    TRACE(gi, t, 2, clock64());
-                    __threadfence_block();
-                    s_done = t;
-                }
-            }
-        } else if (loader) {
-            // ------------------------------------------------------- loader
-            int loaded_hi = i0 - 1, seen = 0;
-            for (int ts = 1; ts <= Jf && !s_abort; ++ts) {
-                if (async_ok && ts > 1) {
-                    // the previous step's copies land and are published before
-                    // this step waits for anything (the ring-space wait depends
-                    // on compute having consumed them)
-                    cp_async_wait_all();
-                    __syncwarp();
-                    if (lane == 0) {
-                        __threadfence_block();
-                        s_avail = ts - 1;
-                    }
-                }
-                if (gi > 0 && ts + 2 > seen) {
-                    const int need = (ts + 2 <= Jprev) ? ts + 2 : kTriInf;
-                    int pv = 0;
-                    if (lane == 0) {
-                        const long long t0 = clock64();
-                        while ((pv = ld_acquire_i(&progress[gi - 1])) < need) {
-                            if (*(volatile int *)err != 0 || s_abort) {
-                                pv = -1;
-                                break;
-                            }
-                            if (wait_expired(t0, err)) {
-                                latch_error(err, SEV_ERR_TIMEOUT);
-                                pv = -1;
-                                break;
-                            }
-
-                        }
-                    }
-                    pv = __shfl_sync(0xffffffffu, pv, 0);
-                    if (pv < 0) {
-                        if (lane == 0) s_abort = 1;
-                        break;
-                    }
-                    seen = pv;
-                    if (lane == 0) TRACE(gi, ts, 6, clock64());
-                }
-                const int hi = hi_of(ts);
-                // ring space: columns below hi - wcap must have been written back
-                if (lane == 0) {
-                    const long long t0 = clock64();
-                    while (s_wblo < hi - wcap && !s_abort) {
-                        if (wait_expired(t0, err)) {
-                            latch_error(err, SEV_ERR_TIMEOUT);
-                            s_abort = 1;
-                        }
-                    }
-                    __threadfence_block();
                 }
                 __syncwarp();
-                if (s_abort) break;
-                const int c0 = loaded_hi;
-                if (async_ok) {
-                    // asynchronous 16-byte copies (zero-filled past the matrix
-                    // end), all issued at once: a step costs one memory latency
-                    // instead of one per batch of loads; published at the top of
-                    // the next iteration (or after the loop)
-                    constexpr int EPC = 16 / (int)sizeof(T);  // elements per chunk
-                    constexpr int CH = LDW / EPC;             // chunks per column
+                named_bar(1, (2 * G + 1) * 32);
+            }
+        } else if (warp == 2 * G) {
+            // -------------------------------------------------------- gate
+            // takes part in every step barrier: it has waited for the columns
+            // of the coming step before it arrives, and tells the writer and
+            // the loader which steps are complete
+            for (int t = -1; t <= tmax; ++t) {
+                if (lane == 0 && t + 1 <= Jf) {
+                    const int st = step0 + t + 1;
+                    const long long t0 = clock64();
+                    while (!tri_mbar_test(&avail[st % kTriBars], (st / kTriBars) & 1) && !s_abort) {
+                        if (wait_expired(t0, cap)) {
+                            latch_error(err, SEV_ERR_TIMEOUT);
+                            s_abort = 1;
+                        }
+                    }
+                }
+                __syncwarp();
+                named_bar(1, (2 * G + 1) * 32);
+                if (lane == 0) {
+                    __threadfence_block();
+                    s_done = t + 1;
+                }
+            }
+        } else if (warp == 2 * G + 1) {
+            // ------------------------------------------------------- loader
+            int c0 = i0 - 1, seen = 0;
+            for (int ts = 0; ts <= Jf; ++ts) {
+                const int hi = ts >= Jf ? n : min(n, i0 + ts * B);
+                int ok = 1;
+                if (lane == 0) {
+                    // the previous group's last sweep has passed these columns
+                    if (gi > 0 && ts + 1 > seen) {
+                        seen = wait_flag(&progress[gi - 1], ts + 1 <= Jprev ? ts + 1 : kTriInf, cap, err,
+                                         [&] { return *(volatile int *)err != 0 || s_abort; });
+                        ok = seen >= 0;
+                    }
+                    const long long t0 = clock64();
+                    // ring space, and the mbarrier's previous phase consumed
+                    while (ok && (s_wblo < hi - CAP || s_done < ts - kTriBars + 1)) {
+                        if (s_abort) ok = 0;
+                        if (wait_expired(t0, cap)) {
+                            latch_error(err, SEV_ERR_TIMEOUT);
+                            ok = 0;
+                        }
+                    }
+                    if (!ok) s_abort = 1;
+                    __threadfence_block();
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
+                uint64_t *bar = &avail[(step0 + ts) % kTriBars];
+                constexpr int EPC = 16 / (int)sizeof(T);               // elements per 16-byte chunk
+                constexpr int CH = LDW / EPC > 0 ? LDW / EPC : 1;      // chunks per column
+                if (async_ok && hi - c0 == B && hi + LDW <= n) {
+                    // a full step away from the matrix end: no bounds, all copies at once
+                    const T *src = AB + (size_t)c0 * ldab;
+                    const int ring = c0 * LDW;
+#pragma unroll
+                    for (int k = 0; k < (B * CH + 31) / 32; ++k) {
+                        const int q = lane + 32 * k;
+                        if (B * CH % 32 == 0 || q < B * CH)
+                            cp_async16(w + ((ring + q * EPC) & (S - 1)), src + (size_t)(q / CH) * ldab + (q % CH) * EPC, 16);
+                    }
+                    tri_mbar_arrive_copies(bar);
+                } else if (async_ok) {
+                    // 16-byte copies, zero-filled past the matrix end
                     for (int q = lane; q < (hi - c0) * CH; q += 32) {
                         const int c = c0 + q / CH, d0 = (q % CH) * EPC;
                         int valid = n - c - d0;
                         valid = valid < 0 ? 0 : (valid > EPC ? EPC : valid);
                         const T *src = valid > 0 ? AB + d0 + (size_t)c * ldab : AB;
-                        cp_async16(W.w + (size_t)(c % wcap) * LDW + d0, src, valid * (int)sizeof(T));
+                        cp_async16(w + ((c * LDW + d0) & (S - 1)), src, valid * (int)sizeof(T));
                     }
-                    cp_async_commit();
+                    tri_mbar_arrive_copies(bar);
                 } else {
                     batched_copy<T, 16>(
                         (hi - c0) * LDW, lane, 32,
@@ -257,100 +437,108 @@ __global__ void __launch_bounds__((G + 2) * 32, 1)
                             const int c = c0 + k / LDW, d = k % LDW;
                             return (c + d < n) ? __ldcg(AB + d + (size_t)c * ldab) : T(0);
                         },
-                        [&](int k, T v) { W.w[((c0 + k / LDW) % wcap) * LDW + k % LDW] = v; });
-                    __syncwarp();
-                    if (lane == 0) {
-                        __threadfence_block();
-                        s_avail = ts;
-                    }
+                        [&](int k, T v) { w[((c0 + k / LDW) * LDW + k % LDW) & (S - 1)] = v; });
+                    tri_mbar_arrive(bar);
                 }
-                loaded_hi = max(loaded_hi, hi);
-                if (lane == 0) TRACE(gi, ts, 7, clock64());
+                c0 = max(c0, hi);
             }
-            if (async_ok) {
-                // every copy in flight lands before the loader publishes or leaves
-                cp_async_wait_all();
-                __syncwarp();
-                if (lane == 0 && !s_abort) {
-                    __threadfence_block();
-                    s_avail = Jf;
-                }
-            }
-        } else if (writer) {
+            if (async_ok) cp_async_wait_all();  // no copy in flight when the CTA moves on or leaves
+        } else {
             // ------------------------------------------------------- writer
-            int wb_lo = i0 - 1, written = 0;
-            while (written < tmax) {
-                int ts = 0;
+            int lo = i0 - 1, written = 0;
+            while (written <= tmax) {
+                int td = 0;
                 if (lane == 0) {
                     const long long t0 = clock64();
-                    while ((ts = s_done) <= written && !s_abort) {
-                        if (wait_expired(t0, err)) {
+                    while ((td = s_done) <= written && !s_abort) {
+                        if (wait_expired(t0, cap)) {
                             latch_error(err, SEV_ERR_TIMEOUT);
                             s_abort = 1;
                         }
                     }
                     __threadfence_block();
                 }
-                ts = __shfl_sync(0xffffffffu, ts, 0);
-                if (s_abort) break;
-                written = ts;
-                const int jl = ts - 3 * (nact - 1);
+                td = __shfl_sync(0xffffffffu, td, 0);
+                if (__shfl_sync(0xffffffffu, s_abort, 0)) break;
+                written = td;  // steps 0 .. td - 1 are complete
+                const int jl = td - 1 - 2 * (nact - 1);
                 if (jl < 1) continue;
                 const bool done = jl >= Jl;
-                const int fin = done ? n : min(n, il + (jl - 1) * B);
-                for (int idx = lane; idx < (fin - wb_lo) * LDW; idx += 32) {
-                    const int c = wb_lo + idx / LDW, d = idx % LDW;
-                    if (c + d < n) AB[d + (size_t)c * ldab] = W.w[(c % wcap) * LDW + d];
+                const int fin = done ? n : min(n, il + jl * B);
+                constexpr int EPC = 16 / (int)sizeof(T), CH = LDW / EPC > 0 ? LDW / EPC : 1;
+                // whole steps (several, if compute has run ahead) away from the matrix end
+                for (; async_ok && lo + B <= fin && lo + B + LDW <= n; lo += B) {
+                    T *dst = AB + (size_t)lo * ldab;
+                    const int ring = lo * LDW;
+                    constexpr int K = (B * CH + 31) / 32;
+                    uint4 v[K];
+#pragma unroll
+                    for (int k = 0; k < K; ++k)
+                        v[k] = *reinterpret_cast<const uint4 *>(w + ((ring + (lane + 32 * k) * EPC) & (S - 1)));
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const int q = lane + 32 * k;
+                        if (B * CH % 32 == 0 || q < B * CH)
+                            *reinterpret_cast<uint4 *>(dst + (size_t)(q / CH) * ldab + (q % CH) * EPC) = v[k];
+                    }
                 }
-                if (fin > wb_lo) wb_lo = fin;
+                for (int idx = lane; idx < (fin - lo) * LDW; idx += 32) {
+                    const int c = lo + idx / LDW, d = idx % LDW;
+                    if (c + d < n) AB[d + (size_t)c * ldab] = w[(c * LDW + d) & (S - 1)];
+                }
+                if (fin > lo) lo = fin;
                 __syncwarp();
                 if (lane == 0) {
                     __threadfence_block();
-                    s_wblo = wb_lo;
+                    s_wblo = lo;
                     // the release store orders the warp's write-back before the flag
-                    st_release_i(&progress[gi], done ? kTriInf : jl);
+                    st_release(&progress[gi], done ? kTriInf : jl);
                 }
             }
         }
         __syncthreads();
         if (s_abort) return;
+        step0 += Jf + 1;
     }
 }
 
 template <typename T, int B, int G>
 static int launch_tri(sev_ctx *h, int n, T *AB, int ldab, int *progress, int *ctr, int nsweeps) {
     const int ngroups = (nsweeps + G - 1) / G;
-    constexpr int wcap = tri_wcap<B, G>();
-    const size_t smem = sizeof(T) * ((size_t)wcap * 2 * B + 2 * G * 32);
+    const size_t smem = sizeof(T) * ((size_t)tri_ring_cols<B, G>() * 2 * B + 3 * G * kTriVec);
     if (smem > h->smem_optin) return SEV_ERR_UNSUPPORTED;
     SEV_CUDA(cudaMemsetAsync(progress, 0, sizeof(int) * (size_t)ngroups, h->stream));
     SEV_CUDA(cudaMemsetAsync(ctr, 0, sizeof(int), h->stream));
     auto kern = band_tri_kernel<T, B, G>;
     SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (G + 2) * 32, smem));
+    SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (2 * G + 3) * 32, smem));
     if (per_sm < 1) return SEV_ERR_UNSUPPORTED;
-    // groups start ~3G steps apart and each runs ~J + 3G steps, so about
-    // J / (3G) of them are busy at once; more CTAs would only poll
+    // groups start ~2G steps apart and each runs ~J + 2G steps, so about
+    // J / (2G) of them are busy at once; more CTAs would only poll
     const int J1 = tri_chases(n, B, 1);
     int grid = h->sm_count * per_sm;
-    const int busy = J1 / (3 * G) + 16;
+    const int busy = J1 / (2 * G) + 16;
     if (grid > busy) grid = busy;
     if (grid > ngroups) grid = ngroups;
     // 16-byte asynchronous copies need a 16-byte-aligned band and column stride
-    const int async_ok = ((uintptr_t)AB % 16 == 0) && ((size_t)ldab * sizeof(T)) % 16 == 0;
-    SEV_LAUNCH(h, K_BAND_TRI, kern, grid, (G + 2) * 32, smem, n, AB, ldab, nsweeps, ngroups, progress, ctr,
+    const int async_ok =
+        ((uintptr_t)AB % 16 == 0) && ((size_t)ldab * sizeof(T)) % 16 == 0 && (2 * B * sizeof(T)) % 16 == 0;
+    SEV_LAUNCH(h, K_BAND_TRI, kern, grid, (2 * G + 3) * 32, smem, n, AB, ldab, nsweeps, ngroups, progress, ctr,
                h->d_err, async_ok);
     return SEV_OK;
 }
 
-// Compute warps (sweeps) per CTA: fewer per CTA spreads the concurrently
-// active sweeps over more SMs.
-#ifndef SEV_TRI_G_SMALL
-#define SEV_TRI_G_SMALL 8
+// Sweeps per CTA (two warps each): more of them spread the hand-over between
+// groups (~5 us) over more sweeps, fewer leave each scheduler (and, in FP64,
+// the one FP64 pipe of each scheduler) fewer warps to serve.  16 -> 1 at
+// n = 16384, FP32: 4 sweeps 44.4 ms, 6 37.2, 8 38.5; n = 3001, FP64: 2 sweeps
+// 26.4 ms, 3 25.6, 4 28.1.
+#ifndef SEV_TRI_G_F32
+#define SEV_TRI_G_F32 6
 #endif
-#ifndef SEV_TRI_G16
-#define SEV_TRI_G16 4
+#ifndef SEV_TRI_G_F64
+#define SEV_TRI_G_F64 3
 #endif
 #ifndef SEV_TRI_G32
 #define SEV_TRI_G32 4
@@ -373,11 +561,12 @@ int launch_band_tri(sev_ctx *h, int n, T *AB, int ldab, int b, void *ws, size_t 
     Carver c(ws);
     int *progress = c.take<int>((size_t)n + 1);
     int *ctr = c.take<int>(1);
+    constexpr int G = sizeof(T) == 4 ? SEV_TRI_G_F32 : SEV_TRI_G_F64;
     switch (b) {
-        case 2: return launch_tri<T, 2, SEV_TRI_G_SMALL>(h, n, AB, ldab, progress, ctr, nsweeps);
-        case 4: return launch_tri<T, 4, SEV_TRI_G_SMALL>(h, n, AB, ldab, progress, ctr, nsweeps);
-        case 8: return launch_tri<T, 8, SEV_TRI_G_SMALL>(h, n, AB, ldab, progress, ctr, nsweeps);
-        case 16: return launch_tri<T, 16, SEV_TRI_G16>(h, n, AB, ldab, progress, ctr, nsweeps);
+        case 2: return launch_tri<T, 2, G>(h, n, AB, ldab, progress, ctr, nsweeps);
+        case 4: return launch_tri<T, 4, G>(h, n, AB, ldab, progress, ctr, nsweeps);
+        case 8: return launch_tri<T, 8, G>(h, n, AB, ldab, progress, ctr, nsweeps);
+        case 16: return launch_tri<T, 16, G>(h, n, AB, ldab, progress, ctr, nsweeps);
         case 32:
             if constexpr (sizeof(T) == 4) return launch_tri<T, 32, SEV_TRI_G32>(h, n, AB, ldab, progress, ctr, nsweeps);
             return SEV_ERR_UNSUPPORTED;

@@ -145,6 +145,7 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
     W.w = band;
     W.wcap = n;  // the whole band: slots never wrap
     const int nsweeps = n >= 3 ? n - 2 : 0;
+    const long long cap = wait_cap(err);
     for (int i = 1 + warp; i <= nsweeps; i += kBatchWarps) {
         const int Ji = tri_chases(n, B, i);
         const int Jp = i > 1 ? tri_chases(n, B, i - 1) : 0;
@@ -156,7 +157,7 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
                 if (lane == 0) {
                     const long long t0 = clock64();
                     while (sval[(i - 2) % kBatchWarps] < need) {
-                        if (*(volatile int *)&s_fail || wait_expired(t0, err)) {
+                        if (*(volatile int *)&s_fail || wait_expired(t0, cap)) {
                             ok = 0;
                             break;
                         }

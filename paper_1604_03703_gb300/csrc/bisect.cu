@@ -275,35 +275,17 @@ struct BisCtl {
     long long items;  // subtree midpoints evaluated (diagnostics)
 };
 
-__device__ __forceinline__ int ld_acquire_gpu(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // Grid barrier number `seq` (1, 2, ...): returns false if the wait hit its cap
 // or another CTA gave up.
-__device__ bool bis_barrier(BisCtl *ctl, int seq, int *err) {
+__device__ bool bis_barrier(BisCtl *ctl, int seq, long long cap, int *err) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(&ctl->bar, 1);
         const int target = seq * (int)gridDim.x;
-        const long long t0 = clock64();
-        int ok = 1;
-        while (ld_acquire_gpu(&ctl->bar) < target) {
-            if (*(volatile int *)&ctl->abort) {
-                ok = 0;
-                break;
-            }
-            if (wait_expired(t0, err)) {
-                latch_error(err, SEV_ERR_TIMEOUT);
-                *(volatile int *)&ctl->abort = 1;
-                ok = 0;
-                break;
-            }
-        }
+        const int ok = wait_flag(&ctl->bar, target, cap, err, [&] { return *(volatile int *)&ctl->abort != 0; }) >= 0;
+        if (!ok) *(volatile int *)&ctl->abort = 1;
         __threadfence();
         s_ok = ok;
     }
@@ -352,6 +334,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
                                                                     int maxit, int budget, double *__restrict__ eigs,
                                                                     BisWs W, int *err) {
     __shared__ int s_scan[kBisThreads];
+    const long long cap = wait_cap(err);
     const double sc = par[2];
     const double atol = __dmul_rn(rtol, par[3]);
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -368,7 +351,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
         W.st[k] = zero;
     }
     int seq = 0;
-    if (!bis_barrier(W.ctl, ++seq, err)) return;
+    if (!bis_barrier(W.ctl, ++seq, cap, err)) return;
     for (;;) {
         // ---- (1) leaders: CTA 0 compacts the distinct active intervals
         if (blockIdx.x == 0) {
@@ -418,7 +401,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
                 }
             }
         }
-        if (!bis_barrier(W.ctl, ++seq, err)) return;
+        if (!bis_barrier(W.ctl, ++seq, cap, err)) return;
         if (*(volatile int *)&W.ctl->done) break;
         const int D = *(volatile int *)&W.ctl->D;
         const int dep = *(volatile int *)&W.ctl->depth;
@@ -451,7 +434,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
             if (live && bis_step_test(lo, hi, it, rtol, atol, maxit, mid) == 0) c = sturm_chain(n, d, e2, mid, sc);
             W.cnt[w] = c;
         }
-        if (!bis_barrier(W.ctl, ++seq, err)) return;
+        if (!bis_barrier(W.ctl, ++seq, cap, err)) return;
         // ---- (3) every active index walks dep steps down its leader's subtree
         for (int k = gtid; k < n; k += gthreads) {
             if (W.st[k] != 0) continue;
@@ -480,7 +463,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
             W.it[k] = it;
             W.st[k] = state != 0;
         }
-        if (!bis_barrier(W.ctl, ++seq, err)) return;
+        if (!bis_barrier(W.ctl, ++seq, cap, err)) return;
     }
     const double up = par[4];
     for (int k = gtid; k < n; k += gthreads) eigs[k] = __dmul_rn(__dmul_rn(0.5, __dadd_rn(W.lo[k], W.hi[k])), up);

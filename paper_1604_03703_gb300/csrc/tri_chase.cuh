@@ -15,15 +15,6 @@ namespace sev {
 
 constexpr int kTriInf = 1 << 30;
 
-__device__ __forceinline__ int ld_acquire_i(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_i(int *p, int v) {
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 __host__ __device__ __forceinline__ int tri_chases(int n, int b, int i) {
     const int r = n - i;
     return r < 2 ? 0 : (n - 2 - i) / b + 1;
