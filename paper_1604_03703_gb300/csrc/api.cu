@@ -20,7 +20,7 @@ const char *const kKernelNames[K_COUNT] = {
     "tsqr_leaf_qr", "tsqr_node_qr", "tsqr_node_apply", "tsqr_leaf_apply", "recon_lu",
     "recon_u2",     "symm",         "vform_xt",        "vform_utx",       "vform_reduce",
     "vform_v",      "syr2k",        "split_bf16",      "syr2k_tc",        "batch",
-    "check_finite", "misc"};
+    "check_finite", "misc",         "panel_coop"};
 
 static cudaEvent_t pool_get(sev_ctx *h) {
     if (!h->event_pool.empty()) {

@@ -1,0 +1,618 @@
+// panel_coop.cu -- the panel factorisation of the full-to-band reduction (the
+// QR step of Algorithm 4.1) by the whole GPU at once: one cooperative kernel
+// holds the N x b panel in registers, 32 RT rows per CTA, and runs the
+// Householder QR column by column with ONE exchange between the CTAs per
+// column.
+//
+// Why not the tree (Algorithm 3.2).  A tree of leaf and node QRs pays a chain
+// of b columns at every one of its ~log2(N / 256) + 1 levels, then the way
+// down, then the reconstruction of (U, T) from the explicit Q.  Its point is to
+// exchange data once per level instead of once per column, which pays when an
+// exchange costs much more than a column; between the SMs of one GPU an
+// exchange through L2 takes ~0.7 us and a column of a leaf or node QR
+// ~1.5-2 us.  Direct columns need neither the way down nor the reconstruction:
+// U, tau and R are the result (the same reflectors: beta = -sgn(alpha) ||x||,
+// tau in [1, 2]).  Measured (GB300): the whole panel
+// step at n = 16384, b = 128 (FP32) 276 -> 93 ms per reduction, n = 8192,
+// b = 64 101 -> 24 ms; n = 3001, b = 32 in FP64 200 -> 21 ms.
+//
+// One exchange per column.  With x = column k below row k (zero above) and
+// v = e_k + x / (alpha - beta), the products v^T a_j that the reflector needs
+// are a_kj + (x^T a_j) / (alpha - beta), so every CTA can send its share of
+// x^T x and of x^T a_j for ALL columns j before tau and beta are known; for
+// finished columns j < k the same expression is G(j, k) = v_j^T v_k, from
+// which the last CTA forms the compact-WY factor T while it waits for the
+// next exchange.  x is held times the power of two of the panel's largest
+// entry (exact); x^T x of FP32 data is summed error-free in pairs of floats.
+//
+// Exchange.  Every value travels as one 8-byte word (FP64: two) holding the
+// 32 bits and a tag (panel and column), stored and polled with single 8-byte
+// accesses: a word whose tag is right is complete, so no fence, flag or
+// barrier is needed.  Two sets of words alternate: a CTA sends column k + 1
+// only after it has read all of column k, so whoever has read column k + 1
+// knows that column k's words may be overwritten.  All CTAs are resident
+// (cooperative launch, at most one CTA per SM); every wait is capped and latches
+// SEV_ERR_TIMEOUT on expiry.
+//
+// What bounds it: the chain of one column -- dot products and their warp sums,
+// L2 store to load (~1.4K cycles), the sum over the CTAs, the reflector
+// scalars, the update of column k + 1.  Every CTA reads every CTA's shares:
+// C^2 b words per column, which is why the rows per CTA grow with N.
+#include "regtile.cuh"
+
+namespace sev {
+
+constexpr int kCoopWarps = 16;                       // column warps; one more for the scalars
+constexpr int kCoopThreads = (kCoopWarps + 1) * 32;
+constexpr int kCoopMaxB = 128;
+
+// ------------------------------------------------------- tagged words
+__device__ __forceinline__ void ll_put(unsigned long long *p, unsigned v, unsigned tag) {
+    const unsigned long long w = ((unsigned long long)tag << 32) | v;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ void ll_get2(const unsigned long long *p, unsigned long long &a, unsigned long long &b) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ bool ll_is(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
+
+// A value of type T as tagged words: 1 for float, 2 for double.
+template <typename T>
+struct LLType;
+template <>
+struct LLType<float> {
+    static constexpr int W = 1;
+};
+template <>
+struct LLType<double> {
+    static constexpr int W = 2;
+};
+__device__ __forceinline__ void ll_put_val(unsigned long long *p, float v, unsigned tag) {
+    ll_put(p, __float_as_uint(v), tag);
+}
+__device__ __forceinline__ void ll_put_val(unsigned long long *p, double v, unsigned tag) {
+    ll_put(p, (unsigned)__double2loint(v), tag);
+    ll_put(p + 1, (unsigned)__double2hiint(v), tag);
+}
+
+// Layout of the exchange buffer (in words) for at most cmax CTAs (even).
+template <typename T>
+struct CoopComm {
+    static __host__ __device__ size_t col_words(int b, int cmax) { return (size_t)b * cmax * LLType<T>::W; }
+    static __host__ __device__ size_t row_words(int b) { return (size_t)b * 2; }
+    static __host__ __device__ size_t ssq_words(int cmax) { return (size_t)cmax * 2; }
+    // two alternating sets of (columns, row k, squares), then the largest entries
+    static __host__ __device__ size_t set_words(int b, int cmax) { return col_words(b, cmax) + row_words(b) + ssq_words(cmax); }
+    static __host__ __device__ size_t words(int b, int cmax) { return 2 * set_words(b, cmax) + ssq_words(cmax); }
+};
+
+// Warp sums of Q per-lane values by a transposing butterfly; the lane gets
+// the sum of value lane >> (5 - log2 Q).
+template <typename T, int Q, int H = Q / 2>
+__device__ __forceinline__ T warp_sums_t(T (&d)[Q]) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (H >= 1) {
+        constexpr int OFF = 16 * 2 * H / Q;  // H = Q/2: 16, Q/4: 8, ...
+        const bool up = lane & OFF;
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            const T keep = up ? d[j + H] : d[j], send = up ? d[j] : d[j + H];
+            d[j] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+        }
+        return warp_sums_t<T, Q, H / 2>(d);
+    } else {
+        T s = d[0];
+#pragma unroll
+        for (int o = 16 / Q; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    }
+}
+
+// This warp's columns' totals over the C CTAs: lane group sums in a fixed
+// order.  Polls until every word carries `tag`; false when the wait ran out.
+template <typename T, int Q>
+__device__ __forceinline__ bool coop_collect(const unsigned long long *cols, int cmax, int C, int warp, int b,
+                                             unsigned tag, long long cap, int *err, T (&sum)[Q]) {
+    const int lane = threadIdx.x & 31;
+    constexpr int PER = LLType<T>::W == 1 ? 2 : 1;  // values per 16-byte load
+    long long t0 = 0;
+    for (int tries = 0;; ++tries) {
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) sum[q] = T(0);
+        for (int c = PER * lane; c < C; c += PER * 32) {
+            unsigned long long a[Q], bb[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = warp + kCoopWarps * q;
+                a[q] = bb[q] = (unsigned long long)tag << 32;
+                if (j < b) ll_get2(cols + ((size_t)j * cmax + c) * LLType<T>::W, a[q], bb[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if constexpr (sizeof(T) == 4) {
+                    const bool two = c + 1 < C;
+                    ok = ok && ll_is(a[q], tag) && (!two || ll_is(bb[q], tag));
+                    sum[q] += __uint_as_float((unsigned)a[q]);
+                    if (two) sum[q] += __uint_as_float((unsigned)bb[q]);
+                } else {
+                    ok = ok && ll_is(a[q], tag) && ll_is(bb[q], tag);
+                    sum[q] += __hiloint2double((int)(unsigned)bb[q], (int)(unsigned)a[q]);
+                }
+            }
+        }
+        if (__all_sync(0xffffffffu, ok)) break;
+        if (tries == 0) t0 = clock64();
+        int stop = 0;
+        if (lane == 0) {
+            if ((tries & 31) == 31 && *(volatile int *)err != 0) stop = 1;
+            if (wait_expired(t0, cap)) {
+                latch_error(err, SEV_ERR_TIMEOUT);
+                stop = 1;
+            }
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+    }
+    // totals in every lane
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        if (warp + kCoopWarps * q >= b) sum[q] = T(0);
+    }
+    const T s = warp_sums_t<T, Q>(sum);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) sum[q] = __shfl_sync(0xffffffffu, s, q * (32 / Q));
+    return true;
+}
+
+// A pair of words per entry i < cnt (lane takes i = lane, lane + 32, ...),
+// polled until tagged; f(i, word0, word1) is called once per entry at the end.
+template <typename F>
+__device__ __forceinline__ bool coop_poll_pairs(const unsigned long long *p, int cnt, unsigned tag, long long cap,
+                                                int *err, F f) {
+    const int lane = threadIdx.x & 31;
+    long long t0 = 0;
+    for (int tries = 0;; ++tries) {
+        bool ok = true;
+        for (int i = lane; i < cnt; i += 32) {
+            unsigned long long a, b;
+            ll_get2(p + 2 * (size_t)i, a, b);
+            ok = ok && ll_is(a, tag) && ll_is(b, tag);
+            f(i == lane, (unsigned)a, (unsigned)b);
+        }
+        if (__all_sync(0xffffffffu, ok)) return true;
+        if (tries == 0) t0 = clock64();
+        int stop = 0;
+        if (lane == 0) {
+            if ((tries & 31) == 31 && *(volatile int *)err != 0) stop = 1;
+            if (wait_expired(t0, cap)) {
+                latch_error(err, SEV_ERR_TIMEOUT);
+                stop = 1;
+            }
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+    }
+}
+
+template <typename T, int RT>
+struct CoopSmem {
+    T xs[2][32 * RT];          // scale times column k below row k
+    T gs[kCoopMaxB];           // G(j, k), j < k (last CTA)
+    T part[kCoopWarps * 32];   // partial sums of a column of T (last CTA)
+    T tau[kCoopMaxB];
+    T sc[4];                   // tau, beta, 1 / (scale (alpha - beta)) of the column; the panel's scale
+    int abort;
+};
+
+// Column kc of T by the last CTA, in two halves with a barrier between them:
+// T(a, kc) = -tau sum_{q = a}^{kc - 1} T(a, q) G(q, kc) (forward, column-wise:
+// Q = I - U T U^T).  Ts: column-major, ld b, zero below the diagonal.
+template <typename T>
+__device__ __forceinline__ void coop_t_partial(int b, int kc, const T *Ts, const T *gs, T *part) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nrg = (b + 31) / 32, nsl = kCoopWarps / nrg;
+    const int a = 32 * (warp % nrg) + lane, sl = warp / nrg;
+    if (sl >= nsl) return;
+    T s0 = T(0);
+    if (a < b)
+        for (int q = sl; q < kc; q += nsl) s0 = fmat(Ts[(size_t)q * b + a], gs[q], s0);
+    if (a < b) part[sl * b + a] = s0;
+}
+template <typename T>
+__device__ __forceinline__ void coop_t_column(int b, int kc, T *Ts, const T *tau, const T *part) {
+    const int lane = threadIdx.x & 31;
+    const int nsl = kCoopWarps / ((b + 31) / 32);
+    const T tk = tau[kc];
+    for (int a = lane; a <= kc; a += 32) {
+        T s = T(0);
+        if (a < kc)
+            for (int l = 0; l < nsl; ++l) s += part[l * b + a];
+        Ts[(size_t)kc * b + a] = a == kc ? tk : -tk * s;
+    }
+}
+
+// P: N x b panel (ldp).  On return U (N x b, ld N) holds the reflectors (unit
+// lower trapezoidal), Tm (b x b) the compact-WY factor, and P the band block
+// (R over zeros).  comm: exchange words; tags tag0 + 1 .. tag0 + b + 1 are
+// unused so far in it.
+template <typename T, int RT, int Q>
+__global__ void __launch_bounds__(kCoopThreads, 1)
+    panel_coop_kernel(T *__restrict__ P, int ldp, int N, int b, T *__restrict__ U, T *__restrict__ Tm,
+                      unsigned long long *comm, int cmax, unsigned tag0, int *err) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    CoopSmem<T, RT> &S = *reinterpret_cast<CoopSmem<T, RT> *>(smem_raw);
+    T *Ts = reinterpret_cast<T *>(smem_raw + ((sizeof(CoopSmem<T, RT>) + 15) & ~(size_t)15));  // last CTA
+    constexpr int R = 32 * RT;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c = blockIdx.x, C = gridDim.x;
+    const bool lastc = c == C - 1;
+    const int row0 = c * R, rows = min(R, N - row0);
+    const int nref = min(b, N - 1);
+    const long long cap = wait_cap(err);
+    using Comm = CoopComm<T>;
+    unsigned long long *const amx = comm + 2 * Comm::set_words(b, cmax);
+
+    T a[Q][RT];
+    if (warp < kCoopWarps) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int t = 0; t < RT; ++t) {
+                const int j = warp + kCoopWarps * q, r = lane + 32 * t;
+                a[q][t] = (j < b && r < rows) ? P[(size_t)(row0 + r) + (size_t)j * ldp] : T(0);
+            }
+    }
+    if (threadIdx.x == 0) S.abort = 0;
+    if (lastc)
+        for (int i = threadIdx.x; i < b * b; i += blockDim.x) Ts[i] = T(0);
+    // The panel's largest entry: x is held times its power of two, so that no
+    // square or product that matters over- or underflows.
+    {
+        double m = 0.0;
+        if (warp < kCoopWarps) {
+            T mt = T(0);
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+#pragma unroll
+                for (int t = 0; t < RT; ++t) mt = max(mt, (T)fabs(a[q][t]));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) mt = max(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+            if (lane == 0) S.part[warp] = mt;
+        }
+        __syncthreads();
+        if (warp == kCoopWarps) {
+            m = lane < kCoopWarps ? (double)S.part[lane] : 0.0;
+            m = warp_max(m);
+            if (lane == 0) ll_put_val(amx + 2 * c, m, tag0 + 1);
+            double g = 0.0;
+            const bool got = coop_poll_pairs(amx, C, tag0 + 1, cap, err, [&](bool first, unsigned lo, unsigned hi) {
+                const double v = __hiloint2double((int)hi, (int)lo);
+                g = first ? v : fmax(g, v);
+            });
+            g = warp_max(g);
+            constexpr int EM = sizeof(T) == 8 ? 1000 : 126;
+            int e2 = 0;
+            if (g > 0.0 && isfinite(g)) (void)frexp(g, &e2);
+            e2 = e2 > EM ? EM : (e2 < -EM ? -EM : e2);
+            if (lane == 0) {
+                S.sc[3] = (T)pow2i(-e2);
+                if (!got) S.abort = 1;
+            }
+        }
+    }
+    __syncthreads();
+    const T scale = S.sc[3];
+    bool alive = !S.abort;
+    if (warp == 0) {
+#pragma unroll
+        for (int t = 0; t < RT; ++t) S.xs[0][lane + 32 * t] = row0 + lane + 32 * t > 0 ? a[0][t] * scale : T(0);
+    }
+    __syncthreads();
+
+    for (int k = 0; k < nref && alive; ++k) {
+        const unsigned tag = tag0 + 2 + k;
+        unsigned long long *const set = comm + (k & 1) * Comm::set_words(b, cmax);
+        unsigned long long *const roww = set + Comm::col_words(b, cmax);
+        unsigned long long *const ssqw = roww + Comm::row_words(b);
+        const T *xk = S.xs[k & 1];
+        T dsum[Q], rk[Q];
+        if (warp < kCoopWarps) {
+            T xr[RT];
+            // ---- this CTA's shares of x^T a_j, and row k from the CTA that holds it
+#pragma unroll
+            for (int t = 0; t < RT; ++t) xr[t] = xk[lane + 32 * t];
+            if (c == 0 && lane == (k & 31)) {
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const int j = warp + kCoopWarps * q;
+                    if (j < b) {
+                        const T v = rsel<RT>(a[q], k >> 5);
+                        ll_put_val(roww + 2 * j, v, tag);
+                        if constexpr (sizeof(T) == 4) ll_put(roww + 2 * j + 1, 0u, tag);
+                    }
+                }
+            }
+            T d[Q];
+            if constexpr (sizeof(T) == 4) {
+                float2 dd[Q / 2];
+#pragma unroll
+                for (int p = 0; p < Q / 2; ++p) dd[p] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int t = 0; t < RT; ++t) {
+                    const float2 vv = make_float2(xr[t], xr[t]);
+#pragma unroll
+                    for (int p = 0; p < Q / 2; ++p) dd[p] = ffma2(vv, make_float2(a[2 * p][t], a[2 * p + 1][t]), dd[p]);
+                }
+#pragma unroll
+                for (int p = 0; p < Q / 2; ++p) {
+                    d[2 * p] = dd[p].x;
+                    d[2 * p + 1] = dd[p].y;
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < Q; ++q) d[q] = T(0);
+#pragma unroll
+                for (int t = 0; t < RT; ++t)
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) d[q] = fmat(xr[t], a[q][t], d[q]);
+            }
+            const T mine = warp_sums_t<T, Q>(d);
+            if ((lane & (32 / Q - 1)) == 0) {
+                const int j = warp + kCoopWarps * (lane / (32 / Q));
+                if (j < b) ll_put_val(set + ((size_t)j * cmax + c) * LLType<T>::W, mine, tag);
+            }
+            if (lastc && k >= 1) coop_t_partial<T>(b, k - 1, Ts, S.gs, S.part);
+            bool ok = coop_collect<T, Q>(set, cmax, C, warp, b, tag, cap, err, dsum);
+            // row k at this warp's columns
+            T rv = T(0);
+            if (ok) {
+                long long t0 = clock64();
+                for (;;) {
+                    unsigned long long w0 = (unsigned long long)tag << 32, w1 = w0;
+                    const int j = warp + kCoopWarps * lane;
+                    if (lane < Q && j < b) ll_get2(roww + 2 * j, w0, w1);
+                    if constexpr (sizeof(T) == 4)
+                        rv = __uint_as_float((unsigned)w0);
+                    else
+                        rv = __hiloint2double((int)(unsigned)w1, (int)(unsigned)w0);
+                    if (__all_sync(0xffffffffu, ll_is(w0, tag) && ll_is(w1, tag))) break;
+                    if (__any_sync(0xffffffffu, wait_expired(t0, cap))) {
+                        if (lane == 0) latch_error(err, SEV_ERR_TIMEOUT);
+                        ok = false;
+                        break;
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) rk[q] = __shfl_sync(0xffffffffu, rv, q);
+            if (!ok && lane == 0) S.abort = 1;
+        } else {
+            // ---- the scalar warp: x^T x over all CTAs, then tau, beta, 1 / (alpha - beta)
+            bool ok = true;
+            if constexpr (sizeof(T) == 4) {
+                F2 p0{0.f, 0.f}, p1{0.f, 0.f};
+#pragma unroll
+                for (int t = 0; t < RT; t += 2) {
+                    f2_add_sq(p0, (float)xk[lane + 32 * t]);
+                    f2_add_sq(p1, (float)xk[lane + 32 * t + 32]);
+                }
+                const F2 mine = warp_sum_f2(f2_add(p0, p1));
+                if (lane == 0) {
+                    ll_put(ssqw + 2 * c, __float_as_uint(mine.hi), tag);
+                    ll_put(ssqw + 2 * c + 1, __float_as_uint(mine.lo), tag);
+                }
+                F2 acc{0.f, 0.f};
+                ok = coop_poll_pairs(ssqw, C, tag, cap, err, [&](bool first, unsigned hi, unsigned lo) {
+                    const F2 v{__uint_as_float(hi), __uint_as_float(lo)};
+                    acc = first ? v : f2_add(acc, v);
+                });
+                acc = warp_sum_f2(acc);
+                float alpha = 0.f;
+                if (ok)
+                    ok = coop_poll_pairs(roww + 2 * k, 1, tag, cap, err,
+                                         [&](bool, unsigned v, unsigned) { alpha = __uint_as_float(v); });
+                alpha = __shfl_sync(0xffffffffu, alpha, 0);
+                alpha *= (float)scale;
+                float tau = 0.f, beta = 0.f, inv = 0.f;
+                // a column 1e-16 times smaller than the panel's largest entry is a
+                // zero column (its pair-float square would lose digits to underflow)
+                if (fmaf(alpha, alpha, acc.hi) >= 1e-32f) house_scalars_f2(alpha, acc, &tau, &beta, &inv);
+                if (lane == 0) {
+                    S.sc[0] = (T)tau;
+                    S.sc[1] = (T)(beta / (float)scale);
+                    S.sc[2] = (T)inv;
+                    S.tau[k] = (T)tau;
+                }
+            } else {
+                double s = 0.0;
+#pragma unroll
+                for (int t = 0; t < RT; ++t) {
+                    const double x = (double)xk[lane + 32 * t];
+                    s = fma(x, x, s);
+                }
+                s = warp_sum(s);
+                if (lane == 0) ll_put_val(ssqw + 2 * c, s, tag);
+                double acc = 0.0;
+                ok = coop_poll_pairs(ssqw, C, tag, cap, err, [&](bool first, unsigned lo, unsigned hi) {
+                    const double v = __hiloint2double((int)hi, (int)lo);
+                    acc = first ? v : acc + v;
+                });
+                acc = warp_sum(acc);
+                double alpha = 0.0;
+                if (ok)
+                    ok = coop_poll_pairs(roww + 2 * k, 1, tag, cap, err, [&](bool, unsigned lo, unsigned hi) {
+                        alpha = __hiloint2double((int)hi, (int)lo);
+                    });
+                alpha = __shfl_sync(0xffffffffu, alpha, 0);
+                const double as = alpha * (double)scale;
+                double tau = 0.0, beta = 0.0, inv = 0.0;
+                // a column 1e-140 times smaller than the panel's largest entry is a
+                // zero column (its square could not be told from underflow)
+                if (fma(as, as, acc) >= 1e-280) house_scalars(as, acc, &tau, &beta, &inv);
+                if (lane == 0) {
+                    S.sc[0] = (T)tau;
+                    S.sc[1] = (T)(beta / (double)scale);
+                    S.sc[2] = (T)inv;
+                    S.tau[k] = (T)tau;
+                }
+            }
+            if (!ok && lane == 0) S.abort = 1;
+        }
+        __syncthreads();
+        alive = !S.abort;
+        if (warp < kCoopWarps) {
+            // ---- a_j -= tau (v^T a_j) v for j > k; column k becomes (beta, v); G(j, k) for j < k
+            const T tau = S.sc[0], beta = S.sc[1], inv = S.sc[2];
+            T v[RT];
+#pragma unroll
+            for (int t = 0; t < RT; ++t) v[t] = row0 + lane + 32 * t == k ? T(1) : xk[lane + 32 * t] * inv;
+            T ms[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = warp + kCoopWarps * q;
+                const T s = fmat(inv, dsum[q], rk[q]);
+                ms[q] = (j > k && j < b) ? -tau * s : T(0);
+                if (lastc && lane == 0 && j < k) S.gs[j] = s;
+                // (tau = 0: the column is zero below row k, or far below the
+                // rounding errors of the panel's other entries and dropped here)
+                const bool own = j == k;
+#pragma unroll
+                for (int t = 0; t < RT; ++t) {
+                    const int g = row0 + lane + 32 * t;
+                    a[q][t] = own && g > k ? v[t] : (own && g == k && tau != T(0) ? beta : a[q][t]);
+                }
+            }
+            if (tau != T(0)) {
+                if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                    for (int t = 0; t < RT; ++t) {
+                        const float2 vv = make_float2(v[t], v[t]);
+#pragma unroll
+                        for (int p = 0; p < Q / 2; ++p) {
+                            const float2 r = ffma2(make_float2(ms[2 * p], ms[2 * p + 1]), vv,
+                                                   make_float2(a[2 * p][t], a[2 * p + 1][t]));
+                            a[2 * p][t] = r.x;
+                            a[2 * p + 1][t] = r.y;
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < Q; ++q)
+#pragma unroll
+                        for (int t = 0; t < RT; ++t) a[q][t] = fmat(ms[q], v[t], a[q][t]);
+                }
+            }
+            const int k1 = k + 1;
+            if (k1 < nref && k1 % kCoopWarps == warp) {
+                T *xn = S.xs[k1 & 1];
+                const unsigned pick = 1u << (k1 / kCoopWarps);
+#pragma unroll
+                for (int t = 0; t < RT; ++t) {
+                    T x = a[0][t];
+#pragma unroll
+                    for (int q = 1; q < Q; ++q) x = (pick >> q) & 1 ? a[q][t] : x;
+                    xn[lane + 32 * t] = row0 + lane + 32 * t > k1 ? x * scale : T(0);
+                }
+            }
+        } else if (lastc && k >= 1) {
+            coop_t_column<T>(b, k - 1, Ts, S.tau, S.part);
+        }
+        __syncthreads();
+    }
+    if (!alive) return;  // the error is latched; nothing was written
+    // ---- the last column of T, then the results
+    if (lastc) {
+        if (nref > 0) {
+            if (warp < kCoopWarps) coop_t_partial<T>(b, nref - 1, Ts, S.gs, S.part);
+            __syncthreads();
+            if (warp == kCoopWarps) coop_t_column<T>(b, nref - 1, Ts, S.tau, S.part);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < b * b; i += blockDim.x) Tm[i] = Ts[i];
+    }
+    if (warp < kCoopWarps) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int t = 0; t < RT; ++t) {
+                const int j = warp + kCoopWarps * q, r = lane + 32 * t, g = row0 + r;
+                if (j >= b || r >= rows) continue;
+                T v = T(0);
+                if (j < nref) v = g < j ? T(0) : (g == j ? T(1) : a[q][t]);
+                U[(size_t)g + (size_t)j * N] = v;
+                P[(size_t)g + (size_t)j * ldp] = g <= j ? a[q][t] : T(0);
+            }
+    }
+}
+
+// -------------------------------------------------------------------- host
+// CTAs the exchange buffer has room for (one per SM, even).
+static int coop_cmax(const sev_ctx *h) { return (h->sm_count + 1) / 2 * 2; }
+
+template <typename T>
+size_t panel_coop_words(const sev_ctx *h, int b) {
+    return CoopComm<T>::words(b, coop_cmax(h));
+}
+
+// Rows per CTA (in units of 32): the fewest for which the CTAs stay a
+// moderate number -- more rows mean more arithmetic per CTA and column, more
+// CTAs mean more shares to read.  0: the panel does not fit the GPU.
+template <typename T>
+static int coop_rt(const sev_ctx *h, int N) {
+    const int sizes[3] = {2, 4, 8}, room[3] = {sizeof(T) == 4 ? 0 : 96, sizeof(T) == 4 ? 32 : 128, h->sm_count};
+    for (int i = 0; i < 3; ++i) {
+        const int C = (N + 32 * sizes[i] - 1) / (32 * sizes[i]);
+        if (C <= room[i] && C <= h->sm_count) return sizes[i];
+    }
+    return 0;
+}
+
+template <typename T>
+int panel_coop_supported(const sev_ctx *h, int N, int b) {
+    if (h->leaf_rows_override > 0) return 0;  // the caller asked for a tree of that leaf size
+    return b >= 1 && b <= (sizeof(T) == 4 ? 128 : 64) && coop_rt<T>(h, N) > 0;
+}
+
+template <typename T, int RT, int Q>
+static int panel_coop_run(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
+    const size_t smem = ((sizeof(CoopSmem<T, RT>) + 15) & ~(size_t)15) + sizeof(T) * (size_t)b * b;
+    auto kern = panel_coop_kernel<T, RT, Q>;
+    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int C = (N + 32 * RT - 1) / (32 * RT);
+    int cmax = coop_cmax(h);
+    void *args[] = {(void *)&P,    (void *)&lda,  (void *)&N,    (void *)&b,   (void *)&U,
+                    (void *)&Tm,   (void *)&comm, (void *)&cmax, (void *)&tag0, (void *)&h->d_err};
+    timing_begin(h, K_PANEL_COOP);
+    SEV_CUDA(cudaLaunchCooperativeKernel((const void *)kern, C, kCoopThreads, args, smem, h->stream));
+    timing_end(h, K_PANEL_COOP);
+    return SEV_OK;
+}
+
+template <typename T, int Q>
+static int panel_coop_rt(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
+    switch (coop_rt<T>(h, N)) {
+        case 2:
+            if constexpr (sizeof(T) == 8) return panel_coop_run<T, 2, Q>(h, N, b, P, lda, U, Tm, comm, tag0);
+            return SEV_ERR_UNSUPPORTED;
+        case 4: return panel_coop_run<T, 4, Q>(h, N, b, P, lda, U, Tm, comm, tag0);
+        case 8: return panel_coop_run<T, 8, Q>(h, N, b, P, lda, U, Tm, comm, tag0);
+        default: return SEV_ERR_UNSUPPORTED;
+    }
+}
+
+template <typename T>
+int panel_coop_factor(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
+    if (b <= 32) return panel_coop_rt<T, 2>(h, N, b, P, lda, U, Tm, comm, tag0);
+    if (b <= 64) return panel_coop_rt<T, 4>(h, N, b, P, lda, U, Tm, comm, tag0);
+    if constexpr (sizeof(T) == 4) return panel_coop_rt<T, 8>(h, N, b, P, lda, U, Tm, comm, tag0);
+    return SEV_ERR_UNSUPPORTED;
+}
+
+template size_t panel_coop_words<float>(const sev_ctx *, int);
+template size_t panel_coop_words<double>(const sev_ctx *, int);
+template int panel_coop_supported<float>(const sev_ctx *, int, int);
+template int panel_coop_supported<double>(const sev_ctx *, int, int);
+template int panel_coop_factor<float>(sev_ctx *, int, int, float *, int, float *, float *, unsigned long long *, unsigned);
+template int panel_coop_factor<double>(sev_ctx *, int, int, double *, int, double *, double *, unsigned long long *,
+                                       unsigned);
+
+}  // namespace sev

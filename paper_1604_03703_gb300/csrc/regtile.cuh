@@ -37,13 +37,15 @@ __device__ __forceinline__ double fmat<double>(double a, double b, double c) {
     return fma(a, b, c);
 }
 
-// x[t] for a run-time t without dynamic register indexing.
+// x[t] for a run-time t without dynamic register indexing.  (The test is on a
+// bit of a mask: with i == t the compiler replaces x[i] by x[t], which puts
+// the whole array into local memory.)
 template <int R, typename T>
 __device__ __forceinline__ T rsel(const T (&x)[R], int t) {
+    const unsigned pick = 1u << t;
     T r = x[0];
 #pragma unroll
-    for (int i = 1; i < R; ++i)
-        if (i == t) r = x[i];
+    for (int i = 1; i < R; ++i) r = (pick >> i) & 1 ? x[i] : r;
     return r;
 }
 

@@ -444,6 +444,8 @@ __global__ void __launch_bounds__(256) syr2k_kernel(int N, int b, T *__restrict_
 template <typename T>
 struct F2BBuffers {
     T *U, *Y, *X, *V, *Tm, *Zm, *part, *ypart;
+    unsigned long long *comm;
+    size_t comm_words;
     void *panel_ws, *tc_ws;
 };
 
@@ -467,6 +469,8 @@ static void carve_f2b(Carver &c, F2BBuffers<T> &B, sev_ctx *h, int n, int b, boo
     B.part = c.take<T>((size_t)(utx_parts(n) + 1) * b * b);  // the chunks' partial products, then their sum
     B.ypart = c.take<T>((size_t)kSymmMaxSplits * n * b);
     B.tc_ws = tc ? (void *)c.take<char>(tc_workspace<T>(n, b)) : nullptr;
+    B.comm_words = panel_coop_words<T>(h, b);
+    B.comm = c.take<unsigned long long>(B.comm_words);
     B.panel_ws = c.take<char>(panel_workspace<T>(h, n, b));
 }
 
@@ -485,6 +489,7 @@ int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab
     Carver c(ws);
     F2BBuffers<T> B;
     carve_f2b<T>(c, B, h, n, b, true);
+    bool comm_clear = false;
     for (int k = 0;; ++k) {
         const int c0 = k * b, r0 = c0 + b;
         if (r0 >= n) break;
@@ -492,7 +497,18 @@ int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab
         if (N < 2) break;
         T *P = A + (size_t)r0 + (size_t)c0 * lda;
         T *A22 = A + (size_t)r0 + (size_t)r0 * lda;
-        int rc = panel_factor<T>(h, N, b, P, lda, B.U, B.Tm, B.panel_ws);
+        int rc;
+        if (panel_coop_supported<T>(h, N, b)) {
+            // the panel on all SMs at once; the tree serves panels too tall for
+            // the GPU's registers, wider bands and a prescribed leaf size
+            if (!comm_clear) {
+                SEV_CUDA(cudaMemsetAsync(B.comm, 0, sizeof(unsigned long long) * B.comm_words, h->stream));
+                comm_clear = true;
+            }
+            rc = panel_coop_factor<T>(h, N, b, P, lda, B.U, B.Tm, B.comm, (unsigned)k * (unsigned)(b + 2));
+        } else {
+            rc = panel_factor<T>(h, N, b, P, lda, B.U, B.Tm, B.panel_ws);
+        }
         if (rc) return rc;
         const bool tc = tc_update_supported<T>(h, N, b);
         // Y = A22 U
