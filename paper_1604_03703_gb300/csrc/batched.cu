@@ -20,6 +20,7 @@
 // is overwritten (both triangles: the kernel first mirrors the lower
 // triangle).  Nothing is allocated and nothing waits on the host, so the
 // launch can be captured in a CUDA graph.
+#include "sturm.cuh"
 #include "tri_chase.cuh"
 
 namespace sev {
@@ -200,37 +201,6 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
 // -------------------------------------------------------------- bisection
 // The same scaling, minors count, stopping rule and IEEE operations as
 // bisect.cu, on shared-memory d and (e 2^-s)^2.
-__device__ __forceinline__ double batch_pow2(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
-
-__device__ __forceinline__ int batch_sturm(int n, const double *d, const double *e2s, double x, double sc) {
-    double a = 1.0, b = __fma_rn(d[0], sc, -x);
-    bool neg = b <= 0.0;
-    int c = neg;
-    for (int i = 1; i < n; ++i) {
-        const double t = __fma_rn(d[i], sc, -x);
-        const double u = __dmul_rn(e2s[i - 1], a);
-        const double p = __fma_rn(t, b, -u);
-        // sign, zero test and exponent from the bits: integer work, so the
-        // FP64 pipe sees only the three operations above
-        const long long pb = __double_as_longlong(p);
-        const bool zero = (pb << 1) == 0;
-        const bool pn = zero ? !neg : pb < 0;
-        c += pn != neg;
-        neg = pn;
-        a = b;
-        b = p;
-        const int ex = (int)((pb >> 52) & 0x7FF);
-        if (__builtin_expect(ex > 1023 + 256 || (ex < 1023 - 256 && !zero), 0)) {
-            int k = 1023 - ex;
-            k = k > 512 ? 512 : (k < -512 ? -512 : k);
-            const double f = batch_pow2(k);
-            a = __dmul_rn(a, f);
-            b = __dmul_rn(b, f);
-        }
-    }
-    return c;
-}
-
 template <typename T, int B>
 __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, double *eigs, int *err) {
     constexpr int LDW = 2 * B;
@@ -239,7 +209,7 @@ __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, 
     double *d = (double *)(smem + BatchLayout<T, B>::e_off(nmax));
     double *e = d + nmax;
     double *e2s = e + nmax;
-    double *par = e2s + nmax;  // gl, gu, sc, tnorm, 2^s, zero
+    double *par = e2s + nmax;  // gl, gu, sc, tnorm, 2^s, zero, no tiny e2s
     double *red = par + 8;     // 32
     for (int i = tid; i < n; i += nt) {
         d[i] = (double)band[(size_t)i * LDW];
@@ -261,7 +231,7 @@ __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, 
         if (!isfinite(tnorm)) latch_error(err, SEV_ERR_NONFINITE);
         int s = 0;
         if (tnorm > 0.0 && isfinite(tnorm)) (void)frexp(tnorm, &s);
-        const double sc = batch_pow2(-s);
+        const double sc = pow2_exact(-s);
         lo = __dmul_rn(lo, sc);
         hi = __dmul_rn(hi, sc);
         tnorm = __dmul_rn(tnorm, sc);
@@ -270,22 +240,24 @@ __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, 
         par[1] = __dadd_rn(hi, pad);
         par[2] = sc;
         par[3] = tnorm;
-        par[4] = batch_pow2(s);
+        par[4] = pow2_exact(s);
         par[5] = tnorm == 0.0 ? 1.0 : 0.0;
+        par[6] = 1.0;
     }
     __syncthreads();
     const double sc = par[2];
     for (int i = tid; i < n; i += nt) {
         if (i + 1 < n) {
-            const double es = __dmul_rn(e[i], sc);
-            e2s[i] = __dmul_rn(es, es);
+            const double es = __dmul_rn(e[i], sc), e2 = __dmul_rn(es, es);
+            e2s[i] = e2;
+            if (es != 0.0 && e2 < 0x1p-322) par[6] = 0.0;
         } else {
             e2s[i] = 0.0;
         }
     }
     __syncthreads();
     const double atol = __dmul_rn(rtol, par[3]);
-    const bool zero = par[5] != 0.0;
+    const bool zero = par[5] != 0.0, plain = par[6] != 0.0;
     for (int k = tid; k < n; k += nt) {
         double a = par[0], b = par[1];
         int it = 0;
@@ -301,7 +273,8 @@ __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, 
             }
             const double mid = __dmul_rn(0.5, __dadd_rn(a, b));
             if (mid <= a || mid >= b) break;
-            if (batch_sturm(n, d, e2s, mid, sc) >= k + 1)
+            if (sturm_count_blocks<4>(
+                    n, [&](int i) { return d[i]; }, [&](int i) { return e2s[i]; }, mid, sc, plain) >= k + 1)
                 b = mid;
             else
                 a = mid;

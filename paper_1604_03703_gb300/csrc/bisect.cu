@@ -16,7 +16,7 @@
 // recurrence in the order written.
 #include <atomic>
 
-#include "common.cuh"
+#include "sturm.cuh"
 
 namespace sev {
 
@@ -94,15 +94,14 @@ template int launch_tridiag_extract<double>(sev_ctx *, int, const double *, int,
 // = 2^-s, par[3] = tnorm (scaled max |end| of the unwidened interval),
 // par[4] = 2^s, par[5] = 1 if T = 0 (a zero Gershgorin bound), par[6] = 1 if
 // the caller's skip flag was set (non-finite input: no bisection, NaN
-// eigenvalues).  e2s[i] = (e_i 2^-s)^2.
-__device__ __forceinline__ double pow2_exact(int k) {  // 2^k, -1022 <= k <= 1023
-    return __longlong_as_double((long long)(1023 + k) << 52);
-}
-
+// eigenvalues), par[7] = 1 if some e2s is nonzero but below 2^-322.  e2s[i] =
+// (e_i 2^-s)^2.
 __global__ void bisect_prep_kernel(int n, const double *__restrict__ d, const double *__restrict__ e,
                                    double *__restrict__ e2s, double *__restrict__ par, const int *skip) {
     __shared__ double red[32];
     __shared__ double s_sc;
+    __shared__ int s_tiny;
+    if (threadIdx.x == 0) s_tiny = 0;
     double lo = INFINITY, hi = -INFINITY;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         double r = 0.0;
@@ -135,77 +134,21 @@ __global__ void bisect_prep_kernel(int n, const double *__restrict__ d, const do
     const double sc = s_sc;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         if (i + 1 < n) {
-            const double es = __dmul_rn(e[i], sc);
-            e2s[i] = __dmul_rn(es, es);
+            const double es = __dmul_rn(e[i], sc), e2 = __dmul_rn(es, es);
+            e2s[i] = e2;
+            if (es != 0.0 && e2 < 0x1p-322) s_tiny = 1;
         } else {
             e2s[i] = 0.0;
         }
     }
+    __syncthreads();
+    if (threadIdx.x == 0) par[7] = s_tiny ? 1.0 : 0.0;
 }
 
-// One step of the minors recurrence with t = d_i sc - x: u = e_{i-1}^2 a,
-// p = t b - u; sign, zero test and exponent from the bits (integer work, so
-// the FP64 pipe sees only the three operations), rescaling by a power of two
-// when |p| leaves [2^-256, 2^256].
-__device__ __forceinline__ void sturm_step(double di, double e2i, double x, double sc, double &a, double &b,
-                                           bool &neg, int &c) {
-    const double t = __fma_rn(di, sc, -x);
-    const double u = __dmul_rn(e2i, a);
-    const double p = __fma_rn(t, b, -u);
-    const long long pb = __double_as_longlong(p);
-    const bool zero = (pb << 1) == 0;
-    const bool pn = zero ? !neg : pb < 0;
-    c += pn != neg;
-    neg = pn;
-    a = b;
-    b = p;
-    const int ex = (int)((pb >> 52) & 0x7FF);
-    if (__builtin_expect(ex > 1023 + 256 || (ex < 1023 - 256 && !zero), 0)) {
-        int k = 1023 - ex;
-        k = k > 512 ? 512 : (k < -512 ? -512 : k);
-        const double f = pow2_exact(k);
-        a = __dmul_rn(a, f);
-        b = __dmul_rn(b, f);
-    }
-}
-
-// The loads of d and e^2 do not depend on the recurrence, so blocks of kSturmU
-// steps are loaded one block ahead (the chain waits on the FP64 pipe, not on
-// a memory latency per step); the operations and their order are those of
-// the plain loop.
-constexpr int kSturmU = 4;
 __device__ __forceinline__ int sturm_count(int n, const double *__restrict__ d, const double *__restrict__ e2s,
-                                           double x, double sc) {
-    double a = 1.0, b = __fma_rn(__ldg(d), sc, -x);
-    bool neg = b <= 0.0;  // p_0 = 1 > 0: a zero p_1 counts as negative
-    int c = neg;
-    double dn[kSturmU], en[kSturmU];
-#pragma unroll
-    for (int u = 0; u < kSturmU; ++u) {
-        const int i = 1 + u;
-        dn[u] = i < n ? __ldg(d + i) : 0.0;
-        en[u] = i < n ? __ldg(e2s + i - 1) : 0.0;
-    }
-    for (int i0 = 1; i0 < n; i0 += kSturmU) {
-        double dc[kSturmU], ec[kSturmU];
-#pragma unroll
-        for (int u = 0; u < kSturmU; ++u) {
-            dc[u] = dn[u];
-            ec[u] = en[u];
-            const int i = i0 + kSturmU + u;
-            dn[u] = i < n ? __ldg(d + i) : 0.0;
-            en[u] = i < n ? __ldg(e2s + i - 1) : 0.0;
-        }
-        if (i0 + kSturmU <= n) {
-#pragma unroll
-            for (int u = 0; u < kSturmU; ++u) sturm_step(dc[u], ec[u], x, sc, a, b, neg, c);
-        } else {
-#pragma unroll
-            for (int u = 0; u < kSturmU; ++u)
-                if (i0 + u < n) sturm_step(dc[u], ec[u], x, sc, a, b, neg, c);
-        }
-    }
-    return c;
+                                           double x, double sc, bool plain) {
+    return sturm_count_blocks<8>(
+        n, [&](int i) { return __ldg(d + i); }, [&](int i) { return __ldg(e2s + i); }, x, sc, plain);
 }
 
 // One thread per eigenvalue index k (the (k+1)-th smallest).
@@ -223,6 +166,7 @@ __global__ void bisect_kernel(int n, const double *__restrict__ d, const double 
         return;
     }
     const double sc = par[2];
+    const bool plain = par[7] == 0.0;
     const double atol = __dmul_rn(rtol, par[3]);
     double lo = par[0], hi = par[1];
     int it = 0;
@@ -238,7 +182,7 @@ __global__ void bisect_kernel(int n, const double *__restrict__ d, const double 
         }
         const double mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
         if (mid <= lo || mid >= hi) break;
-        if (sturm_count(n, d, e2s, mid, sc) >= k + 1)
+        if (sturm_count(n, d, e2s, mid, sc, plain) >= k + 1)
             hi = mid;
         else
             lo = mid;
@@ -309,11 +253,6 @@ __device__ __forceinline__ int bis_step_test(double lo, double hi, int it, doubl
     return 0;
 }
 
-__device__ __forceinline__ int sturm_chain(int n, const double *__restrict__ d, const double *__restrict__ e2s, double x,
-                                        double sc) {
-    return sturm_count(n, d, e2s, x, sc);
-}
-
 struct BisWs {
     double *lo, *hi;
     int *it, *st;        // steps taken; state: 0 active, 1 finished
@@ -325,8 +264,179 @@ struct BisWs {
 #ifndef SEV_BIS_CHAINS_PER_SM
 #define SEV_BIS_CHAINS_PER_SM 128
 #endif
-constexpr int kBisThreads = 1024;
+constexpr int kBisThreads = 512;  // 128 registers a thread for the Sturm blocks
 constexpr int kBisMaxItems = 131072;
+
+// Depth of a round's subtrees for D distinct intervals: fewest rounds per
+// level, counting a round as one chain latency while its items fit the budget
+// of chains the GPU keeps in flight, and proportionally longer beyond it.
+__device__ __forceinline__ int bis_depth(int D, int budget, int most) {
+    int dep = 1;
+    float best = 2.f;
+    for (int t = 1; t <= 24; ++t) {
+        const long items = (long)D * ((1L << t) - 1);
+        if (items > most) break;
+        const float cost = fmaxf(1.f, (float)items / (float)budget) / (float)t;
+        if (cost < best) {
+            best = cost;
+            dep = t;
+        }
+    }
+    return dep;
+}
+
+// Count at midpoint m (heap order) of the subtree under [lo, hi]; -1 when the
+// bisection ends before it.
+__device__ __forceinline__ int bis_item(int n, const double *__restrict__ d, const double *__restrict__ e2, double lo,
+                                        double hi, int it, int m, double rtol, double atol, int maxit, double sc,
+                                        bool plain) {
+    // node m: its depth is floor(log2(m + 1)); the bits of m + 1 below the
+    // leading one, top first, are the turns (1 = right)
+    const int path = m + 1;
+    double mid = 0.0;
+    for (int l = 30 - __clz(path); l >= 0; --l) {
+        if (bis_step_test(lo, hi, it, rtol, atol, maxit, mid) != 0) return -1;
+        if ((path >> l) & 1)
+            lo = mid;
+        else
+            hi = mid;
+        ++it;
+    }
+    if (bis_step_test(lo, hi, it, rtol, atol, maxit, mid) != 0) return -1;
+    return sturm_count(n, d, e2, mid, sc, plain);
+}
+
+// Index k walks at most dep steps down its subtree: cnt(node) >= k + 1 turns
+// left.  Returns the stopping test's state after the last step.
+template <typename F>
+__device__ __forceinline__ int bis_walk(int k, int dep, double &lo, double &hi, int &it, double rtol, double atol,
+                                        int maxit, F cnt) {
+    double mid = 0.0;
+    int node = 0;
+    for (int l = 0; l < dep; ++l) {
+        const int r = bis_step_test(lo, hi, it, rtol, atol, maxit, mid);
+        if (r != 0) return r;
+        if (cnt(node) >= k + 1) {
+            hi = mid;
+            node = 2 * node + 1;
+        } else {
+            lo = mid;
+            node = 2 * node + 2;
+        }
+        ++it;
+    }
+    return bis_step_test(lo, hi, it, rtol, atol, maxit, mid);
+}
+
+// Small orders: the same rounds with every CTA keeping ALL indices' intervals
+// in shared memory and running the leader list and the walk for itself, so
+// that only the counts travel and a round has one grid barrier instead of
+// three (at these orders a round's chain is shorter than its barriers:
+// n = 100 217 -> 111 us with the faster Sturm
+// loop, n = 2048 3.07 -> 2.10 ms).  The counts of alternate rounds go to
+// alternate halves of W.cnt: a CTA writes round r + 2 only after barrier
+// r + 1, which every CTA reaches after it has read round r.
+constexpr int kBisSmallN = 2048;
+constexpr int kBisStage = 16384;  // counts of a round held in shared memory (16 bits each)
+constexpr int kBisSmallItems = kBisMaxItems / 2;
+__host__ __device__ constexpr size_t bis_small_smem(int n) { return (size_t)n * 24 + 64 + kBisStage * 2; }
+
+__global__ void __launch_bounds__(kBisThreads)
+    bisect_small_kernel(int n, const double *__restrict__ d, const double *__restrict__ e2,
+                        const double *__restrict__ par, double rtol, int maxit, int budget, double *__restrict__ eigs,
+                        int *cnt, BisCtl *ctl, int *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    double *lo = (double *)smem, *hi = lo + n;
+    short *lead = (short *)(hi + n), *leadof = lead + n, *it = leadof + n, *st = it + n;
+    short *stage = st + n;
+    __shared__ int s_warp[32];
+    const long long cap = wait_cap(err);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (par[6] != 0.0) {  // non-finite input (every CTA reads the same flag: no barrier is entered)
+        if (blockIdx.x == 0)
+            for (int k = tid; k < n; k += kBisThreads) eigs[k] = __longlong_as_double(0x7ff8000000000000LL);
+        return;
+    }
+    const double sc = par[2], atol = __dmul_rn(rtol, par[3]);
+    const bool plain = par[7] == 0.0;
+    const int zero = par[5] != 0.0;  // T = 0: every eigenvalue is exactly 0
+    for (int k = tid; k < n; k += kBisThreads) {
+        lo[k] = zero ? 0.0 : par[0];
+        hi[k] = zero ? 0.0 : par[1];
+        it[k] = 0;
+        st[k] = (short)zero;
+    }
+    __syncthreads();
+    constexpr int kPer = kBisSmallN / kBisThreads;  // indices per thread, consecutive
+    for (int round = 0;; ++round) {
+        // ---- leaders: the first index of every distinct active interval
+        bool is[kPer];
+        int mine = 0;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const int k = tid * kPer + u;
+            is[u] = k < n && st[k] == 0 && (k == 0 || st[k - 1] != 0 || lo[k] != lo[k - 1] || hi[k] != hi[k - 1]);
+            mine += is[u];
+        }
+        int pos = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += v;
+        }
+        if (lane == 31) s_warp[warp] = pos;
+        __syncthreads();
+        int before = 0, D = 0;
+#pragma unroll
+        for (int w = 0; w < kBisThreads / 32; ++w) {
+            const int v = s_warp[w];
+            before += w < warp ? v : 0;
+            D += v;
+        }
+        if (D == 0) break;
+        pos += before - mine;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const int k = tid * kPer + u;
+            if (is[u]) lead[pos++] = (short)k;
+            if (k < n) leadof[k] = (short)(pos - 1);
+        }
+        __syncthreads();
+        // ---- counts of this CTA's share of the round's midpoints
+        const int dep = bis_depth(D, budget, kBisSmallItems);
+        const int M = (1 << dep) - 1, items = D * M;
+        int *cr = cnt + (round & 1) * kBisSmallItems;
+        for (int w = blockIdx.x + tid * gridDim.x; w < items; w += gridDim.x * kBisThreads) {
+            const int k = lead[w / M];
+            __stcg(cr + w, bis_item(n, d, e2, lo[k], hi[k], it[k], w % M, rtol, atol, maxit, sc, plain));
+        }
+        if (!bis_barrier(ctl, round + 1, cap, err)) return;
+        const bool staged = items <= kBisStage;
+        if (staged) {
+            for (int w = tid; w < items; w += kBisThreads) stage[w] = (short)__ldcg(cr + w);
+            __syncthreads();
+        }
+        // ---- every active index walks down its leader's subtree
+        for (int k = tid; k < n; k += kBisThreads) {
+            if (st[k] != 0) continue;
+            const int j0 = (int)leadof[k] * M;
+            double l = lo[k], h = hi[k];
+            int i = it[k];
+            const int state = bis_walk(k, dep, l, h, i, rtol, atol, maxit, [&](int node) {
+                return staged ? (int)stage[j0 + node] : __ldcg(cr + j0 + node);
+            });
+            if (state == 2) latch_error(err, SEV_ERR_NOCONV);
+            lo[k] = l;
+            hi[k] = h;
+            it[k] = (short)i;
+            st[k] = state != 0;
+        }
+        __syncthreads();
+    }
+    const double up = par[4];
+    if (blockIdx.x == 0)
+        for (int k = tid; k < n; k += kBisThreads) eigs[k] = __dmul_rn(__dmul_rn(0.5, __dadd_rn(lo[k], hi[k])), up);
+}
 
 __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const double *__restrict__ d,
                                                                     const double *__restrict__ e2,
@@ -336,6 +446,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
     __shared__ int s_scan[kBisThreads];
     const long long cap = wait_cap(err);
     const double sc = par[2];
+    const bool plain = par[7] == 0.0;
     const double atol = __dmul_rn(rtol, par[3]);
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const int gthreads = gridDim.x * blockDim.x;
@@ -380,18 +491,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
                 // chain latency while its items fit the budget of chains the
                 // GPU keeps in flight, and proportionally longer beyond it
                 const int D = s_scan[kBisThreads - 1];
-                const long cap = n > kBisMaxItems ? n : kBisMaxItems;
-                int dep = 1;
-                double best = 2.0;
-                for (int t = 1; t <= 24; ++t) {
-                    const long items = (long)D * ((1L << t) - 1);
-                    if (items > cap) break;
-                    const double cost = fmax(1.0, (double)items / (double)budget) / t;
-                    if (cost < best) {
-                        best = cost;
-                        dep = t;
-                    }
-                }
+                const int dep = bis_depth(D, budget, n > kBisMaxItems ? n : kBisMaxItems);
                 W.ctl->D = D;
                 W.ctl->depth = dep;
                 W.ctl->done = D == 0;
@@ -412,51 +512,16 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
         for (long w = blockIdx.x + (long)threadIdx.x * gridDim.x; w < items; w += gthreads) {
             const int j = (int)(w / M), m = (int)(w % M);
             const int k = W.lead[j];
-            double lo = W.lo[k], hi = W.hi[k], mid = 0.0;
-            int it = W.it[k];
-            // node m in heap order: its depth is floor(log2(m + 1)); the bits of
-            // m + 1 below the leading one, top first, are the turns (1 = right)
-            const int path = m + 1;
-            const int lev = 31 - __clz(path);
-            bool live = true;
-            for (int l = lev - 1; l >= 0 && live; --l) {
-                if (bis_step_test(lo, hi, it, rtol, atol, maxit, mid) != 0) {
-                    live = false;
-                    break;
-                }
-                if ((path >> l) & 1)
-                    lo = mid;
-                else
-                    hi = mid;
-                ++it;
-            }
-            int c = -1;
-            if (live && bis_step_test(lo, hi, it, rtol, atol, maxit, mid) == 0) c = sturm_chain(n, d, e2, mid, sc);
-            W.cnt[w] = c;
+            W.cnt[w] = bis_item(n, d, e2, W.lo[k], W.hi[k], W.it[k], m, rtol, atol, maxit, sc, plain);
         }
         if (!bis_barrier(W.ctl, ++seq, cap, err)) return;
         // ---- (3) every active index walks dep steps down its leader's subtree
         for (int k = gtid; k < n; k += gthreads) {
             if (W.st[k] != 0) continue;
-            const int j = W.leadof[k];
-            double lo = W.lo[k], hi = W.hi[k], mid = 0.0;
-            int it = W.it[k], node = 0, state = 0;
-            for (int l = 0; l < dep; ++l) {
-                const int r = bis_step_test(lo, hi, it, rtol, atol, maxit, mid);
-                if (r != 0) {
-                    state = r;
-                    break;
-                }
-                if (W.cnt[(long)j * M + node] >= k + 1) {
-                    hi = mid;
-                    node = 2 * node + 1;
-                } else {
-                    lo = mid;
-                    node = 2 * node + 2;
-                }
-                ++it;
-            }
-            if (state == 0) state = bis_step_test(lo, hi, it, rtol, atol, maxit, mid);
+            const int *cj = W.cnt + (long)W.leadof[k] * M;
+            double lo = W.lo[k], hi = W.hi[k];
+            int it = W.it[k];
+            const int state = bis_walk(k, dep, lo, hi, it, rtol, atol, maxit, [&](int node) { return cj[node]; });
             if (state == 2) latch_error(err, SEV_ERR_NOCONV);
             W.lo[k] = lo;
             W.hi[k] = hi;
@@ -503,23 +568,25 @@ int launch_bisect(sev_ctx *h, int n, const double *d, const double *e, double rt
         return SEV_OK;
     }
     SEV_CUDA(cudaMemsetAsync(W.ctl, 0, sizeof(BisCtl), h->stream));
-    // one CTA per SM: enough Sturm chains in flight to cover the FP64 divide
-    // latency, and every CTA resident for the grid barrier
-    int per_sm = 0;
-    SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bisect_rounds_kernel, kBisThreads, 0));
-    if (per_sm < 1) return SEV_ERR_UNSUPPORTED;
-    // A Sturm step is three FP64 instructions on its dependence chain.  The
-    // budget of chains per round (128 per SM) is the measured best at
-    // n = 16384 since the Sturm loop loads ahead (64: 63.0 ms, 128: 58.5,
-    // 256: 58.3 on a random tridiagonal); 1024 threads per CTA run a round
-    // of up to 150K chains in a single pass.
-    const int grid = h->sm_count;
+    // One chain a scheduler and lane (128 chains per SM) keeps the FP64 pipe
+    // ~75 % busy; a round with more items takes proportionally longer.
+    const int grid = h->sm_count;  // one CTA per SM, all resident for the grid barrier
     int budget = grid * SEV_BIS_CHAINS_PER_SM;
     int maxit = 200;
+    const bool small = n <= kBisSmallN;
+    const void *kern = small ? (const void *)bisect_small_kernel : (const void *)bisect_rounds_kernel;
+    const size_t smem = small ? bis_small_smem(n) : 0;
+    if (small)
+        SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bis_small_smem(kBisSmallN)));
+    int per_sm = 0;
+    SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBisThreads, smem));
+    if (per_sm < 1) return SEV_ERR_UNSUPPORTED;
     void *args[] = {(void *)&n, (void *)&d, (void *)&e2, (void *)&par, (void *)&rtol, (void *)&maxit,
                     (void *)&budget, (void *)&eigs, (void *)&W, (void *)&h->d_err};
+    void *args_small[] = {(void *)&n, (void *)&d, (void *)&e2, (void *)&par, (void *)&rtol, (void *)&maxit,
+                          (void *)&budget, (void *)&eigs, (void *)&W.cnt, (void *)&W.ctl, (void *)&h->d_err};
     timing_begin(h, K_BISECT);
-    SEV_CUDA(cudaLaunchCooperativeKernel((const void *)bisect_rounds_kernel, grid, kBisThreads, args, 0, h->stream));
+    SEV_CUDA(cudaLaunchCooperativeKernel(kern, grid, kBisThreads, small ? args_small : args, smem, h->stream));
     timing_end(h, K_BISECT);
     return SEV_OK;
 }
