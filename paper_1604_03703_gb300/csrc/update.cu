@@ -4,14 +4,16 @@
 // Per panel, with U (N x b) and T (b x b) from panel.cu and A22 the lower-
 // stored trailing matrix:
 //   Y  = A22 U                       (symm: reads A22 symmetrically)
-//   X  = Y T                         (= W T in the algorithm's notation)
-//   Zm = T^T (U^T X)
-//   V  = 1/2 U Zm - X                (the V_1 line of Algorithm 4.1)
+//   M  = U^T Y,  Zh = T^T M T / 2    (X = Y T = W T in the algorithm's notation:
+//   V  = U Zh - Y T                   Zh = T^T U^T X / 2, V = U Zh - X, the V_1
+//                                     line of Algorithm 4.1)
 //   A22 <- A22 + U V^T + V U^T       (syr2k, lower tiles only)
 //
 // The FP64 form runs all of it on SIMT tiles (64 x 64 outputs, 4 x 4 per
 // thread, DFMA); the mixed form's symm runs on larger FP32 tiles
 // (symm_f32_kernel) and its syr2k on the tensor cores (update_tc.cu).
+#include <cuda_bf16.h>
+
 #include "common.cuh"
 
 namespace sev {
@@ -23,99 +25,109 @@ size_t panel_workspace(sev_ctx *h, int n, int b);
 template <typename T>
 int tc_update_supported(sev_ctx *h, int N, int b);
 template <typename T>
-int tc_syr2k(sev_ctx *h, int N, int b, T *A22, int lda, const T *U, const T *V, void *ws);
+void tc_panels(int N, int b, void *ws, __nv_bfloat16 **P, __nv_bfloat16 **Q, int *K6p);
+template <typename T>
+int tc_syr2k(sev_ctx *h, int N, int b, T *A22, int lda, void *ws);
 template <typename T>
 size_t tc_workspace(int n, int b);
 template <typename T>
 int tc_symm_supported(sev_ctx *h, int N, int b, const T *A22, int lda);
 template <typename T>
-int tc_symm(sev_ctx *h, int N, int b, const T *A22, int lda, const T *U, T *Y, T *ypart, int max_splits, void *ws);
+int tc_symm(sev_ctx *h, int N, int b, const T *A22, int lda, const T *U, T *ypart, int max_splits, int *splits,
+            void *ws);
 
-constexpr int BM = 64, BN = 64, BK = 16, PADT = 4;
+constexpr int BM = 64, BK = 16, PADT = 4;
 
-template <typename T>
+// A 64 x TN output tile of 256 threads, rows tx + 16 i, columns ty + 16 j
+// (TN = 32 for bands up to 32: a 64-wide tile would do twice the work).
+template <typename T, int TN>
 struct Tile {
     T As[BK][BM + PADT];
-    T Bs[BK][BN + PADT];
+    T Bs[BK][TN + PADT];
 };
 
-template <typename T>
-__device__ __forceinline__ void tile_mma(const Tile<T> &t, T (&acc)[4][4]) {
+template <typename T, int TN>
+__device__ __forceinline__ void tile_mma(const Tile<T, TN> &t, T (&acc)[4][TN / 16]) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
-        T a[4], bb[4];
+        T a[4], bb[TN / 16];
 #pragma unroll
         for (int i = 0; i < 4; ++i) a[i] = t.As[k][tx + 16 * i];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) bb[j] = t.Bs[k][ty + 16 * j];
+        for (int j = 0; j < TN / 16; ++j) bb[j] = t.Bs[k][ty + 16 * j];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * bb[j];
+            for (int j = 0; j < TN / 16; ++j) acc[i][j] += a[i] * bb[j];
     }
 }
 
-// A slab (BM x BK) where element (m, k) = src[m + k*ld] (m contiguous).
+// One thread's share of a slab, loaded into registers: element (m, k) of the
+// A slab and (k, n) of the B slab of the step at k0.
 template <typename T>
-__device__ __forceinline__ void load_a_mcont(Tile<T> &t, const T *src, int ld, int m0, int k0, int M, int K) {
-    for (int idx = threadIdx.x; idx < BM * BK; idx += blockDim.x) {
-        const int m = idx % BM, k = idx / BM;
+__device__ __forceinline__ void symm_slab_a(T (&ra)[4], const T *A, int lda, int N, int m0, int k0, int kend) {
+    const bool below = k0 + BK <= m0, above = k0 >= m0 + BM;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int idx = threadIdx.x + 256 * r;
+        // below and on the diagonal block: down the columns; above it A(m, k) = A(k, m): along k
+        const int m = above ? idx >> 4 : idx & 63, k = above ? idx & 15 : idx >> 6;
         const int gm = m0 + m, gk = k0 + k;
-        t.As[k][m] = (gm < M && gk < K) ? src[(size_t)gm + (size_t)gk * ld] : T(0);
-    }
-}
-// A slab where element (m, k) = src[k + m*ld] (k contiguous).
-template <typename T>
-__device__ __forceinline__ void load_a_kcont(Tile<T> &t, const T *src, int ld, int m0, int k0, int M, int K) {
-    for (int idx = threadIdx.x; idx < BM * BK; idx += blockDim.x) {
-        const int k = idx % BK, m = idx / BK;
-        const int gm = m0 + m, gk = k0 + k;
-        t.As[k][m] = (gm < M && gk < K) ? src[(size_t)gk + (size_t)gm * ld] : T(0);
-    }
-}
-// B slab (BK x BN) where element (k, n) = src[k + n*ld] (k contiguous).
-template <typename T>
-__device__ __forceinline__ void load_b_kcont(Tile<T> &t, const T *src, int ld, int k0, int n0, int K, int N) {
-    for (int idx = threadIdx.x; idx < BK * BN; idx += blockDim.x) {
-        const int k = idx % BK, n = idx / BK;
-        const int gk = k0 + k, gn = n0 + n;
-        t.Bs[k][n] = (gk < K && gn < N) ? src[(size_t)gk + (size_t)gn * ld] : T(0);
-    }
-}
-// B slab where element (k, n) = src[n + k*ld] (n contiguous).
-template <typename T>
-__device__ __forceinline__ void load_b_ncont(Tile<T> &t, const T *src, int ld, int k0, int n0, int K, int N) {
-    for (int idx = threadIdx.x; idx < BK * BN; idx += blockDim.x) {
-        const int n = idx % BN, k = idx / BN;
-        const int gk = k0 + k, gn = n0 + n;
-        t.Bs[k][n] = (gk < K && gn < N) ? src[(size_t)gn + (size_t)gk * ld] : T(0);
+        T v = T(0);
+        if (gm < N && gk < kend)
+            v = (below || (!above && gm >= gk)) ? A[(size_t)gm + (size_t)gk * lda] : A[(size_t)gk + (size_t)gm * lda];
+        ra[r] = v;
     }
 }
 
-// Y = A22 U, A22 symmetric N x N stored in its lower triangle.
-template <typename T>
+// Partial products of Y = A22 U (A22 symmetric N x N, its lower triangle
+// stored): CTA (x, y, z) sums rows [z kchunk, (z + 1) kchunk) of the K range for
+// the 64 x TN tile (x, y); the splits are summed in order by uty_kernel.
+// What bounds it: in FP64 the FP64 pipes (2 FMAs per cycle and SM), so the
+// host picks the number of splits that fills whole waves of CTAs; the next
+// slab's loads are in flight while this one is multiplied.  n = 3001, b = 32,
+// FP64: 148.7 ms per reduction with 64-wide tiles on one wave of 47 CTAs,
+// now 16.9 ms (floor 15.0 ms at
+// 1.2 TFLOP/s).
+template <typename T, int TN>
 __global__ void __launch_bounds__(256) symm_kernel(int N, int b, const T *__restrict__ A, int lda,
-                                                   const T *__restrict__ U, int ldu, T *__restrict__ Y, int ldy) {
-    __shared__ Tile<T> t;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    T acc[4][4] = {};
-    for (int k0 = 0; k0 < N; k0 += BK) {
-        if (k0 + BK <= m0) {
-            load_a_mcont(t, A, lda, m0, k0, N, N);  // strictly below the diagonal
-        } else if (k0 >= m0 + BM) {
-            load_a_kcont(t, A, lda, m0, k0, N, N);  // strictly above: A(m,k) = A(k,m)
-        } else {
-            for (int idx = threadIdx.x; idx < BM * BK; idx += blockDim.x) {
-                const int m = idx % BM, k = idx / BM;
-                const int gm = m0 + m, gk = k0 + k;
-                T v = 0;
-                if (gm < N && gk < N) v = gm >= gk ? A[(size_t)gm + (size_t)gk * lda] : A[(size_t)gk + (size_t)gm * lda];
-                t.As[k][m] = v;
-            }
+                                                   const T *__restrict__ U, int ldu, int kchunk,
+                                                   T *__restrict__ Yout, size_t split_stride) {
+    __shared__ Tile<T, TN> t;
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * TN;
+    const int kbeg = blockIdx.z * kchunk, kend = min(N, kbeg + kchunk);
+    T *Y = Yout + (size_t)blockIdx.z * split_stride;
+    T acc[4][TN / 16] = {};
+    T ra[4], rb[TN / 16];
+    auto slab_b = [&](int k0) {
+#pragma unroll
+        for (int r = 0; r < TN / 16; ++r) {
+            const int idx = threadIdx.x + 256 * r, k = idx & 15, n = idx >> 4;
+            rb[r] = (k0 + k < kend && n0 + n < b) ? U[(size_t)(k0 + k) + (size_t)(n0 + n) * ldu] : T(0);
         }
-        load_b_kcont(t, U, ldu, k0, n0, N, b);
+    };
+    if (kbeg < kend) {
+        symm_slab_a<T>(ra, A, lda, N, m0, kbeg, kend);
+        slab_b(kbeg);
+    }
+    for (int k0 = kbeg; k0 < kend; k0 += BK) {
+        const bool above = k0 >= m0 + BM;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int idx = threadIdx.x + 256 * r;
+            t.As[above ? idx & 15 : idx >> 6][above ? idx >> 4 : idx & 63] = ra[r];
+        }
+#pragma unroll
+        for (int r = 0; r < TN / 16; ++r) {
+            const int idx = threadIdx.x + 256 * r;
+            t.Bs[idx & 15][idx >> 4] = rb[r];
+        }
         __syncthreads();
+        if (k0 + BK < kend) {
+            symm_slab_a<T>(ra, A, lda, N, m0, k0 + BK, kend);
+            slab_b(k0 + BK);
+        }
         tile_mma(t, acc);
         __syncthreads();
     }
@@ -123,9 +135,9 @@ __global__ void __launch_bounds__(256) symm_kernel(int N, int b, const T *__rest
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TN / 16; ++j) {
             const int m = m0 + tx + 16 * i, n = n0 + ty + 16 * j;
-            if (m < N && n < b) Y[(size_t)m + (size_t)n * ldy] = acc[i][j];
+            if (m < N && n < b) Y[(size_t)m + (size_t)n * N] = acc[i][j];
         }
 }
 
@@ -285,116 +297,223 @@ __global__ void __launch_bounds__(256) symm_f32_kernel(int N, int b, const float
     }
 }
 
-// Y = sum over the splits of the partial tiles, in split order.
-__global__ void symm_reduce_kernel(int N, int b, int splits, const float *__restrict__ part, size_t split_stride,
-                                   float *__restrict__ Y, int ldy) {
-    const size_t total = (size_t)N * b;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
-        const int m = (int)(idx % N), n = (int)(idx / N);
-        float s = 0.f;
-        for (int z = 0; z < splits; ++z) s += part[(size_t)z * split_stride + idx];
-        Y[(size_t)m + (size_t)n * ldy] = s;
-    }
-}
-
-int launch_symm_reduce(sev_ctx *h, int N, int b, int splits, const float *part, float *Y) {
-    int g = (int)(((size_t)N * b + 255) / 256);
-    if (g > h->sm_count * 8) g = h->sm_count * 8;
-    SEV_LAUNCH(h, K_SYMM, symm_reduce_kernel, g, 256, 0, N, b, splits, part, (size_t)N * b, Y, N);
-    return SEV_OK;
-}
-
-// C = alpha * A B + beta * D, A (M x K, m contiguous), B (K x Nc, k contiguous, ld ldb).
-// Used for X = Y T and V = 1/2 U Zm - X.
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_nn_kernel(int M, int Nc, int K, T alpha, const T *__restrict__ A, int lda,
-                                                      const T *__restrict__ B, int ldb, T beta,
-                                                      const T *__restrict__ D, int ldd, T *__restrict__ C, int ldc) {
-    __shared__ Tile<T> t;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    T acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        load_a_mcont(t, A, lda, m0, k0, M, K);
-        load_b_kcont(t, B, ldb, k0, n0, K, Nc);
-        __syncthreads();
-        tile_mma(t, acc);
-        __syncthreads();
-    }
+// M_p = U_p^T Y_p (b x b) for row chunk p, with Y = the sum of the symmetric
+// product's split partials in split order (written back when there is more
+// than one; the tiles of a chunk that share Y columns write them once).
+template <typename T, int TN>
+__global__ void __launch_bounds__(256)
+    uty_kernel(int N, int b, int chunk, const T *__restrict__ U, int splits, const T *__restrict__ ypart,
+               size_t split_stride, T *__restrict__ Y, T *__restrict__ part) {
+    constexpr int TM = TN, KB = 32;  // TM x TN outputs, KB rows at a time
+    __shared__ T As[KB][TM + 1], Bs[KB][TN + 1];
+    const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN, p = blockIdx.z;
+    const int kbeg = p * chunk, kend = min(N, kbeg + chunk);
+    constexpr int PER = TN / 16;
+    T acc[PER][PER] = {};
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    constexpr int L = KB * TN / 256;  // elements per thread and operand
+    for (int k0 = kbeg; k0 < kend; k0 += KB) {
+        T ru[L], ry[L];
+        const int k = threadIdx.x & 31, gk = k0 + k;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int r = 0; r < L; ++r) {
+            const int c = (threadIdx.x >> 5) + 8 * r;
+            ru[r] = (gk < kend && m0 + c < b) ? U[(size_t)gk + (size_t)(m0 + c) * N] : T(0);
+            ry[r] = (gk < kend && n0 + c < b) ? ypart[(size_t)gk + (size_t)(n0 + c) * N] : T(0);
+        }
+        for (int z = 1; z < splits; ++z)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int m = m0 + tx + 16 * i, n = n0 + ty + 16 * j;
-            if (m < M && n < Nc) {
-                T v = alpha * acc[i][j];
-                if (beta != T(0)) v += beta * D[(size_t)m + (size_t)n * ldd];
-                C[(size_t)m + (size_t)n * ldc] = v;
+            for (int r = 0; r < L; ++r) {
+                const int c = (threadIdx.x >> 5) + 8 * r;
+                if (gk < kend && n0 + c < b) ry[r] += ypart[(size_t)z * split_stride + gk + (size_t)(n0 + c) * N];
             }
-        }
-}
-
-// Partial products P_s = U[rows_s]^T X[rows_s] (b x b) for row chunk s.
-template <typename T>
-__global__ void __launch_bounds__(256) utx_partial_kernel(int N, int b, int chunk, const T *__restrict__ U, int ldu,
-                                                          const T *__restrict__ X, int ldx, T *__restrict__ part) {
-    __shared__ Tile<T> t;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN, s = blockIdx.z;
-    const int kbeg = s * chunk, kend = min(N, kbeg + chunk);
-    T acc[4][4] = {};
-    for (int k0 = kbeg; k0 < kend; k0 += BK) {
-        // A(m = a, k = i) = U[i, a] (k contiguous); B(k = i, n = c) = X[i, c]
-        for (int idx = threadIdx.x; idx < BM * BK; idx += blockDim.x) {
-            const int k = idx % BK, m = idx / BK;
-            const int gm = m0 + m, gk = k0 + k;
-            t.As[k][m] = (gm < b && gk < kend) ? U[(size_t)gk + (size_t)gm * ldu] : T(0);
-        }
-        for (int idx = threadIdx.x; idx < BK * BN; idx += blockDim.x) {
-            const int k = idx % BK, n = idx / BK;
-            const int gk = k0 + k, gn = n0 + n;
-            t.Bs[k][n] = (gk < kend && gn < b) ? X[(size_t)gk + (size_t)gn * ldx] : T(0);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < L; ++r) {
+            const int c = (threadIdx.x >> 5) + 8 * r;
+            As[k][c] = ru[r];
+            Bs[k][c] = ry[r];
+            if (splits > 1 && m0 == 0 && gk < kend && n0 + c < b) Y[(size_t)gk + (size_t)(n0 + c) * N] = ry[r];
         }
         __syncthreads();
-        tile_mma(t, acc);
-        __syncthreads();
+#pragma unroll 8
+        for (int kk = 0; kk < KB; ++kk) {
+            T a[PER], bb[PER];
+#pragma unroll
+            for (int i = 0; i < PER; ++i) a[i] = As[kk][tx + 16 * i];
+#pragma unroll
+            for (int j = 0; j < PER; ++j) bb[j] = Bs[kk][ty + 16 * j];
+#pragma unroll
+            for (int i = 0; i < PER; ++i)
+#pragma unroll
+                for (int j = 0; j < PER; ++j) acc[i][j] += a[i] * bb[j];
+        }
     }
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    T *P = part + (size_t)s * b * b;
+    T *P = part + (size_t)p * b * b;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < PER; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < PER; ++j) {
             const int m = m0 + tx + 16 * i, n = n0 + ty + 16 * j;
             if (m < b && n < b) P[m + (size_t)n * b] = acc[i][j];
         }
 }
 
-// M = sum_s P_s, entry by entry, the partials in a fixed order (deterministic).
+// M = sum_p M_p, entry by entry, the partials in a fixed order (deterministic).
 template <typename T>
-__global__ void __launch_bounds__(256) utx_sum_kernel(int bb, int nparts, const T *__restrict__ part, T *__restrict__ M) {
+__global__ void __launch_bounds__(256) uty_sum_kernel(int bb, int nparts, const T *__restrict__ part, T *__restrict__ M) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= bb) return;
-    T s = 0;
-    for (int p = 0; p < nparts; ++p) s += part[(size_t)p * bb + idx];
-    M[idx] = s;
+    T s[4] = {};
+    int p = 0;
+    for (; p + 4 <= nparts; p += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s[u] += part[(size_t)(p + u) * bb + idx];
+    for (; p < nparts; ++p) s[0] += part[(size_t)p * bb + idx];
+    M[idx] = (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// Zm = T^T M (M = sum_s P_s, b x b; T upper triangular): CTA handles 4
-// columns; Zm(a, c) = sum_{q <= a} T(q, a) M(q, c), summed in q order.
-template <typename T>
-__global__ void __launch_bounds__(256) utx_tmul_kernel(int b, const T *__restrict__ M, const T *__restrict__ Tm,
-                                                       T *__restrict__ Zm) {
+// Zh = T^T M T / 2 (b x b, T upper triangular), NC columns per CTA: R = M T(:, c)
+// in shared memory, then T^T R; a warp's lanes share a dot product.
+template <typename T, int NC>
+__global__ void __launch_bounds__(256) uty_zh_kernel(int b, const T *__restrict__ M, const T *__restrict__ Tm,
+                                                     T *__restrict__ Zh) {
     extern __shared__ __align__(16) unsigned char smem[];
-    T *Ms = (T *)smem;  // b x 4
-    const int c0 = blockIdx.x * 4;
-    const int nc = min(4, b - c0);
-    for (int idx = threadIdx.x; idx < b * nc; idx += blockDim.x) Ms[idx] = M[idx % b + (size_t)(c0 + idx / b) * b];
+    T *Ts = (T *)smem, *Rs = Ts + (size_t)b * NC;  // T's columns of this CTA; R (b x NC)
+    const int c0 = blockIdx.x * NC, nc = min(NC, b - c0);
+    for (int idx = threadIdx.x; idx < b * nc; idx += 256) Ts[idx] = Tm[(size_t)c0 * b + idx];
     __syncthreads();
-    for (int idx = threadIdx.x; idx < b * nc; idx += blockDim.x) {
+    // R(a, c) = sum_{q <= c} M(a, q) T(q, c): thread per entry, M read along a
+    for (int idx = threadIdx.x; idx < b * nc; idx += 256) {
         const int a = idx % b, c = idx / b;
-        T s = 0;
-        for (int q = 0; q <= a; ++q) s += Tm[q + (size_t)a * b] * Ms[q + (size_t)c * b];
-        Zm[a + (size_t)(c0 + c) * b] = s;
+        T s0 = 0, s1 = 0;
+        int q = 0;
+        for (; q + 1 <= c0 + c; q += 2) {
+            s0 += M[a + (size_t)q * b] * Ts[q + (size_t)c * b];
+            s1 += M[a + (size_t)(q + 1) * b] * Ts[q + 1 + (size_t)c * b];
+        }
+        if (q <= c0 + c) s0 += M[a + (size_t)q * b] * Ts[q + (size_t)c * b];
+        Rs[idx] = s0 + s1;
+    }
+    __syncthreads();
+    // Zh(a, c) = sum_{q <= a} T(q, a) R(q, c) / 2: a warp per entry row a, lanes over q
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int a = warp; a < b; a += 8) {
+        T s[NC] = {};
+        for (int q = lane; q <= a; q += 32) {
+            const T tq = Tm[q + (size_t)a * b];
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (c < nc) s[c] += tq * Rs[q + (size_t)c * b];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (lane == c && c < nc) Zh[a + (size_t)(c0 + c) * b] = T(0.5) * s[c];
+    }
+}
+
+// V = U Zh - Y T for the 64 x TN tile (x, y).  With P and Q (mixed form) V
+// itself is not stored: the tile's U and V go straight into the BF16 operand
+// panels of the tensor-core update (see tc_syr2k), rows of 64 at a time.
+template <typename T, int TN>
+__global__ void __launch_bounds__(256)
+    vform_kernel(int N, int b, const T *__restrict__ U, const T *__restrict__ Y, const T *__restrict__ Zh,
+                 const T *__restrict__ Tm, T *__restrict__ V, int K6p, __nv_bfloat16 *__restrict__ P,
+                 __nv_bfloat16 *__restrict__ Q) {
+    __shared__ Tile<T, TN> t;
+    __shared__ T Vs[BM][TN + 1];
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * TN;
+    T acc[4][TN / 16] = {};
+    // K = 2b: U against Zh, then Y against -T
+    for (int h = 0; h < 2; ++h) {
+        const T *A = h ? Y : U, *B = h ? Tm : Zh;
+        const int klen = h ? min(b, n0 + TN) : b;  // T is upper triangular
+        for (int k0 = 0; k0 < klen; k0 += BK) {
+            T ra[4], rb[TN / 16];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int idx = threadIdx.x + 256 * r, m = idx & 63, k = idx >> 6;
+                ra[r] = (m0 + m < N && k0 + k < b) ? A[(size_t)(m0 + m) + (size_t)(k0 + k) * N] : T(0);
+            }
+#pragma unroll
+            for (int r = 0; r < TN / 16; ++r) {
+                const int idx = threadIdx.x + 256 * r, k = idx & 15, n = idx >> 4;
+                const T v = (k0 + k < b && n0 + n < b) ? B[(k0 + k) + (size_t)(n0 + n) * b] : T(0);
+                rb[r] = h ? -v : v;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int idx = threadIdx.x + 256 * r;
+                t.As[idx >> 6][idx & 63] = ra[r];
+            }
+#pragma unroll
+            for (int r = 0; r < TN / 16; ++r) {
+                const int idx = threadIdx.x + 256 * r;
+                t.Bs[idx & 15][idx >> 4] = rb[r];
+            }
+            __syncthreads();
+            tile_mma(t, acc);
+        }
+    }
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    if (P == nullptr) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < TN / 16; ++j) {
+                const int m = m0 + tx + 16 * i, n = n0 + ty + 16 * j;
+                if (m < N && n < b) V[(size_t)m + (size_t)n * N] = acc[i][j];
+            }
+        return;
+    }
+    if constexpr (sizeof(T) == 4) {
+        // V's tile to rows, then U's: a row's columns are contiguous in P and Q
+        float vv[BM * TN / 256];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < TN / 16; ++j) Vs[tx + 16 * i][ty + 16 * j] = acc[i][j];
+        __syncthreads();
+        const int c = threadIdx.x % TN, r0 = threadIdx.x / TN;
+        constexpr int RS = 256 / TN;
+#pragma unroll
+        for (int q = 0; q < BM / RS; ++q) vv[q] = Vs[r0 + RS * q][c];
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < BM * TN; idx += 256) {
+            const int m = idx & 63, n = idx >> 6;
+            Vs[m][n] = (m0 + m < N && n0 + n < b) ? U[(size_t)(m0 + m) + (size_t)(n0 + n) * N] : T(0);
+        }
+        __syncthreads();
+        const int gc = n0 + c;
+#pragma unroll
+        for (int q = 0; q < BM / RS; ++q) {
+            const int r = r0 + RS * q, gr = m0 + r;
+            if (gr >= N) continue;
+            if (gc < b) {
+                const float u = Vs[r][c], v = vv[q];
+                const __nv_bfloat16 uh = __float2bfloat16_rn(u), vh = __float2bfloat16_rn(v);
+                const __nv_bfloat16 ul = __float2bfloat16_rn(u - __bfloat162float(uh));
+                const __nv_bfloat16 vl = __float2bfloat16_rn(v - __bfloat162float(vh));
+                __nv_bfloat16 *p = P + (size_t)gr * K6p + gc, *w = Q + (size_t)gr * K6p + gc;
+                p[0] = uh, w[0] = vh;
+                p[b] = vh, w[b] = uh;
+                p[2 * b] = uh, w[2 * b] = vl;
+                p[3 * b] = vh, w[3 * b] = ul;
+                p[4 * b] = ul, w[4 * b] = vh;
+                p[5 * b] = vl, w[5 * b] = uh;
+            }
+            // the padding of K to whole 64-wide boxes
+            if (blockIdx.y == 0)
+                for (int k = 6 * b + c; k < K6p; k += TN) {
+                    P[(size_t)gr * K6p + k] = __float2bfloat16_rn(0.f);
+                    Q[(size_t)gr * K6p + k] = __float2bfloat16_rn(0.f);
+                }
+        }
     }
 }
 
@@ -402,7 +521,8 @@ __global__ void __launch_bounds__(256) utx_tmul_kernel(int b, const T *__restric
 template <typename T>
 __global__ void __launch_bounds__(256) syr2k_kernel(int N, int b, T *__restrict__ A, int lda, const T *__restrict__ U,
                                                     int ldu, const T *__restrict__ V, int ldv) {
-    __shared__ Tile<T> t;
+    constexpr int BN = 64;
+    __shared__ Tile<T, BN> t;
     const long x = blockIdx.x;
     int I = (int)((sqrt(8.0 * (double)x + 1.0) - 1.0) * 0.5);
     while ((long)(I + 1) * (I + 2) / 2 <= x) ++I;
@@ -443,31 +563,35 @@ __global__ void __launch_bounds__(256) syr2k_kernel(int N, int b, T *__restrict_
 // --------------------------------------------------------------- driver
 template <typename T>
 struct F2BBuffers {
-    T *U, *Y, *X, *V, *Tm, *Zm, *part, *ypart;
+    T *U, *Y, *V, *Tm, *Zm, *part, *ypart;
     unsigned long long *comm;
     size_t comm_words;
     void *panel_ws, *tc_ws;
 };
 
-constexpr int kSymmMaxSplits = 8;
-
-// Row chunks of U^T X: 256 rows or more each, at most 64 (a wave of CTAs at
-// b = 128: 2 x 2 tiles x 64 chunks).
-static int utx_parts(int N) {
-    int p = (N + 255) / 256;
-    return p < 1 ? 1 : (p > 64 ? 64 : p);
+// Partial products of Y kept at most: FP64 at moderate orders takes up to 16
+// splits (whole waves of CTAs), else 8.
+template <typename T>
+static int symm_max_splits(int n) {
+    return sizeof(T) == 8 && n <= 8192 ? 16 : 8;
 }
+
+// Row chunks of U^T Y: 64 rows or more each, at most 128.
+static int uty_chunk(int N) {
+    const int c = ((N + 127) / 128 + 31) / 32 * 32;
+    return c < 64 ? 64 : c;
+}
+static int uty_parts(int N) { return (N + uty_chunk(N) - 1) / uty_chunk(N); }
 
 template <typename T>
 static void carve_f2b(Carver &c, F2BBuffers<T> &B, sev_ctx *h, int n, int b, bool tc) {
     B.U = c.take<T>((size_t)n * b);
     B.Y = c.take<T>((size_t)n * b);
-    B.X = c.take<T>((size_t)n * b);
     B.V = c.take<T>((size_t)n * b);
     B.Tm = c.take<T>((size_t)b * b);
     B.Zm = c.take<T>((size_t)b * b);
-    B.part = c.take<T>((size_t)(utx_parts(n) + 1) * b * b);  // the chunks' partial products, then their sum
-    B.ypart = c.take<T>((size_t)kSymmMaxSplits * n * b);
+    B.part = c.take<T>((size_t)129 * b * b);  // the chunks' partial products, then their sum
+    B.ypart = c.take<T>((size_t)symm_max_splits<T>(n) * n * b);
     B.tc_ws = tc ? (void *)c.take<char>(tc_workspace<T>(n, b)) : nullptr;
     B.comm_words = panel_coop_words<T>(h, b);
     B.comm = c.take<unsigned long long>(B.comm_words);
@@ -511,50 +635,64 @@ int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab
         }
         if (rc) return rc;
         const bool tc = tc_update_supported<T>(h, N, b);
-        // Y = A22 U
+        // partial products of Y = A22 U
+        int splits = 1;
         if (tc_symm_supported<T>(h, N, b, A22, lda)) {
-            rc = tc_symm<T>(h, N, b, A22, lda, B.U, B.Y, B.ypart, kSymmMaxSplits, B.tc_ws);
+            rc = tc_symm<T>(h, N, b, A22, lda, B.U, B.ypart, symm_max_splits<T>(n), &splits, B.tc_ws);
             if (rc) return rc;
         } else if (sizeof(T) == 4 && lda % 4 == 0 && ((uintptr_t)A22 & 15) == 0) {
             // split K until the grid covers ~2 CTAs per SM
             const int mt = (N + SBM - 1) / SBM, nt = (b + SBN - 1) / SBN;
-            int splits = 1;
-            while (splits < kSymmMaxSplits && mt * nt * splits < 2 * h->sm_count && N / (splits * 2) >= 256) splits *= 2;
+            while (splits < 8 && mt * nt * splits < 2 * h->sm_count && N / (splits * 2) >= 256) splits *= 2;
             const int kchunk = ((N + splits - 1) / splits + SBK - 1) / SBK * SBK;
-            float *dst = splits > 1 ? (float *)B.ypart : (float *)B.Y;
             SEV_LAUNCH(h, K_SYMM, symm_f32_kernel, dim3(mt, nt, splits), 256, 0, N, b, (const float *)A22, lda,
-                       (const float *)B.U, N, kchunk, dst, N, (size_t)N * b);
-            if (splits > 1) {
-                int g = (int)(((size_t)N * b + 255) / 256);
-                if (g > h->sm_count * 8) g = h->sm_count * 8;
-                SEV_LAUNCH(h, K_SYMM, symm_reduce_kernel, g, 256, 0, N, b, splits, (const float *)B.ypart,
-                           (size_t)N * b, (float *)B.Y, N);
-            }
+                       (const float *)B.U, N, kchunk, (float *)B.ypart, N, (size_t)N * b);
         } else {
-            SEV_LAUNCH(h, K_SYMM, symm_kernel<T>, dim3((N + BM - 1) / BM, (b + BN - 1) / BN), 256, 0, N, b, A22, lda,
-                       B.U, N, B.Y, N);
+            const int tn = b <= 32 ? 32 : 64, mt = (N + BM - 1) / BM, nt = (b + tn - 1) / tn;
+            // the number of splits that leaves the last wave of CTAs fullest
+            // (one CTA keeps an SM's FP64 pipes busy), each of 64 rows or more
+            float best = 0.f;
+            for (int z = 1; z <= symm_max_splits<T>(n) && (z == 1 || N / z >= 64); ++z) {
+                const float waves = (float)(mt * nt * z) / (float)h->sm_count;
+                const float eff = waves / ceilf(waves) * (waves < 2.f ? 0.9f : 1.f);
+                if (eff > best + 0.01f) {
+                    best = eff;
+                    splits = z;
+                }
+            }
+            const int kchunk = ((N + splits - 1) / splits + BK - 1) / BK * BK;
+            splits = (N + kchunk - 1) / kchunk;
+            if (tn == 32)
+                SEV_LAUNCH(h, K_SYMM, (symm_kernel<T, 32>), dim3(mt, nt, splits), 256, 0, N, b, A22, lda, B.U, N, kchunk,
+                           B.ypart, (size_t)N * b);
+            else
+                SEV_LAUNCH(h, K_SYMM, (symm_kernel<T, 64>), dim3(mt, nt, splits), 256, 0, N, b, A22, lda, B.U, N, kchunk,
+                           B.ypart, (size_t)N * b);
         }
-        // X = Y T
-        SEV_LAUNCH(h, K_VFORM_XT, gemm_nn_kernel<T>, dim3((N + BM - 1) / BM, (b + BN - 1) / BN), 256, 0, N, b, b, T(1),
-                   B.Y, N, B.Tm, b, T(0), (const T *)nullptr, N, B.X, N);
-        // Zm = T^T (U^T X)
-        const int parts = utx_parts(N);
-        const int chunk = (((N + parts - 1) / parts) + BK - 1) / BK * BK;
-        SEV_LAUNCH(h, K_VFORM_UTX, utx_partial_kernel<T>, dim3((b + BM - 1) / BM, (b + BN - 1) / BN, parts), 256, 0, N,
-                   b, chunk, B.U, N, B.X, N, B.part);
-        {
-            // the chunks summed by b^2 threads, then T^T applied (4 columns a CTA)
-            T *Msum = B.part + (size_t)parts * b * b;
-            SEV_LAUNCH(h, K_VFORM_REDUCE, utx_sum_kernel<T>, (b * b + 255) / 256, 256, 0, b * b, parts, B.part, Msum);
-            SEV_LAUNCH(h, K_VFORM_REDUCE, utx_tmul_kernel<T>, (b + 3) / 4, 256, sizeof(T) * (size_t)b * 4, b, Msum,
-                       B.Tm, B.Zm);
-        }
-        // V = 1/2 U Zm - X
-        SEV_LAUNCH(h, K_VFORM_V, gemm_nn_kernel<T>, dim3((N + BM - 1) / BM, (b + BN - 1) / BN), 256, 0, N, b, b,
-                   T(0.5), B.U, N, B.Zm, b, T(-1), B.X, N, B.V, N);
+        // M = U^T Y; Zh = T^T M T / 2; V = U Zh - Y T (= U (T^T U^T X) / 2 - X with X = Y T)
+        const T *Y = splits > 1 ? B.Y : B.ypart;
+        const int chunk = uty_chunk(N), parts = uty_parts(N);
+        T *Msum = B.part + (size_t)parts * b * b;
+        __nv_bfloat16 *bp = nullptr, *bq = nullptr;
+        int K6p = 0;
+        if (tc) tc_panels<T>(N, b, B.tc_ws, &bp, &bq, &K6p);
+        const size_t s_zh = sizeof(T) * (size_t)b * 8;
+        auto vform = [&](auto tnc) -> int {
+            constexpr int TN = decltype(tnc)::value;
+            const int nt = (b + TN - 1) / TN;
+            SEV_LAUNCH(h, K_VFORM_UTX, (uty_kernel<T, TN>), dim3(nt, nt, parts), 256, 0, N, b, chunk, B.U, splits,
+                       B.ypart, (size_t)N * b, B.Y, B.part);
+            SEV_LAUNCH(h, K_VFORM_REDUCE, uty_sum_kernel<T>, (b * b + 255) / 256, 256, 0, b * b, parts, B.part, Msum);
+            SEV_LAUNCH(h, K_VFORM_REDUCE, (uty_zh_kernel<T, 4>), (b + 3) / 4, 256, s_zh, b, Msum, B.Tm, B.Zm);
+            SEV_LAUNCH(h, K_VFORM_V, (vform_kernel<T, TN>), dim3((N + BM - 1) / BM, nt), 256, 0, N, b, B.U, Y, B.Zm,
+                       B.Tm, B.V, K6p, bp, bq);
+            return SEV_OK;
+        };
+        rc = b <= 32 ? vform(std::integral_constant<int, 32>{}) : vform(std::integral_constant<int, 64>{});
+        if (rc) return rc;
         // A22 += U V^T + V U^T
         if (tc) {
-            rc = tc_syr2k<T>(h, N, b, A22, lda, B.U, B.V, B.tc_ws);
+            rc = tc_syr2k<T>(h, N, b, A22, lda, B.tc_ws);
             if (rc) return rc;
         } else {
             const long nt = (N + BM - 1) / BM;

@@ -138,33 +138,6 @@ constexpr uint32_t kIdescBF16_128x128 =
 constexpr int kTcStages = 3;
 constexpr int kTcStageBytes = 2 * 128 * 64 * 2;  // A + B tile
 
-// ----------------------------------------------------------- split kernel
-__global__ void split_bf16x3_kernel(int N, int b, int K6p, const float *__restrict__ U, const float *__restrict__ V,
-                                    __nv_bfloat16 *__restrict__ P, __nv_bfloat16 *__restrict__ Q) {
-    const long total = (long)N * K6p;
-    for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / K6p), k = (int)(idx % K6p);
-        __nv_bfloat16 p = __float2bfloat16_rn(0.f), q = p;
-        if (k < 6 * b) {
-            const int seg = k / b, c = k % b;
-            const float u = U[(size_t)r + (size_t)c * N], v = V[(size_t)r + (size_t)c * N];
-            const __nv_bfloat16 uh = __float2bfloat16_rn(u), vh = __float2bfloat16_rn(v);
-            const __nv_bfloat16 ul = __float2bfloat16_rn(u - __bfloat162float(uh));
-            const __nv_bfloat16 vl = __float2bfloat16_rn(v - __bfloat162float(vh));
-            switch (seg) {
-                case 0: p = uh; q = vh; break;
-                case 1: p = vh; q = uh; break;
-                case 2: p = uh; q = vl; break;
-                case 3: p = vh; q = ul; break;
-                case 4: p = ul; q = vh; break;
-                default: p = vl; q = uh; break;
-            }
-        }
-        P[idx] = p;
-        Q[idx] = q;
-    }
-}
-
 // ------------------------------------------------------------ GEMM kernel
 __global__ void __launch_bounds__(128, 1)
     syr2k_tc_kernel(const __grid_constant__ CUtensorMap mapP, const __grid_constant__ CUtensorMap mapQ, int N,
@@ -297,7 +270,7 @@ __global__ void __launch_bounds__(128, 1)
 // ------------------------------------------------------ symmetric product
 // Y = A22 U, the first product of the V formation (W = A22 U in Eq. 4.1 /
 // Algorithm 4.1), for FP32 data on the tensor cores in BF16x3:
-// Y ~ Ah Uh + Ah Ul + Al Uh (hi/lo splits as in split_bf16x3_kernel; the
+// Y ~ Ah Uh + Ah Ul + Al Uh (hi/lo splits as above; the
 // Al Ul term, ~2^-16 relative, dropped).
 //
 // CTA (I, s) computes rows [128 I, 128 I + 128) of Y over the 64-wide
@@ -688,19 +661,24 @@ size_t tc_workspace(int n, int b) {
     return c.bytes();
 }
 
+// The operand panels P and Q (N x K6p, rows contiguous), which vform_kernel
+// fills; they follow one another in ws.
 template <typename T>
-int tc_syr2k(sev_ctx *h, int N, int b, T *A22, int lda, const T *U, const T *V, void *ws) {
+void tc_panels(int N, int b, void *ws, __nv_bfloat16 **P, __nv_bfloat16 **Q, int *K6p) {
+    *K6p = k6p_of(b);
+    Carver c(ws);
+    *P = c.take<__nv_bfloat16>((size_t)N * *K6p);
+    *Q = c.take<__nv_bfloat16>((size_t)N * *K6p);
+}
+
+template <typename T>
+int tc_syr2k(sev_ctx *h, int N, int b, T *A22, int lda, void *ws) {
     if constexpr (sizeof(T) != 4) {
         return SEV_ERR_UNSUPPORTED;
     } else {
-        const int K6p = k6p_of(b);
-        Carver c(ws);
-        __nv_bfloat16 *P = c.take<__nv_bfloat16>((size_t)N * K6p);
-        __nv_bfloat16 *Q = c.take<__nv_bfloat16>((size_t)N * K6p);
-        const long total = (long)N * K6p;
-        int g = (int)((total + 255) / 256);
-        if (g > h->sm_count * 32) g = h->sm_count * 32;
-        SEV_LAUNCH(h, K_SPLIT_BF16, split_bf16x3_kernel, g, 256, 0, N, b, K6p, U, V, P, Q);
+        __nv_bfloat16 *P, *Q;
+        int K6p;
+        tc_panels<T>(N, b, ws, &P, &Q, &K6p);
         CUtensorMap mP, mQ;
         int rc = make_map(&mP, P, N, K6p);
         if (rc) return rc;
@@ -724,10 +702,11 @@ int tc_symm_supported(sev_ctx *h, int N, int b, const T *A22, int lda) {
     return (b == 32 || b == 64 || b == 128) && N >= 256 && lda % 4 == 0 && ((uintptr_t)A22 & 15) == 0;
 }
 
-// Y = A22 U on the tensor cores; partial products of the K splits go to
-// ypart (kSymmMaxSplits x N x b) and are summed in split order into Y.
+// Y = A22 U on the tensor cores: the partial products of the K splits go to
+// ypart (*splits x N x b); their sum in split order is Y.
 template <typename T>
-int tc_symm(sev_ctx *h, int N, int b, const T *A22, int lda, const T *U, T *Y, T *ypart, int max_splits, void *ws) {
+int tc_symm(sev_ctx *h, int N, int b, const T *A22, int lda, const T *U, T *ypart, int max_splits, int *splits,
+            void *ws) {
     if constexpr (sizeof(T) != 4) {
         return SEV_ERR_UNSUPPORTED;
     } else {
@@ -753,27 +732,24 @@ int tc_symm(sev_ctx *h, int N, int b, const T *A22, int lda, const T *U, T *Y, T
         const size_t smem = (size_t)kSyRaw * kSyRawBytes + (size_t)kSyCvt * sy_cvt_bytes(b) + 1024;
         auto kern = b == 128 ? symm_tc_kernel<128> : (b == 64 ? symm_tc_kernel<64> : symm_tc_kernel<32>);
         SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        float *dst = S > 1 ? (float *)ypart : (float *)Y;
         SEV_LAUNCH(h, K_SYMM, kern, dim3(rb, S), kSyThreads, smem, mAc, mAr, mUh, mUl, (const float *)A22, lda, N, per,
-                   dst, (size_t)N * b, h->d_err);
-        if (S > 1) {
-            rc = launch_symm_reduce(h, N, b, S, (const float *)ypart, (float *)Y);
-            if (rc) return rc;
-        }
+                   (float *)ypart, (size_t)N * b, h->d_err);
+        *splits = S;
         return SEV_OK;
     }
 }
 
 template int tc_update_supported<float>(sev_ctx *, int, int);
 template int tc_update_supported<double>(sev_ctx *, int, int);
-template int tc_syr2k<float>(sev_ctx *, int, int, float *, int, const float *, const float *, void *);
-template int tc_syr2k<double>(sev_ctx *, int, int, double *, int, const double *, const double *, void *);
+template void tc_panels<float>(int, int, void *, __nv_bfloat16 **, __nv_bfloat16 **, int *);
+template void tc_panels<double>(int, int, void *, __nv_bfloat16 **, __nv_bfloat16 **, int *);
+template int tc_syr2k<float>(sev_ctx *, int, int, float *, int, void *);
+template int tc_syr2k<double>(sev_ctx *, int, int, double *, int, void *);
 template size_t tc_workspace<float>(int, int);
 template int tc_symm_supported<float>(sev_ctx *, int, int, const float *, int);
 template int tc_symm_supported<double>(sev_ctx *, int, int, const double *, int);
-template int tc_symm<float>(sev_ctx *, int, int, const float *, int, const float *, float *, float *, int, void *);
-template int tc_symm<double>(sev_ctx *, int, int, const double *, int, const double *, double *, double *, int,
-                             void *);
+template int tc_symm<float>(sev_ctx *, int, int, const float *, int, const float *, float *, int, int *, void *);
+template int tc_symm<double>(sev_ctx *, int, int, const double *, int, const double *, double *, int, int *, void *);
 template size_t tc_workspace<double>(int, int);
 
 }  // namespace sev
