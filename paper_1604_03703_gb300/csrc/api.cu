@@ -189,7 +189,14 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     const int ldab = 2 * b0 > 2 ? 2 * b0 : 2;
     void *ws = nullptr;
     const size_t need = eig_workspace<T>(h, n, b0);
-    int rc = get_workspace(h, need, &ws);
+    // (a caller's workspace of the queried size has no room for the copy; the
+    // reduction then runs on A as it is)
+    size_t copy = full_to_band_copy_bytes<T>(h, n, b0, A, lda);
+    int rc = get_workspace(h, need + copy, &ws);
+    if (rc && copy) {
+        copy = 0;
+        rc = get_workspace(h, need, &ws);
+    }
     if (rc) return rc;
     Carver c(ws);
     T *AB = c.take<T>((size_t)ldab * n);
@@ -202,10 +209,12 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     // (bounded work, no data-dependent control flow) and the bisection,
     // whose step count depends on the data, is skipped (NaN eigenvalues)
     SEV_CUDA(cudaMemsetAsync(nonfinite, 0, sizeof(int), h->stream));
-    rc = launch_check_finite<T>(h, n, A, lda, nonfinite);
+    T *const work = copy ? (T *)((char *)ws + need) : A;
+    const int ldw = copy ? copy_ld(n) : lda;
+    rc = launch_check_finite<T>(h, n, A, lda, nonfinite, copy ? work : nullptr, ldw);
     if (rc) return rc;
     if (b0 < n - 1) {
-        rc = launch_full_to_band<T>(h, n, A, lda, b0, AB, ldab, stage, stage_bytes);
+        rc = launch_full_to_band<T>(h, n, work, ldw, b0, AB, ldab, stage, stage_bytes);
     } else {
         rc = launch_band_from_dense<T>(h, n, A, lda, b0, AB, ldab);
     }
@@ -218,6 +227,27 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     if (rc) return rc;
     const double rtol = sizeof(T) == 8 ? 1e-14 : 1e-9;
     return launch_bisect(h, n, d, e, rtol, eigs, stage, stage_bytes, nonfinite);
+}
+
+// sev_full_to_band past its argument checks.
+template <typename T>
+static int full_to_band_t(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab) {
+    const size_t need = full_to_band_workspace<T>(h, n, b);
+    size_t copy = full_to_band_copy_bytes<T>(h, n, b, A, lda);
+    void *ws = nullptr;
+    int rc = get_workspace(h, need + copy, &ws);
+    if (rc && copy) {
+        copy = 0;
+        rc = get_workspace(h, need, &ws);
+    }
+    if (rc) return rc;
+    T *const work = copy ? (T *)((char *)ws + need) : A;
+    const int ldw = copy ? copy_ld(n) : lda;
+    rc = launch_check_finite<T>(h, n, A, lda, nullptr, copy ? work : nullptr, ldw);
+    if (rc) return rc;
+    rc = launch_full_to_band<T>(h, n, work, ldw, b, AB, ldab, ws, need);
+    if (rc || !copy) return rc;
+    return launch_dense_from_band<T>(h, n, A, lda, b, AB, ldab);
 }
 
 }  // namespace sev
@@ -384,7 +414,8 @@ int sev_eigvalsh_host(sev_handle h, int n, const void *A_host, int lda, int b0, 
     if (n == 0) return SEV_OK;
     if (cudaSetDevice(h->device) != cudaSuccess) return SEV_ERR_CUDA;
     const size_t es = prec == SEV_FP64 ? sizeof(double) : sizeof(float);
-    const size_t abytes = ((es * (size_t)n * n + 255) & ~(size_t)255);
+    const int ld = copy_ld(n);  // aligned columns whatever the order
+    const size_t abytes = ((es * (size_t)n * ld + 255) & ~(size_t)255);
     const size_t need = abytes + sizeof(double) * (size_t)n;
     if (h->h_stage_bytes < need) {
         if (h->h_stage) {
@@ -401,8 +432,8 @@ int sev_eigvalsh_host(sev_handle h, int n, const void *A_host, int lda, int b0, 
     }
     void *dA = h->h_stage;
     double *dE = (double *)((char *)h->h_stage + abytes);
-    SEV_CUDA(cudaMemcpy2DAsync(dA, es * n, A_host, es * lda, es * n, n, cudaMemcpyHostToDevice, h->stream));
-    int rc = sev_eigvalsh(h, n, dA, n, b0, prec, dE);
+    SEV_CUDA(cudaMemcpy2DAsync(dA, es * ld, A_host, es * lda, es * n, n, cudaMemcpyHostToDevice, h->stream));
+    int rc = sev_eigvalsh(h, n, dA, ld, b0, prec, dE);
     if (rc) return rc;
     SEV_CUDA(cudaMemcpyAsync(eigs_host, dE, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
     return sev_get_error(h);
@@ -423,15 +454,8 @@ int sev_full_to_band(sev_handle h, int n, void *A, int lda, int b, int prec, voi
         return prec == SEV_FP64 ? launch_band_from_dense<double>(h, n, (double *)A, lda, b, (double *)AB, ldab)
                                 : launch_band_from_dense<float>(h, n, (float *)A, lda, b, (float *)AB, ldab);
     }
-    const size_t need = prec == SEV_FP64 ? full_to_band_workspace<double>(h, n, b) : full_to_band_workspace<float>(h, n, b);
-    void *ws = nullptr;
-    int rc = get_workspace(h, need, &ws);
-    if (rc) return rc;
-    rc = prec == SEV_FP64 ? launch_check_finite<double>(h, n, (const double *)A, lda, nullptr)
-                          : launch_check_finite<float>(h, n, (const float *)A, lda, nullptr);
-    if (rc) return rc;
-    return prec == SEV_FP64 ? launch_full_to_band<double>(h, n, (double *)A, lda, b, (double *)AB, ldab, ws, need)
-                            : launch_full_to_band<float>(h, n, (float *)A, lda, b, (float *)AB, ldab, ws, need);
+    return prec == SEV_FP64 ? full_to_band_t<double>(h, n, (double *)A, lda, b, (double *)AB, ldab)
+                            : full_to_band_t<float>(h, n, (float *)A, lda, b, (float *)AB, ldab);
 }
 
 int sev_band_to_band(sev_handle h, int n, void *AB, int ldab, int b, int hh, int prec) {
@@ -547,8 +571,9 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
     size_t need = 0;
     for (const auto &g : P->big) {
         const int b0 = pick_b0(h, g.n, prec);
-        const size_t w = prec == SEV_FP64 ? eig_workspace<double>(h, g.n, b0 > g.n - 1 ? g.n - 1 : b0)
-                                          : eig_workspace<float>(h, g.n, b0 > g.n - 1 ? g.n - 1 : b0);
+        const int bc = b0 > g.n - 1 ? g.n - 1 : b0;
+        size_t w = prec == SEV_FP64 ? eig_workspace<double>(h, g.n, bc) : eig_workspace<float>(h, g.n, bc);
+        if (prec == SEV_MIXED && !h->ws_ext) w += full_to_band_copy_bytes<float>(h, g.n, bc, (const float *)g.A, g.lda);
         if (w > need) need = w;
     }
     if (need) {

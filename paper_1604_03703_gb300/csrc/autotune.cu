@@ -177,8 +177,9 @@ static int autotune_t(sev_ctx *h, int n, int prec, int b0_req, TunedBands *out, 
         const size_t f = full_to_band_workspace<T>(h, n, cand_b0[q]);
         if (f > stage) stage = f;
     }
+    const int ldn = copy_ld(n);  // aligned columns, as the solver's working copy has them
     Carver cv(nullptr);
-    cv.take<T>((size_t)n * n);
+    cv.take<T>((size_t)ldn * n);
     cv.take<T>((size_t)ldab * n);
     const size_t own = cv.bytes();
     char *buf = nullptr;
@@ -187,7 +188,7 @@ static int autotune_t(sev_ctx *h, int n, int prec, int b0_req, TunedBands *out, 
         return SEV_ERR_WORKSPACE;
     }
     Carver c(buf);
-    T *A = c.take<T>((size_t)n * n);
+    T *A = c.take<T>((size_t)ldn * n);
     T *AB = c.take<T>((size_t)ldab * n);
     void *ws = nullptr;
     int rc = get_workspace(h, stage, &ws);
@@ -245,16 +246,16 @@ static int autotune_t(sev_ctx *h, int n, int prec, int b0_req, TunedBands *out, 
         const int b0 = cand_b0[q], l = wlog(b0);
         if (best[l] < 0.0) continue;
         const int nw = 2 * b0 + 2 < n ? 2 * b0 + 2 : n;  // warm-up order: a couple of panels
-        tune_fill_sym_kernel<T><<<grid, 256, 0, h->stream>>>(nw, A, nw, 0xF00Dull);
-        rc = launch_full_to_band<T>(h, nw, A, nw, b0, AB, ldab, ws, stage);
+        tune_fill_sym_kernel<T><<<grid, 256, 0, h->stream>>>(nw, A, ldn, 0xF00Dull);
+        rc = launch_full_to_band<T>(h, nw, A, ldn, b0, AB, ldab, ws, stage);
         if (rc == SEV_ERR_UNSUPPORTED) {  // this width has no full-to-band kernel here
             rc = SEV_OK;
             continue;
         }
         if (rc) break;
-        tune_fill_sym_kernel<T><<<grid, 256, 0, h->stream>>>(n, A, n, 0xF00Eull + b0);
+        tune_fill_sym_kernel<T><<<grid, 256, 0, h->stream>>>(n, A, ldn, 0xF00Eull + b0);
         float ms = 0.f;
-        rc = time_ms(h, [&] { return launch_full_to_band<T>(h, n, A, n, b0, AB, ldab, ws, stage); }, &ms);
+        rc = time_ms(h, [&] { return launch_full_to_band<T>(h, n, A, ldn, b0, AB, ldab, ws, stage); }, &ms);
         if (rc == SEV_ERR_UNSUPPORTED) {
             rc = SEV_OK;
             continue;

@@ -62,12 +62,18 @@ int launch_tridiag_extract(sev_ctx *h, int n, const T *AB, int ldab, double *d, 
 }
 
 // Non-finite scan of the lower triangle (diagonal included): CTA c takes
-// columns c, c + grid, ...; its threads read down a column (coalesced).
+// columns c, c + grid, ...; its threads read down a column (coalesced).  With
+// dst the triangle is copied to it on the way (leading dimension ldd).
 template <typename T>
-__global__ void check_finite_kernel(int n, const T *__restrict__ A, int lda, int *__restrict__ flag, int *err) {
+__global__ void check_finite_kernel(int n, const T *__restrict__ A, int lda, int *__restrict__ flag, int *err,
+                                    T *__restrict__ dst, int ldd) {
     bool bad = false;
     for (int j = blockIdx.x; j < n; j += gridDim.x)
-        for (int i = j + threadIdx.x; i < n; i += blockDim.x) bad |= !isfinite(A[(size_t)i + (size_t)j * lda]);
+        for (int i = j + threadIdx.x; i < n; i += blockDim.x) {
+            const T v = A[(size_t)i + (size_t)j * lda];
+            bad |= !isfinite(v);
+            if (dst) dst[(size_t)i + (size_t)j * ldd] = v;
+        }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) {
         latch_error(err, SEV_ERR_NONFINITE);
         if (flag) atomicExch(flag, 1);
@@ -75,15 +81,34 @@ __global__ void check_finite_kernel(int n, const T *__restrict__ A, int lda, int
 }
 
 template <typename T>
-int launch_check_finite(sev_ctx *h, int n, const T *A, int lda, int *flag) {
+int launch_check_finite(sev_ctx *h, int n, const T *A, int lda, int *flag, T *dst, int ldd) {
     if (n <= 0) return SEV_OK;
     int grid = n < h->sm_count * 8 ? n : h->sm_count * 8;
-    SEV_LAUNCH(h, K_CHECK_FINITE, check_finite_kernel<T>, grid, kThreads, 0, n, A, lda, flag, h->d_err);
+    SEV_LAUNCH(h, K_CHECK_FINITE, check_finite_kernel<T>, grid, kThreads, 0, n, A, lda, flag, h->d_err, dst, ldd);
     return SEV_OK;
 }
 
-template int launch_check_finite<float>(sev_ctx *, int, const float *, int, int *);
-template int launch_check_finite<double>(sev_ctx *, int, const double *, int, int *);
+// The lower triangle of A from the packed band (half-bandwidth b): the band's
+// entries and exact zeros below them.
+template <typename T>
+__global__ void dense_from_band_kernel(int n, T *__restrict__ A, int lda, int b, const T *__restrict__ AB, int ldab) {
+    for (int j = blockIdx.x; j < n; j += gridDim.x)
+        for (int i = j + threadIdx.x; i < n; i += blockDim.x)
+            A[(size_t)i + (size_t)j * lda] = i - j <= b ? AB[(i - j) + (size_t)j * ldab] : T(0);
+}
+
+template <typename T>
+int launch_dense_from_band(sev_ctx *h, int n, T *A, int lda, int b, const T *AB, int ldab) {
+    if (n <= 0) return SEV_OK;
+    int grid = n < h->sm_count * 8 ? n : h->sm_count * 8;
+    SEV_LAUNCH(h, K_BAND_FROM_DENSE, dense_from_band_kernel<T>, grid, kThreads, 0, n, A, lda, b, AB, ldab);
+    return SEV_OK;
+}
+
+template int launch_dense_from_band<float>(sev_ctx *, int, float *, int, int, const float *, int);
+template int launch_dense_from_band<double>(sev_ctx *, int, double *, int, int, const double *, int);
+template int launch_check_finite<float>(sev_ctx *, int, const float *, int, int *, float *, int);
+template int launch_check_finite<double>(sev_ctx *, int, const double *, int, int *, double *, int);
 template int launch_band_from_dense<float>(sev_ctx *, int, const float *, int, int, float *, int);
 template int launch_band_from_dense<double>(sev_ctx *, int, const double *, int, int, double *, int);
 template int launch_tridiag_extract<float>(sev_ctx *, int, const float *, int, double *, double *);
