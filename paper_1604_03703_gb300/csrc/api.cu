@@ -214,7 +214,7 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     rc = launch_check_finite<T>(h, n, A, lda, nonfinite, copy ? work : nullptr, ldw);
     if (rc) return rc;
     if (b0 < n - 1) {
-        rc = launch_full_to_band<T>(h, n, work, ldw, b0, AB, ldab, stage, stage_bytes);
+        rc = launch_full_to_band<T>(h, n, work, ldw, b0, AB, ldab, stage, stage_bytes, copy != 0);
     } else {
         rc = launch_band_from_dense<T>(h, n, A, lda, b0, AB, ldab);
     }
@@ -245,7 +245,7 @@ static int full_to_band_t(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ld
     const int ldw = copy ? copy_ld(n) : lda;
     rc = launch_check_finite<T>(h, n, A, lda, nullptr, copy ? work : nullptr, ldw);
     if (rc) return rc;
-    rc = launch_full_to_band<T>(h, n, work, ldw, b, AB, ldab, ws, need);
+    rc = launch_full_to_band<T>(h, n, work, ldw, b, AB, ldab, ws, need, copy != 0);
     if (rc || !copy) return rc;
     return launch_dense_from_band<T>(h, n, A, lda, b, AB, ldab);
 }
@@ -414,8 +414,7 @@ int sev_eigvalsh_host(sev_handle h, int n, const void *A_host, int lda, int b0, 
     if (n == 0) return SEV_OK;
     if (cudaSetDevice(h->device) != cudaSuccess) return SEV_ERR_CUDA;
     const size_t es = prec == SEV_FP64 ? sizeof(double) : sizeof(float);
-    const int ld = copy_ld(n);  // aligned columns whatever the order
-    const size_t abytes = ((es * (size_t)n * ld + 255) & ~(size_t)255);
+    const size_t abytes = ((es * (size_t)n * n + 255) & ~(size_t)255);
     const size_t need = abytes + sizeof(double) * (size_t)n;
     if (h->h_stage_bytes < need) {
         if (h->h_stage) {
@@ -432,8 +431,8 @@ int sev_eigvalsh_host(sev_handle h, int n, const void *A_host, int lda, int b0, 
     }
     void *dA = h->h_stage;
     double *dE = (double *)((char *)h->h_stage + abytes);
-    SEV_CUDA(cudaMemcpy2DAsync(dA, es * ld, A_host, es * lda, es * n, n, cudaMemcpyHostToDevice, h->stream));
-    int rc = sev_eigvalsh(h, n, dA, ld, b0, prec, dE);
+    SEV_CUDA(cudaMemcpy2DAsync(dA, es * n, A_host, es * lda, es * n, n, cudaMemcpyHostToDevice, h->stream));
+    int rc = sev_eigvalsh(h, n, dA, n, b0, prec, dE);
     if (rc) return rc;
     SEV_CUDA(cudaMemcpyAsync(eigs_host, dE, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
     return sev_get_error(h);

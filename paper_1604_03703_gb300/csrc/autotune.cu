@@ -255,7 +255,7 @@ static int autotune_t(sev_ctx *h, int n, int prec, int b0_req, TunedBands *out, 
         if (rc) break;
         tune_fill_sym_kernel<T><<<grid, 256, 0, h->stream>>>(n, A, ldn, 0xF00Eull + b0);
         float ms = 0.f;
-        rc = time_ms(h, [&] { return launch_full_to_band<T>(h, n, A, ldn, b0, AB, ldab, ws, stage); }, &ms);
+        rc = time_ms(h, [&] { return launch_full_to_band<T>(h, n, A, ldn, b0, AB, ldab, ws, stage, n % 4 != 0); }, &ms);
         if (rc == SEV_ERR_UNSUPPORTED) {
             rc = SEV_OK;
             continue;

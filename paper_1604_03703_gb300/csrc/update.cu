@@ -606,22 +606,24 @@ size_t full_to_band_workspace(sev_ctx *h, int n, int b) {
     return c.bytes();
 }
 
-// The tensor-core product loads A22 by TMA: 16-byte aligned base and columns.
-// An FP32 matrix that has neither (an odd order in contiguous storage: three
-// orders of four) is reduced in an aligned copy of its lower triangle, made
-// by the pass that looks for NaN and Inf: n = 2731, b = 64 7.1 -> 0.9 ms of
-// products per reduction for ~10 us of copying.  Below ~512 rows the SIMT
-// product costs no more.
+// An FP32 matrix without 16-byte aligned columns (an odd order in contiguous
+// storage: three orders of four) is multiplied in FP32 by SIMT tiles -- the
+// tensor-core product needs TMA, and its BF16x3 splits are less exact, so such
+// matrices do not change over to it.  The SIMT kernel with 16-byte loads and a
+// split K range wants aligned columns too, so the reduction runs on an aligned
+// copy of the lower triangle, made by the pass that looks for NaN and Inf:
+// n = 2731, b = 64 7.1 -> 1.6 ms of products per reduction for ~10 us of
+// copying.  Below ~512 rows it makes no difference.
 template <typename T>
 size_t full_to_band_copy_bytes(sev_ctx *h, int n, int b, const T *A, int lda) {
     if (sizeof(T) != 4 || n - b < 512 || b >= n - 1) return 0;
     if (lda % 4 == 0 && ((uintptr_t)A & 15) == 0) return 0;
-    if (!tc_symm_supported<T>(h, n - b, b, (const T *)nullptr, 4)) return 0;
     return (sizeof(T) * (size_t)copy_ld(n) * n + 255) & ~(size_t)255;
 }
 
 template <typename T>
-int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab, void *ws, size_t ws_bytes) {
+int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab, void *ws, size_t ws_bytes,
+                        bool fp32_product) {
     if (n <= 0) return SEV_OK;
     if (ws_bytes < full_to_band_workspace<T>(h, n, b)) return SEV_ERR_WORKSPACE;
     Carver c(ws);
@@ -651,7 +653,7 @@ int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab
         const bool tc = tc_update_supported<T>(h, N, b);
         // partial products of Y = A22 U
         int splits = 1;
-        if (tc_symm_supported<T>(h, N, b, A22, lda)) {
+        if (!fp32_product && tc_symm_supported<T>(h, N, b, A22, lda)) {
             rc = tc_symm<T>(h, N, b, A22, lda, B.U, B.ypart, symm_max_splits<T>(n), &splits, B.tc_ws);
             if (rc) return rc;
         } else if (sizeof(T) == 4 && lda % 4 == 0 && ((uintptr_t)A22 & 15) == 0) {
@@ -717,8 +719,8 @@ int launch_full_to_band(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab
     return launch_band_from_dense<T>(h, n, A, lda, b, AB, ldab);
 }
 
-template int launch_full_to_band<float>(sev_ctx *, int, float *, int, int, float *, int, void *, size_t);
-template int launch_full_to_band<double>(sev_ctx *, int, double *, int, int, double *, int, void *, size_t);
+template int launch_full_to_band<float>(sev_ctx *, int, float *, int, int, float *, int, void *, size_t, bool);
+template int launch_full_to_band<double>(sev_ctx *, int, double *, int, int, double *, int, void *, size_t, bool);
 template size_t full_to_band_copy_bytes<float>(sev_ctx *, int, int, const float *, int);
 template size_t full_to_band_copy_bytes<double>(sev_ctx *, int, int, const double *, int);
 template size_t full_to_band_workspace<float>(sev_ctx *, int, int);
