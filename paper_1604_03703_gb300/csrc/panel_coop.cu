@@ -12,9 +12,9 @@
 // exchange through L2 takes ~0.7 us and a column of a leaf or node QR
 // ~1.5-2 us.  Direct columns need neither the way down nor the reconstruction:
 // U, tau and R are the result (the same reflectors: beta = -sgn(alpha) ||x||,
-// tau in [1, 2]).  Measured (GB300): the whole panel
-// step at n = 16384, b = 128 (FP32) 276 -> 93 ms per reduction, n = 8192,
-// b = 64 101 -> 24 ms; n = 3001, b = 32 in FP64 200 -> 21 ms.
+// tau in [1, 2]).  Measured (GB300): the whole panel step at n = 16384, b = 128
+// (FP32) 276 -> 83 ms per reduction, n = 8192, b = 64 101 -> 19 ms, n = 2048, b =
+// 64 16.1 -> 4.0 ms; n = 3001, b = 32 in FP64 200 -> 16 ms.
 //
 // One exchange per column.  With x = column k below row k (zero above) and
 // v = e_k + x / (alpha - beta), the products v^T a_j that the reflector needs
@@ -30,8 +30,10 @@
 // accesses: a word whose tag is right is complete, so no fence, flag or
 // barrier is needed.  Two sets of words alternate: a CTA sends column k + 1
 // only after it has read all of column k, so whoever has read column k + 1
-// knows that column k's words may be overwritten.  All CTAs are resident
-// (cooperative launch, at most one CTA per SM); every wait is capped and latches
+// knows that column k's words may be overwritten.  Panels of up to 4096 rows
+// (FP64: 1024) run on one cluster of at most 16 CTAs, the words going from
+// shared memory to shared memory; taller ones on the whole GPU (cooperative
+// launch, at most one CTA per SM) through L2.  Every wait is capped and latches
 // SEV_ERR_TIMEOUT on expiry.
 //
 // What bounds it: the chain of one column -- dot products and their warp sums,
@@ -42,17 +44,39 @@
 
 namespace sev {
 
-constexpr int kCoopWarps = 16;                       // column warps; one more for the scalars
-constexpr int kCoopThreads = (kCoopWarps + 1) * 32;
+// NW column warps and one more for the scalars.  8 column warps hold up to 64
+// columns (fewer warps: fewer sums, barriers and copies of x per column); 16
+// hold 128.
 constexpr int kCoopMaxB = 128;
 
 // ------------------------------------------------------- tagged words
-__device__ __forceinline__ void ll_put(unsigned long long *p, unsigned v, unsigned tag) {
-    const unsigned long long w = ((unsigned long long)tag << 32) | v;
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+// CL = false: words in global memory.  CL = true: every CTA of the cluster has
+// the whole exchange buffer in its shared memory; a value is stored into each
+// peer's copy (at the peer's address of the buffer) and polled in the own one.
+__device__ __forceinline__ unsigned ll_peer(const void *own, int peer) {
+    unsigned at;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(at)
+                 : "r"((unsigned)__cvta_generic_to_shared(own)), "r"(peer));
+    return at;
 }
+template <bool CL>
+__device__ __forceinline__ void ll_put(unsigned long long *buf, unsigned peer, size_t word, unsigned v, unsigned tag) {
+    const unsigned long long w = ((unsigned long long)tag << 32) | v;
+    if constexpr (CL)
+        asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(peer + 8 * (unsigned)word), "l"(w) : "memory");
+    else
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(buf + word), "l"(w) : "memory");
+}
+template <bool CL>
 __device__ __forceinline__ void ll_get2(const unsigned long long *p, unsigned long long &a, unsigned long long &b) {
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    if constexpr (CL)
+        asm volatile("ld.relaxed.cluster.shared::cta.v2.u64 {%0, %1}, [%2];"
+                     : "=l"(a), "=l"(b)
+                     : "r"((unsigned)__cvta_generic_to_shared(p))
+                     : "memory");
+    else
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
 }
 __device__ __forceinline__ bool ll_is(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
 
@@ -67,22 +91,29 @@ template <>
 struct LLType<double> {
     static constexpr int W = 2;
 };
-__device__ __forceinline__ void ll_put_val(unsigned long long *p, float v, unsigned tag) {
-    ll_put(p, __float_as_uint(v), tag);
+template <bool CL>
+__device__ __forceinline__ void ll_put_val(unsigned long long *buf, unsigned peer, size_t word, float v, unsigned tag) {
+    ll_put<CL>(buf, peer, word, __float_as_uint(v), tag);
 }
-__device__ __forceinline__ void ll_put_val(unsigned long long *p, double v, unsigned tag) {
-    ll_put(p, (unsigned)__double2loint(v), tag);
-    ll_put(p + 1, (unsigned)__double2hiint(v), tag);
+template <bool CL>
+__device__ __forceinline__ void ll_put_val(unsigned long long *buf, unsigned peer, size_t word, double v, unsigned tag) {
+    ll_put<CL>(buf, peer, word, (unsigned)__double2loint(v), tag);
+    ll_put<CL>(buf, peer, word + 1, (unsigned)__double2hiint(v), tag);
+}
+__device__ __forceinline__ void coop_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Layout of the exchange buffer (in words) for at most cmax CTAs (even).
+// Layout of the exchange buffer (in words) for at most cmax - 1 CTAs (cmax
+// even): per column one entry per CTA, its share of x^T a_j, and behind them
+// the entry of row k; then two words per CTA for its share of x^T x.
 template <typename T>
 struct CoopComm {
     static __host__ __device__ size_t col_words(int b, int cmax) { return (size_t)b * cmax * LLType<T>::W; }
-    static __host__ __device__ size_t row_words(int b) { return (size_t)b * 2; }
     static __host__ __device__ size_t ssq_words(int cmax) { return (size_t)cmax * 2; }
-    // two alternating sets of (columns, row k, squares), then the largest entries
-    static __host__ __device__ size_t set_words(int b, int cmax) { return col_words(b, cmax) + row_words(b) + ssq_words(cmax); }
+    // two alternating sets of (columns, squares), then the largest entries
+    static __host__ __device__ size_t set_words(int b, int cmax) { return col_words(b, cmax) + ssq_words(cmax); }
     static __host__ __device__ size_t words(int b, int cmax) { return 2 * set_words(b, cmax) + ssq_words(cmax); }
 };
 
@@ -108,96 +139,117 @@ __device__ __forceinline__ T warp_sums_t(T (&d)[Q]) {
     }
 }
 
-// This warp's columns' totals over the C CTAs: lane group sums in a fixed
-// order.  Polls until every word carries `tag`; false when the wait ran out.
-template <typename T, int Q>
-__device__ __forceinline__ bool coop_collect(const unsigned long long *cols, int cmax, int C, int warp, int b,
-                                             unsigned tag, long long cap, int *err, T (&sum)[Q]) {
+// A failed try of a polling loop: true when the wait has to be given up.
+__device__ __forceinline__ bool coop_give_up(int tries, long long &t0, long long cap, int *err) {
+    if (tries == 0) t0 = clock64();
+    int stop = 0;
+    if ((threadIdx.x & 31) == 0) {
+        if ((tries & 31) == 31 && *(volatile int *)err != 0) stop = 1;
+        if (wait_expired(t0, cap)) {
+            latch_error(err, SEV_ERR_TIMEOUT);
+            stop = 1;
+        }
+    }
+    return __shfl_sync(0xffffffffu, stop, 0) != 0;
+}
+
+// Totals over the C CTAs of QH of this warp's columns (warp + NW (q0 + q)) into
+// sd, their entries of row k into sr (shared memory, by column).  Every lane
+// polls its entries until all carry `tag` (the tags of a try are compared with
+// one OR per word, nothing else is done before they fit) and sums them in
+// order; false when the wait ran out.
+template <typename T, int QH, int NW, bool CL>
+__device__ __forceinline__ bool coop_collect(const unsigned long long *cols, int cmax, int C, int warp, int q0, int b,
+                                             unsigned tag, long long cap, int *err, T *sd, T *sr) {
     const int lane = threadIdx.x & 31;
-    constexpr int PER = LLType<T>::W == 1 ? 2 : 1;  // values per 16-byte load
-    long long t0 = 0;
-    for (int tries = 0;; ++tries) {
-        bool ok = true;
+    constexpr int W = LLType<T>::W, PER = W == 1 ? 2 : 1;  // entries per 16-byte load
+    const unsigned long long *base = cols + (size_t)(warp + NW * q0) * cmax * W + PER * W * lane;
+    const size_t step = (size_t)NW * cmax * W;
+    T sum[QH], row[QH];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) sum[q] = T(0);
-        for (int c = PER * lane; c < C; c += PER * 32) {
-            unsigned long long a[Q], bb[Q];
+    for (int q = 0; q < QH; ++q) sum[q] = row[q] = T(0);
+    for (int c0 = 0; c0 <= C; c0 += 32 * PER) {
+        const int c = c0 + PER * lane;
+        const unsigned my = c <= C ? 0xffffffffu : 0u, my1 = W == 2 || c + 1 <= C ? my : 0u;
+        unsigned long long x[QH], y[QH];
+        long long t0 = 0;
+        for (int tries = 0;; ++tries) {
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const int j = warp + kCoopWarps * q;
-                a[q] = bb[q] = (unsigned long long)tag << 32;
-                if (j < b) ll_get2(cols + ((size_t)j * cmax + c) * LLType<T>::W, a[q], bb[q]);
+            for (int q = 0; q < QH; ++q) {
+                x[q] = y[q] = (unsigned long long)tag << 32;
+                if (warp + NW * (q0 + q) < b && c <= C) ll_get2<CL>(base + q * step + (size_t)c0 * W, x[q], y[q]);
             }
+            unsigned bad = 0;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                if constexpr (sizeof(T) == 4) {
-                    const bool two = c + 1 < C;
-                    ok = ok && ll_is(a[q], tag) && (!two || ll_is(bb[q], tag));
-                    sum[q] += __uint_as_float((unsigned)a[q]);
-                    if (two) sum[q] += __uint_as_float((unsigned)bb[q]);
-                } else {
-                    ok = ok && ll_is(a[q], tag) && ll_is(bb[q], tag);
-                    sum[q] += __hiloint2double((int)(unsigned)bb[q], (int)(unsigned)a[q]);
-                }
+            for (int q = 0; q < QH; ++q) bad |= (((unsigned)(x[q] >> 32) ^ tag) & my) | (((unsigned)(y[q] >> 32) ^ tag) & my1);
+            if (__all_sync(0xffffffffu, bad == 0)) break;
+            if (coop_give_up(tries, t0, cap, err)) return false;
+        }
+#pragma unroll
+        for (int q = 0; q < QH; ++q) {
+            if constexpr (W == 1) {
+                const float v0 = __uint_as_float((unsigned)x[q]), v1 = __uint_as_float((unsigned)y[q]);
+                sum[q] += c < C ? v0 : 0.f;
+                sum[q] += c + 1 < C ? v1 : 0.f;
+                row[q] = c == C ? v0 : (c + 1 == C ? v1 : row[q]);
+            } else {
+                const double v = __hiloint2double((int)(unsigned)y[q], (int)(unsigned)x[q]);
+                sum[q] += c < C ? v : 0.0;
+                row[q] = c == C ? v : row[q];
             }
         }
-        if (__all_sync(0xffffffffu, ok)) break;
-        if (tries == 0) t0 = clock64();
-        int stop = 0;
-        if (lane == 0) {
-            if ((tries & 31) == 31 && *(volatile int *)err != 0) stop = 1;
-            if (wait_expired(t0, cap)) {
-                latch_error(err, SEV_ERR_TIMEOUT);
-                stop = 1;
-            }
-        }
-        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
     }
-    // totals in every lane
+    const T s = warp_sums_t<T, QH>(sum);
+    const int j = warp + NW * (q0 + lane / (32 / QH));
+    if ((lane & (32 / QH - 1)) == 0 && j < b) sd[j] = s;
+    if (lane == (C / PER) % 32) {
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        if (warp + kCoopWarps * q >= b) sum[q] = T(0);
+        for (int q = 0; q < QH; ++q)
+            if (warp + NW * (q0 + q) < b) sr[warp + NW * (q0 + q)] = row[q];
     }
-    const T s = warp_sums_t<T, Q>(sum);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) sum[q] = __shfl_sync(0xffffffffu, s, q * (32 / Q));
     return true;
 }
 
-// A pair of words per entry i < cnt (lane takes i = lane, lane + 32, ...),
-// polled until tagged; f(i, word0, word1) is called once per entry at the end.
-template <typename F>
-__device__ __forceinline__ bool coop_poll_pairs(const unsigned long long *p, int cnt, unsigned tag, long long cap,
-                                                int *err, F f) {
+// A pair of words per entry i < cnt (lane takes i = lane, lane + 32, ...) and
+// (ENTRY) one entry of the columns for lane 0, polled until tagged.  f(i ==
+// lane, word0, word1) is called for every entry, in order, of the last try.
+template <typename T, bool CL, bool ENTRY, typename F>
+__device__ __forceinline__ bool coop_poll_pairs(const unsigned long long *p, int cnt, const unsigned long long *entry,
+                                                T &val, unsigned tag, long long cap, int *err, F f) {
     const int lane = threadIdx.x & 31;
     long long t0 = 0;
     for (int tries = 0;; ++tries) {
         bool ok = true;
+        if (ENTRY && lane == 0) {
+            // (the 16-byte aligned pair that holds the entry)
+            const bool odd = ((uintptr_t)entry & 8) != 0;
+            unsigned long long a, b;
+            ll_get2<CL>(entry - (odd ? 1 : 0), a, b);
+            if constexpr (sizeof(T) == 4) {
+                ok = ll_is(odd ? b : a, tag);
+                val = __uint_as_float((unsigned)(odd ? b : a));
+            } else {
+                ok = ll_is(a, tag) && ll_is(b, tag);
+                val = __hiloint2double((int)(unsigned)b, (int)(unsigned)a);
+            }
+        }
         for (int i = lane; i < cnt; i += 32) {
             unsigned long long a, b;
-            ll_get2(p + 2 * (size_t)i, a, b);
+            ll_get2<CL>(p + 2 * (size_t)i, a, b);
             ok = ok && ll_is(a, tag) && ll_is(b, tag);
             f(i == lane, (unsigned)a, (unsigned)b);
         }
         if (__all_sync(0xffffffffu, ok)) return true;
-        if (tries == 0) t0 = clock64();
-        int stop = 0;
-        if (lane == 0) {
-            if ((tries & 31) == 31 && *(volatile int *)err != 0) stop = 1;
-            if (wait_expired(t0, cap)) {
-                latch_error(err, SEV_ERR_TIMEOUT);
-                stop = 1;
-            }
-        }
-        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+        if (coop_give_up(tries, t0, cap, err)) return false;
     }
 }
 
 template <typename T, int RT>
 struct CoopSmem {
     T xs[2][32 * RT];          // scale times column k below row k
+    T sd[kCoopMaxB], sr[kCoopMaxB];  // x^T a_j and row k of the column being formed
     T gs[kCoopMaxB];           // G(j, k), j < k (last CTA)
-    T part[kCoopWarps * 32];   // partial sums of a column of T (last CTA)
+    T part[16 * 32];           // partial sums of a column of T (last CTA)
     T tau[kCoopMaxB];
     T sc[4];                   // tau, beta, 1 / (scale (alpha - beta)) of the column; the panel's scale
     int abort;
@@ -206,10 +258,10 @@ struct CoopSmem {
 // Column kc of T by the last CTA, in two halves with a barrier between them:
 // T(a, kc) = -tau sum_{q = a}^{kc - 1} T(a, q) G(q, kc) (forward, column-wise:
 // Q = I - U T U^T).  Ts: column-major, ld b, zero below the diagonal.
-template <typename T>
+template <typename T, int NW>
 __device__ __forceinline__ void coop_t_partial(int b, int kc, const T *Ts, const T *gs, T *part) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nrg = (b + 31) / 32, nsl = kCoopWarps / nrg;
+    const int nrg = (b + 31) / 32, nsl = NW / nrg;
     const int a = 32 * (warp % nrg) + lane, sl = warp / nrg;
     if (sl >= nsl) return;
     T s0 = T(0);
@@ -217,10 +269,10 @@ __device__ __forceinline__ void coop_t_partial(int b, int kc, const T *Ts, const
         for (int q = sl; q < kc; q += nsl) s0 = fmat(Ts[(size_t)q * b + a], gs[q], s0);
     if (a < b) part[sl * b + a] = s0;
 }
-template <typename T>
+template <typename T, int NW>
 __device__ __forceinline__ void coop_t_column(int b, int kc, T *Ts, const T *tau, const T *part) {
     const int lane = threadIdx.x & 31;
-    const int nsl = kCoopWarps / ((b + 31) / 32);
+    const int nsl = NW / ((b + 31) / 32);
     const T tk = tau[kc];
     for (int a = lane; a <= kc; a += 32) {
         T s = T(0);
@@ -234,8 +286,8 @@ __device__ __forceinline__ void coop_t_column(int b, int kc, T *Ts, const T *tau
 // lower trapezoidal), Tm (b x b) the compact-WY factor, and P the band block
 // (R over zeros).  comm: exchange words; tags tag0 + 1 .. tag0 + b + 1 are
 // unused so far in it.
-template <typename T, int RT, int Q>
-__global__ void __launch_bounds__(kCoopThreads, 1)
+template <typename T, int RT, int Q, int NW, bool CL>
+__global__ void __launch_bounds__((NW + 1) * 32, 1)
     panel_coop_kernel(T *__restrict__ P, int ldp, int N, int b, T *__restrict__ U, T *__restrict__ Tm,
                       unsigned long long *comm, int cmax, unsigned tag0, int *err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -249,15 +301,39 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
     const int nref = min(b, N - 1);
     const long long cap = wait_cap(err);
     using Comm = CoopComm<T>;
+    if constexpr (CL) {
+        // the exchange buffer of this CTA behind T; no tag may be found in what
+        // the memory held before, nor a word arrive before that is so
+        comm = reinterpret_cast<unsigned long long *>(Ts + (size_t)((b * b + 3) & ~3));
+        const int nw = (int)Comm::words(b, cmax);
+        for (int i = threadIdx.x; i < nw; i += blockDim.x) comm[i] = 0;
+        coop_cluster_sync();
+    }
     unsigned long long *const amx = comm + 2 * Comm::set_words(b, cmax);
+    // A column warp's lanes lane / (32 / Q) = q serve column q, the peers dealt to
+    // them; the scalar warp's lanes one peer each.  (Global memory: one place.)
+    constexpr int LPQ = 32 / Q, NP = CL ? (16 + LPQ - 1) / LPQ : 1;
+    unsigned peer[NP];
+    int npeer = 0;
+    if constexpr (CL) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const int to = warp < NW ? (lane & (LPQ - 1)) + LPQ * i : lane;
+            peer[i] = to < C ? ll_peer(comm, to) : 0;
+            npeer += to < C && (warp < NW || i == 0);
+        }
+    } else {
+        peer[0] = 0;
+        npeer = (warp < NW ? (lane & (LPQ - 1)) : lane) == 0;
+    }
 
     T a[Q][RT];
-    if (warp < kCoopWarps) {
+    if (warp < NW) {
 #pragma unroll
         for (int q = 0; q < Q; ++q)
 #pragma unroll
             for (int t = 0; t < RT; ++t) {
-                const int j = warp + kCoopWarps * q, r = lane + 32 * t;
+                const int j = warp + NW * q, r = lane + 32 * t;
                 a[q][t] = (j < b && r < rows) ? P[(size_t)(row0 + r) + (size_t)j * ldp] : T(0);
             }
     }
@@ -268,7 +344,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
     // square or product that matters over- or underflows.
     {
         double m = 0.0;
-        if (warp < kCoopWarps) {
+        if (warp < NW) {
             T mt = T(0);
 #pragma unroll
             for (int q = 0; q < Q; ++q)
@@ -279,12 +355,14 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
             if (lane == 0) S.part[warp] = mt;
         }
         __syncthreads();
-        if (warp == kCoopWarps) {
-            m = lane < kCoopWarps ? (double)S.part[lane] : 0.0;
+        if (warp == NW) {
+            m = lane < NW ? (double)S.part[lane] : 0.0;
             m = warp_max(m);
-            if (lane == 0) ll_put_val(amx + 2 * c, m, tag0 + 1);
+            if (npeer) ll_put_val<CL>(comm, peer[0], (amx - comm) + 2 * c, m, tag0 + 1);
             double g = 0.0;
-            const bool got = coop_poll_pairs(amx, C, tag0 + 1, cap, err, [&](bool first, unsigned lo, unsigned hi) {
+            T none = T(0);
+            const bool got = coop_poll_pairs<T, CL, false>(amx, C, nullptr, none, tag0 + 1, cap, err,
+                                                                [&](bool first, unsigned lo, unsigned hi) {
                 const double v = __hiloint2double((int)hi, (int)lo);
                 g = first ? v : fmax(g, v);
             });
@@ -300,7 +378,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         }
     }
     __syncthreads();
-    const T scale = S.sc[3];
+    const T scale = S.sc[3], unscale = T(1) / scale;
     bool alive = !S.abort;
     if (warp == 0) {
 #pragma unroll
@@ -310,27 +388,27 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
 
     for (int k = 0; k < nref && alive; ++k) {
         const unsigned tag = tag0 + 2 + k;
-        unsigned long long *const set = comm + (k & 1) * Comm::set_words(b, cmax);
-        unsigned long long *const roww = set + Comm::col_words(b, cmax);
-        unsigned long long *const ssqw = roww + Comm::row_words(b);
+        const size_t set = (k & 1) * Comm::set_words(b, cmax), ssqw = set + Comm::col_words(b, cmax);
         const T *xk = S.xs[k & 1];
-        T dsum[Q], rk[Q];
-        if (warp < kCoopWarps) {
-            T xr[RT];
-            // ---- this CTA's shares of x^T a_j, and row k from the CTA that holds it
-#pragma unroll
-            for (int t = 0; t < RT; ++t) xr[t] = xk[lane + 32 * t];
-            if (c == 0 && lane == (k & 31)) {
+        if (warp < NW) {
+            // ---- row k from the CTA that holds it, this CTA's shares of x^T a_j
+            const int jq = warp + NW * (lane / LPQ);  // this lane's column to send
+            if (c == 0) {
+                T v = T(0);
 #pragma unroll
                 for (int q = 0; q < Q; ++q) {
-                    const int j = warp + kCoopWarps * q;
-                    if (j < b) {
-                        const T v = rsel<RT>(a[q], k >> 5);
-                        ll_put_val(roww + 2 * j, v, tag);
-                        if constexpr (sizeof(T) == 4) ll_put(roww + 2 * j + 1, 0u, tag);
-                    }
+                    const T rv = __shfl_sync(0xffffffffu, rsel<RT>(a[q], k >> 5), k & 31);
+                    v = lane / LPQ == q ? rv : v;
                 }
+                if (jq < b)
+#pragma unroll
+                    for (int i = 0; i < NP; ++i)
+                        if (i < npeer)
+                            ll_put_val<CL>(comm, peer[i], set + ((size_t)jq * cmax + C) * LLType<T>::W, v, tag);
             }
+            T xr[RT];
+#pragma unroll
+            for (int t = 0; t < RT; ++t) xr[t] = xk[lane + 32 * t];
             T d[Q];
             if constexpr (sizeof(T) == 4) {
                 float2 dd[Q / 2];
@@ -356,34 +434,23 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
                     for (int q = 0; q < Q; ++q) d[q] = fmat(xr[t], a[q][t], d[q]);
             }
             const T mine = warp_sums_t<T, Q>(d);
-            if ((lane & (32 / Q - 1)) == 0) {
-                const int j = warp + kCoopWarps * (lane / (32 / Q));
-                if (j < b) ll_put_val(set + ((size_t)j * cmax + c) * LLType<T>::W, mine, tag);
-            }
-            if (lastc && k >= 1) coop_t_partial<T>(b, k - 1, Ts, S.gs, S.part);
-            bool ok = coop_collect<T, Q>(set, cmax, C, warp, b, tag, cap, err, dsum);
-            // row k at this warp's columns
-            T rv = T(0);
-            if (ok) {
-                long long t0 = clock64();
-                for (;;) {
-                    unsigned long long w0 = (unsigned long long)tag << 32, w1 = w0;
-                    const int j = warp + kCoopWarps * lane;
-                    if (lane < Q && j < b) ll_get2(roww + 2 * j, w0, w1);
-                    if constexpr (sizeof(T) == 4)
-                        rv = __uint_as_float((unsigned)w0);
-                    else
-                        rv = __hiloint2double((int)(unsigned)w1, (int)(unsigned)w0);
-                    if (__all_sync(0xffffffffu, ll_is(w0, tag) && ll_is(w1, tag))) break;
-                    if (__any_sync(0xffffffffu, wait_expired(t0, cap))) {
-                        if (lane == 0) latch_error(err, SEV_ERR_TIMEOUT);
-                        ok = false;
-                        break;
-                    }
+            if (jq < b)
+#pragma unroll
+                for (int i = 0; i < NP; ++i)
+                    if (i < npeer) ll_put_val<CL>(comm, peer[i], set + ((size_t)jq * cmax + c) * LLType<T>::W, mine, tag);
+            if (lastc && k >= 1) coop_t_partial<T, NW>(b, k - 1, Ts, S.gs, S.part);
+            constexpr int QH = Q > 4 && NW == 16 ? 4 : Q;  // (16 warps: 96 registers a thread)
+            if (!CL) {
+                // the slowest share is ~1.5K cycles away: a first look that fails only
+                // loads the L2 (n = 8192 20.5 -> 19.3 ms of panels per reduction)
+                const long long ts = clock64();
+                while (clock64() - ts < 400) {
                 }
             }
+            bool ok = true;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) rk[q] = __shfl_sync(0xffffffffu, rv, q);
+            for (int q0 = 0; q0 < Q; q0 += QH)
+                ok = ok && coop_collect<T, QH, NW, CL>(comm + set, cmax, C, warp, q0, b, tag, cap, err, S.sd, S.sr);
             if (!ok && lane == 0) S.abort = 1;
         } else {
             // ---- the scalar warp: x^T x over all CTAs, then tau, beta, 1 / (alpha - beta)
@@ -396,29 +463,26 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
                     f2_add_sq(p1, (float)xk[lane + 32 * t + 32]);
                 }
                 const F2 mine = warp_sum_f2(f2_add(p0, p1));
-                if (lane == 0) {
-                    ll_put(ssqw + 2 * c, __float_as_uint(mine.hi), tag);
-                    ll_put(ssqw + 2 * c + 1, __float_as_uint(mine.lo), tag);
+                if (npeer) {
+                    ll_put<CL>(comm, peer[0], ssqw + 2 * c, __float_as_uint(mine.hi), tag);
+                    ll_put<CL>(comm, peer[0], ssqw + 2 * c + 1, __float_as_uint(mine.lo), tag);
                 }
                 F2 acc{0.f, 0.f};
-                ok = coop_poll_pairs(ssqw, C, tag, cap, err, [&](bool first, unsigned hi, unsigned lo) {
-                    const F2 v{__uint_as_float(hi), __uint_as_float(lo)};
-                    acc = first ? v : f2_add(acc, v);
-                });
-                acc = warp_sum_f2(acc);
                 float alpha = 0.f;
-                if (ok)
-                    ok = coop_poll_pairs(roww + 2 * k, 1, tag, cap, err,
-                                         [&](bool, unsigned v, unsigned) { alpha = __uint_as_float(v); });
-                alpha = __shfl_sync(0xffffffffu, alpha, 0);
-                alpha *= (float)scale;
+                ok = coop_poll_pairs<float, CL, true>(comm + ssqw, C, comm + set + (size_t)k * cmax + C, alpha, tag, cap,
+                                                      err, [&](bool first, unsigned hi, unsigned lo) {
+                                                          const F2 v{__uint_as_float(hi), __uint_as_float(lo)};
+                                                          acc = first ? v : f2_add(acc, v);
+                                                      });
+                alpha = __shfl_sync(0xffffffffu, alpha, 0) * (float)scale;
+                acc = warp_sum_f2(acc);
                 float tau = 0.f, beta = 0.f, inv = 0.f;
                 // a column 1e-16 times smaller than the panel's largest entry is a
                 // zero column (its pair-float square would lose digits to underflow)
                 if (fmaf(alpha, alpha, acc.hi) >= 1e-32f) house_scalars_f2(alpha, acc, &tau, &beta, &inv);
                 if (lane == 0) {
                     S.sc[0] = (T)tau;
-                    S.sc[1] = (T)(beta / (float)scale);
+                    S.sc[1] = (T)(beta * (float)unscale);
                     S.sc[2] = (T)inv;
                     S.tau[k] = (T)tau;
                 }
@@ -430,18 +494,14 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
                     s = fma(x, x, s);
                 }
                 s = warp_sum(s);
-                if (lane == 0) ll_put_val(ssqw + 2 * c, s, tag);
-                double acc = 0.0;
-                ok = coop_poll_pairs(ssqw, C, tag, cap, err, [&](bool first, unsigned lo, unsigned hi) {
-                    const double v = __hiloint2double((int)hi, (int)lo);
-                    acc = first ? v : acc + v;
-                });
+                if (npeer) ll_put_val<CL>(comm, peer[0], ssqw + 2 * c, s, tag);
+                double acc = 0.0, alpha = 0.0;
+                ok = coop_poll_pairs<double, CL, true>(comm + ssqw, C, comm + set + ((size_t)k * cmax + C) * 2, alpha, tag,
+                                                       cap, err, [&](bool first, unsigned lo, unsigned hi) {
+                                                           const double v = __hiloint2double((int)hi, (int)lo);
+                                                           acc = first ? v : acc + v;
+                                                       });
                 acc = warp_sum(acc);
-                double alpha = 0.0;
-                if (ok)
-                    ok = coop_poll_pairs(roww + 2 * k, 1, tag, cap, err, [&](bool, unsigned lo, unsigned hi) {
-                        alpha = __hiloint2double((int)hi, (int)lo);
-                    });
                 alpha = __shfl_sync(0xffffffffu, alpha, 0);
                 const double as = alpha * (double)scale;
                 double tau = 0.0, beta = 0.0, inv = 0.0;
@@ -450,7 +510,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
                 if (fma(as, as, acc) >= 1e-280) house_scalars(as, acc, &tau, &beta, &inv);
                 if (lane == 0) {
                     S.sc[0] = (T)tau;
-                    S.sc[1] = (T)(beta / (double)scale);
+                    S.sc[1] = (T)(beta * (double)unscale);
                     S.sc[2] = (T)inv;
                     S.tau[k] = (T)tau;
                 }
@@ -459,7 +519,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         }
         __syncthreads();
         alive = !S.abort;
-        if (warp < kCoopWarps) {
+        if (warp < NW) {
             // ---- a_j -= tau (v^T a_j) v for j > k; column k becomes (beta, v); G(j, k) for j < k
             const T tau = S.sc[0], beta = S.sc[1], inv = S.sc[2];
             T v[RT];
@@ -468,18 +528,24 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
             T ms[Q];
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
-                const int j = warp + kCoopWarps * q;
-                const T s = fmat(inv, dsum[q], rk[q]);
+                const int j = warp + NW * q;
+                const T s = fmat(inv, S.sd[j], S.sr[j]);
                 ms[q] = (j > k && j < b) ? -tau * s : T(0);
                 if (lastc && lane == 0 && j < k) S.gs[j] = s;
-                // (tau = 0: the column is zero below row k, or far below the
+            }
+            if (warp == k % NW) {
+                // column k itself.  (tau = 0: it is zero below row k, or far below the
                 // rounding errors of the panel's other entries and dropped here)
-                const bool own = j == k;
+                const unsigned pick = 1u << (k / NW);
 #pragma unroll
-                for (int t = 0; t < RT; ++t) {
-                    const int g = row0 + lane + 32 * t;
-                    a[q][t] = own && g > k ? v[t] : (own && g == k && tau != T(0) ? beta : a[q][t]);
-                }
+                for (int q = 0; q < Q; ++q)
+                    if ((pick >> q) & 1) {
+#pragma unroll
+                        for (int t = 0; t < RT; ++t) {
+                            const int g = row0 + lane + 32 * t;
+                            a[q][t] = g > k ? v[t] : (g == k && tau != T(0) ? beta : a[q][t]);
+                        }
+                    }
             }
             if (tau != T(0)) {
                 if constexpr (sizeof(T) == 4) {
@@ -502,39 +568,44 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
                 }
             }
             const int k1 = k + 1;
-            if (k1 < nref && k1 % kCoopWarps == warp) {
+            if (k1 < nref && k1 % NW == warp) {
                 T *xn = S.xs[k1 & 1];
-                const unsigned pick = 1u << (k1 / kCoopWarps);
+                const unsigned pick = 1u << (k1 / NW);
 #pragma unroll
-                for (int t = 0; t < RT; ++t) {
-                    T x = a[0][t];
+                for (int q = 0; q < Q; ++q)
+                    if ((pick >> q) & 1) {
 #pragma unroll
-                    for (int q = 1; q < Q; ++q) x = (pick >> q) & 1 ? a[q][t] : x;
-                    xn[lane + 32 * t] = row0 + lane + 32 * t > k1 ? x * scale : T(0);
-                }
+                        for (int t = 0; t < RT; ++t)
+                            xn[lane + 32 * t] = row0 + lane + 32 * t > k1 ? a[q][t] * scale : T(0);
+                    }
             }
         } else if (lastc && k >= 1) {
-            coop_t_column<T>(b, k - 1, Ts, S.tau, S.part);
+            coop_t_column<T, NW>(b, k - 1, Ts, S.tau, S.part);
         }
         __syncthreads();
+    }
+    // no CTA leaves while a peer may still store into its shared memory
+    if constexpr (CL) {
+        __syncwarp();
+        coop_cluster_sync();
     }
     if (!alive) return;  // the error is latched; nothing was written
     // ---- the last column of T, then the results
     if (lastc) {
         if (nref > 0) {
-            if (warp < kCoopWarps) coop_t_partial<T>(b, nref - 1, Ts, S.gs, S.part);
+            if (warp < NW) coop_t_partial<T, NW>(b, nref - 1, Ts, S.gs, S.part);
             __syncthreads();
-            if (warp == kCoopWarps) coop_t_column<T>(b, nref - 1, Ts, S.tau, S.part);
+            if (warp == NW) coop_t_column<T, NW>(b, nref - 1, Ts, S.tau, S.part);
         }
         __syncthreads();
         for (int i = threadIdx.x; i < b * b; i += blockDim.x) Tm[i] = Ts[i];
     }
-    if (warp < kCoopWarps) {
+    if (warp < NW) {
 #pragma unroll
         for (int q = 0; q < Q; ++q)
 #pragma unroll
             for (int t = 0; t < RT; ++t) {
-                const int j = warp + kCoopWarps * q, r = lane + 32 * t, g = row0 + r;
+                const int j = warp + NW * q, r = lane + 32 * t, g = row0 + r;
                 if (j >= b || r >= rows) continue;
                 T v = T(0);
                 if (j < nref) v = g < j ? T(0) : (g == j ? T(1) : a[q][t]);
@@ -545,17 +616,18 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
 }
 
 // -------------------------------------------------------------------- host
-// CTAs the exchange buffer has room for (one per SM, even).
-static int coop_cmax(const sev_ctx *h) { return (h->sm_count + 1) / 2 * 2; }
+// CTAs the exchange buffer in global memory has room for (one per SM, even).
+static int coop_cmax(const sev_ctx *h) { return (h->sm_count + 2) / 2 * 2; }
+constexpr int kCoopClMax = 16;  // CTAs of the largest cluster
 
 template <typename T>
 size_t panel_coop_words(const sev_ctx *h, int b) {
     return CoopComm<T>::words(b, coop_cmax(h));
 }
 
-// Rows per CTA (in units of 32): the fewest for which the CTAs stay a
-// moderate number -- more rows mean more arithmetic per CTA and column, more
-// CTAs mean more shares to read.  0: the panel does not fit the GPU.
+// Rows per CTA (in units of 32) on the whole GPU: the fewest for which the CTAs
+// stay a moderate number -- more rows mean more arithmetic per CTA and column,
+// more CTAs mean more shares to read.  0: the panel does not fit the GPU.
 template <typename T>
 static int coop_rt(const sev_ctx *h, int N) {
     const int sizes[3] = {2, 4, 8}, room[3] = {sizeof(T) == 4 ? 0 : 96, sizeof(T) == 4 ? 32 : 128, h->sm_count};
@@ -566,44 +638,102 @@ static int coop_rt(const sev_ctx *h, int N) {
     return 0;
 }
 
+// The same on one cluster, whose CTAs exchange through shared memory (N = 2048,
+// b = 64: 129 us a panel against 165 through L2); 0: not there.  FP64 keeps few rows per
+// CTA (its FP64 pipes bound the column, not the exchange).
+template <typename T>
+static int coop_cl_rt(int N) {
+    if (sizeof(T) == 8) return N <= 64 * kCoopClMax ? 2 : 0;
+    return N <= 128 * 8 ? 4 : (N <= 256 * kCoopClMax ? 8 : 0);
+}
+
 template <typename T>
 int panel_coop_supported(const sev_ctx *h, int N, int b) {
     if (h->leaf_rows_override > 0) return 0;  // the caller asked for a tree of that leaf size
     return b >= 1 && b <= (sizeof(T) == 4 ? 128 : 64) && coop_rt<T>(h, N) > 0;
 }
 
-template <typename T, int RT, int Q>
+template <typename T, int RT>
+static size_t coop_smem(int b) {
+    return ((sizeof(CoopSmem<T, RT>) + 15) & ~(size_t)15) + sizeof(T) * (size_t)((b * b + 3) & ~3);
+}
+
+template <typename T, int RT, int Q, int NW>
 static int panel_coop_run(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
-    const size_t smem = ((sizeof(CoopSmem<T, RT>) + 15) & ~(size_t)15) + sizeof(T) * (size_t)b * b;
-    auto kern = panel_coop_kernel<T, RT, Q>;
+    const size_t smem = coop_smem<T, RT>(b);
+    auto kern = panel_coop_kernel<T, RT, Q, NW, false>;
     SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int C = (N + 32 * RT - 1) / (32 * RT);
     int cmax = coop_cmax(h);
     void *args[] = {(void *)&P,    (void *)&lda,  (void *)&N,    (void *)&b,   (void *)&U,
                     (void *)&Tm,   (void *)&comm, (void *)&cmax, (void *)&tag0, (void *)&h->d_err};
     timing_begin(h, K_PANEL_COOP);
-    SEV_CUDA(cudaLaunchCooperativeKernel((const void *)kern, C, kCoopThreads, args, smem, h->stream));
+    SEV_CUDA(cudaLaunchCooperativeKernel((const void *)kern, C, (NW + 1) * 32, args, smem, h->stream));
     timing_end(h, K_PANEL_COOP);
     return SEV_OK;
 }
 
-template <typename T, int Q>
+// One cluster of C CTAs; SEV_ERR_UNSUPPORTED where the GPU cannot hold it.
+template <typename T, int RT, int Q, int NW>
+static int panel_coop_run_cl(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm) {
+    const int C = (N + 32 * RT - 1) / (32 * RT), cmax = (C + 2) / 2 * 2;
+    const size_t smem = coop_smem<T, RT>(b) + 8 * CoopComm<T>::words(b, cmax);
+    if (smem > h->smem_optin) return SEV_ERR_UNSUPPORTED;
+    auto kern = panel_coop_kernel<T, RT, Q, NW, true>;
+    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3((NW + 1) * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (C > 8) {
+        // clusters of more than 8 CTAs depend on the GPU's layout: asked once per handle and size
+        signed char &ok = h->cluster_ok[sizeof(T) == 8][C];
+        if (ok == 0) {
+            int fit = 0;
+            ok = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit > 0 ? 1 : -1;
+            cudaGetLastError();
+        }
+        if (ok < 0) return SEV_ERR_UNSUPPORTED;
+    }
+    timing_begin(h, K_PANEL_COOP);
+    SEV_CUDA(cudaLaunchKernelEx(&cfg, kern, P, lda, N, b, U, Tm, (unsigned long long *)nullptr, cmax, 0u, h->d_err));
+    timing_end(h, K_PANEL_COOP);
+    return SEV_OK;
+}
+
+template <typename T, int Q, int NW>
 static int panel_coop_rt(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
+    int rc = SEV_ERR_UNSUPPORTED;
+    if constexpr (sizeof(T) == 8) {
+        if (coop_cl_rt<T>(N) == 2) rc = panel_coop_run_cl<T, 2, Q, NW>(h, N, b, P, lda, U, Tm);
+    } else {
+        if (coop_cl_rt<T>(N) == 4) rc = panel_coop_run_cl<T, 4, Q, NW>(h, N, b, P, lda, U, Tm);
+        if (coop_cl_rt<T>(N) == 8) rc = panel_coop_run_cl<T, 8, Q, NW>(h, N, b, P, lda, U, Tm);
+    }
+    if (rc != SEV_ERR_UNSUPPORTED) return rc;
     switch (coop_rt<T>(h, N)) {
         case 2:
-            if constexpr (sizeof(T) == 8) return panel_coop_run<T, 2, Q>(h, N, b, P, lda, U, Tm, comm, tag0);
+            if constexpr (sizeof(T) == 8) return panel_coop_run<T, 2, Q, NW>(h, N, b, P, lda, U, Tm, comm, tag0);
             return SEV_ERR_UNSUPPORTED;
-        case 4: return panel_coop_run<T, 4, Q>(h, N, b, P, lda, U, Tm, comm, tag0);
-        case 8: return panel_coop_run<T, 8, Q>(h, N, b, P, lda, U, Tm, comm, tag0);
+        case 4: return panel_coop_run<T, 4, Q, NW>(h, N, b, P, lda, U, Tm, comm, tag0);
+        case 8: return panel_coop_run<T, 8, Q, NW>(h, N, b, P, lda, U, Tm, comm, tag0);
         default: return SEV_ERR_UNSUPPORTED;
     }
 }
 
 template <typename T>
 int panel_coop_factor(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
-    if (b <= 32) return panel_coop_rt<T, 2>(h, N, b, P, lda, U, Tm, comm, tag0);
-    if (b <= 64) return panel_coop_rt<T, 4>(h, N, b, P, lda, U, Tm, comm, tag0);
-    if constexpr (sizeof(T) == 4) return panel_coop_rt<T, 8>(h, N, b, P, lda, U, Tm, comm, tag0);
+    if (b <= 32) return panel_coop_rt<T, 4, 8>(h, N, b, P, lda, U, Tm, comm, tag0);
+    if (b <= 64) return panel_coop_rt<T, 8, 8>(h, N, b, P, lda, U, Tm, comm, tag0);
+    if constexpr (sizeof(T) == 4) return panel_coop_rt<T, 8, 16>(h, N, b, P, lda, U, Tm, comm, tag0);
     return SEV_ERR_UNSUPPORTED;
 }
 
