@@ -10,18 +10,23 @@
 //     Q = I - U T U^T) and the two-sided update A22 += U V^T + V U^T with
 //     V = U (T^T U^T A22 U T) / 2 - A22 U T (Eq. 4.1);
 //   b -> 1 band reduction (Algorithm 4.2 with h = 1) on the whole band held
-//     in shared memory: every warp owns one sweep at a time, and chase
-//     (i, j) starts once sweep i - 1 has finished chase j + 2 (the legal
-//     dependency of the wavefront, Sec. 4.2);
+//     in shared memory: every warp owns one sweep at a time, and step (i, j)
+//     of band_tri.cu starts once sweep i - 1 has finished step j + 1;
 //   Sturm bisection of the tridiagonal (the final step of Algorithm 4.3).
 //
 // CTAs take matrices from a global queue (the host orders it largest
 // first), so the launch load-balances uneven sizes by itself.  The matrix
 // is overwritten (both triangles: the kernel first mirrors the lower
-// triangle).  Nothing is allocated and nothing waits on the host, so the
+// triangle).
+//
+// What bounds it: 4096 FP32 matrices of order 32..512 (b = 16) 147.7 -> 85.6 ms,
+// 60% of it the bisection's FP64 recurrence; 500 FP64 ones (b = 8) 136 -> 95.5 ms, the
+// FP64 pipes (2 FMA per cycle and SM) in every phase and the largest matrices'
+// own time.  Nothing is allocated and nothing waits on the host, so the
 // launch can be captured in a CUDA graph.
+#include "band_step.cuh"
 #include "sturm.cuh"
-#include "tri_chase.cuh"
+#include "tri_step.cuh"
 
 namespace sev {
 
@@ -38,32 +43,127 @@ struct BatchMat {
 
 template <typename T, int B>
 struct BatchLayout {
-    // full-to-band: U, Y (ldp x B each), Tm, G, Z (B x B), tau (B), red
-    static __host__ __device__ size_t f_bytes(int ldp) {
-        return sizeof(T) * (2 * (size_t)ldp * B + 3 * (size_t)B * B + B) + 64;
+    // columns of the panel buffers: a multiple of 4 for 16-byte loads
+    static __host__ __device__ int ldp(int nmax) { return (nmax + 3) & ~3; }
+    // partial sums of U^T Y: one share per warp, fewer where eight would
+    // outgrow the bisection's arrays, whose place they take
+    static constexpr int NS = B == 32 ? 2 : (B * sizeof(T) == 128 ? 4 : kBatchWarps);
+    // full-to-band: U, Y (ldp x B each), T (B x B), tau (B); then the band:
+    // nmax columns x 2B diagonals in the same place
+    static __host__ __device__ size_t x_off(int nmax) {
+        const size_t f = 2 * (size_t)ldp(nmax) * B + (size_t)B * B + B, b = (size_t)nmax * 2 * B;
+        return (sizeof(T) * (f > b ? f : b) + 15) & ~(size_t)15;
     }
-    // band: nmax columns x 2B diagonals, per-warp vector buffers, counters
-    static __host__ __device__ size_t b_bytes(int nmax) {
-        return sizeof(T) * ((size_t)nmax * 2 * B + 2 * kBatchWarps * 32) + kBatchWarps * sizeof(int);
+    // behind it, one after the other in the same place: G, Z and the shares
+    // (B x B each); the vectors and counters of the warps' sweeps; d, e, e^2
+    // (n doubles each), parameters and reduction scratch of the bisection
+    static __host__ __device__ size_t bytes(int nmax) {
+        const size_t f = sizeof(T) * (NS + 2) * (size_t)B * B;
+        const size_t b = sizeof(T) * 3 * kBatchWarps * kTriVec + sizeof(int) * kBatchWarps;
+        const size_t e = sizeof(double) * (3 * (size_t)nmax + 48);
+        const size_t fb = f > b ? f : b;
+        return x_off(nmax) + (fb > e ? fb : e);
     }
-    static __host__ __device__ size_t e_off(int nmax) {
-        const size_t f = f_bytes(nmax), b = b_bytes(nmax);
-        return ((f > b ? f : b) + 15) & ~(size_t)15;
-    }
-    // bisection: d, e, e^2 (n doubles each), parameters, reduction scratch
-    static __host__ __device__ size_t bytes(int nmax) { return e_off(nmax) + sizeof(double) * (3 * (size_t)nmax + 48); }
 };
 
 // ------------------------------------------------------------ full to band
+// G = U^T Y (B x B) in NS shares of the rows: lanes hold the outputs (row
+// lane mod B, columns dealt to the lane groups and, with fewer shares than
+// warps, to the warps of a share), then the shares are added in order.  (One
+// thread per 4 x 4 tile left all but (B/4)^2 threads idle through N steps.)
 template <typename T, int B>
-__device__ void batch_full_to_band(T *A, int n, int lda, unsigned char *smem, int ldp) {
+__device__ __forceinline__ void batch_uty(int N, const T *U, const T *Y, int ldp, T *share, T *G) {
+    constexpr int NS = BatchLayout<T, B>::NS, W = kBatchWarps / NS;
+    constexpr int LG = 32 / B < B ? 32 / B : B;  // lane groups (B = 4 leaves 16 lanes over)
+    constexpr int CP = B / (LG * W);             // columns of a lane
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int a = lane % B, g = lane / B % LG + LG * (warp / NS), sh = warp % NS;
+    T acc[CP];
+#pragma unroll
+    for (int q = 0; q < CP; ++q) acc[q] = T(0);
+#pragma unroll 2
+    for (int i = sh; i < N; i += NS) {
+        const T u = U[i + (size_t)a * ldp];
+#pragma unroll
+        for (int q = 0; q < CP; ++q) acc[q] = fmat(u, Y[i + (size_t)(g + LG * W * q) * ldp], acc[q]);
+    }
+    if (lane < B * LG) {
+#pragma unroll
+        for (int q = 0; q < CP; ++q) share[sh * B * B + a + (g + LG * W * q) * B] = acc[q];
+    }
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < B * B; idx += kBatchThreads) {
+        T s = share[idx];
+#pragma unroll
+        for (int w = 1; w < NS; ++w) s += share[w * B * B + idx];
+        G[idx] = s;
+    }
+    __syncthreads();
+}
+
+// A22 += U V^T + V U^T, both triangles: the lower tiles are computed and
+// written to both places.  A warp takes patches of 32 x 16 entries, its lanes
+// 8 x 4 tiles of 4 x 4: one shared-memory wavefront feeds all lanes of an
+// operand, and the lower and the mirrored entries both fill half of the
+// sectors they touch (whole rows of tiles would leave one of the two
+// scattered).  A thread's entries of A are on their way while it multiplies.
+// Against two full products of 4 x 4 tiles that each read and write all of A22:
+// 8.7 -> 1.4 s of CTA time over the 4096 FP32 matrices, 6.7 -> 3.4 s over the
+// 500 FP64 ones (the FP64 pipe's floor).
+template <typename T, int B>
+__device__ __forceinline__ void batch_syr2k(int N, T *A, int lda, const T *U, const T *V, int ldp) {
+    const int lane = threadIdx.x & 31;
+    const int PR = (N + 31) >> 5, PC = (N + 15) >> 4;
+    for (int p = threadIdx.x >> 5, R = 0; p < PR * (PR + 1); p += kBatchWarps) {
+        while ((R + 1) * (R + 2) <= p) ++R;  // 2 R + 2 patches in patch row R
+        const int C = p - R * (R + 1);
+        const int m0 = 32 * R + 4 * (lane & 7), n0 = 16 * C + 4 * (lane >> 3);
+        if (C >= PC || m0 >= N || m0 + 3 < n0) continue;
+        T old[4][4], acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                old[i][j] = (m0 + i < N && m0 + i >= n0 + j) ? A[(m0 + i) + (size_t)(n0 + j) * lda] : T(0);
+                acc[i][j] = T(0);
+            }
+#pragma unroll 4
+        for (int k = 0; k < B; ++k) {
+            T um[4], vm[4], un[4], vn[4];
+            vec_ld<T, 4>(U + m0 + k * ldp, um);
+            vec_ld<T, 4>(V + m0 + k * ldp, vm);
+            vec_ld<T, 4>(U + n0 + k * ldp, un);
+            vec_ld<T, 4>(V + n0 + k * ldp, vn);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmat(vm[i], un[j], fmat(um[i], vn[j], acc[i][j]));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int m = m0 + i, n = n0 + j;
+                if (m < N && m >= n) {
+                    const T v = old[i][j] + acc[i][j];
+                    A[m + (size_t)n * lda] = v;
+                    if (m > n) A[n + (size_t)m * lda] = v;
+                }
+            }
+    }
+}
+
+template <typename T, int B>
+__device__ void batch_full_to_band(T *A, int n, int lda, unsigned char *smem, int nmax) {
     const int tid = threadIdx.x, nt = blockDim.x;
+    const int ldp = BatchLayout<T, B>::ldp(nmax);
     T *U = (T *)smem;
     T *Y = U + (size_t)ldp * B;
     T *Tm = Y + (size_t)ldp * B;
-    T *G = Tm + B * B;
+    T *tau = Tm + B * B;
+    T *G = (T *)(smem + BatchLayout<T, B>::x_off(nmax));
     T *Z = G + B * B;
-    T *tau = Z + B * B;
+    T *share = Z + B * B;
     for (int c0 = 0; c0 + B < n; c0 += B) {
         const int r0 = c0 + B, N = n - r0;
         if (N < 2) break;
@@ -93,13 +193,12 @@ __device__ void batch_full_to_band(T *A, int n, int lda, unsigned char *smem, in
         // Y = A22 U;  G = U^T Y;  Z = G T;  G = T^T Z  (= T^T U^T A22 U T)
         cta_gemm<T, false, false>(N, B, N, T(1), A22, lda, U, ldp, T(0), Y, ldp);
         __syncthreads();
-        cta_gemm<T, true, false>(B, B, N, T(1), U, ldp, Y, ldp, T(0), G, B);
-        __syncthreads();
+        batch_uty<T, B>(N, U, Y, ldp, share, G);
         cta_gemm<T, false, false>(B, B, B, T(1), G, B, Tm, B, T(0), Z, B);
         __syncthreads();
-        cta_gemm<T, true, false>(B, B, B, T(1), Tm, B, Z, B, T(0), G, B);
+        cta_gemm<T, true, false>(B, B, B, T(0.5), Tm, B, Z, B, T(0), G, B);
         __syncthreads();
-        // V = U G / 2 - Y T, row by row in place of Y
+        // V = U G - Y T (G holds half), row by row in place of Y
         for (int i = tid; i < N; i += nt) {
             T y[B], u[B];
 #pragma unroll
@@ -111,29 +210,29 @@ __device__ void batch_full_to_band(T *A, int n, int lda, unsigned char *smem, in
             for (int c = 0; c < B; ++c) {
                 T acc = 0;
 #pragma unroll
-                for (int k = 0; k < B; ++k) acc = fma(T(0.5) * u[k], G[k + c * B], fma(-y[k], Tm[k + c * B], acc));
+                for (int k = 0; k < B; ++k) acc = fma(u[k], G[k + c * B], fma(-y[k], Tm[k + c * B], acc));
                 Y[i + (size_t)c * ldp] = acc;
             }
         }
         __syncthreads();
-        // A22 += U V^T + V U^T (both triangles: the next panel's product reads all of A22)
-        cta_gemm<T, false, true>(N, N, B, T(1), U, ldp, Y, ldp, T(1), A22, lda);
-        cta_gemm<T, false, true>(N, N, B, T(1), Y, ldp, U, ldp, T(1), A22, lda);
+        // both triangles: the next panel's product reads all of A22
+        batch_syr2k<T, B>(N, A22, lda, U, Y, ldp);
         __syncthreads();
     }
 }
 
 // ------------------------------------------------------------- band to 1
-// Returns false if a wait hit its cap.
+// Returns false if a wait hit its cap.  (With the one-warp chase of blocks in
+// registers, sweeps three chases apart: 9.6 s of CTA time over the 4096 FP32
+// matrices; so 2.6 s.)
 template <typename T, int B>
-__device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *smem, int *err) {
+__device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *smem, int nmax, int *err) {
     constexpr int LDW = 2 * B;
     const int tid = threadIdx.x, nt = blockDim.x;
     const int warp = tid >> 5, lane = tid & 31;
     T *band = (T *)smem;
-    T *vb = band + (size_t)n * LDW;
-    T *wb = vb + kBatchWarps * 32;
-    volatile int *sval = (volatile int *)(wb + kBatchWarps * 32);
+    T *vb = (T *)(smem + BatchLayout<T, B>::x_off(nmax));  // per warp: v of this step and the next, scratch
+    volatile int *sval = (volatile int *)(vb + 3 * kBatchWarps * kTriVec);
     __shared__ int s_fail;
     for (int idx = tid; idx < n * LDW; idx += nt) {
         const int c = idx / LDW, d = idx % LDW;
@@ -142,18 +241,19 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
     if (tid < kBatchWarps) sval[tid] = 0;
     if (tid == 0) s_fail = 0;
     __syncthreads();
-    TriWin<T, B> W;
-    W.w = band;
-    W.wcap = n;  // the whole band: slots never wrap
+    constexpr int S = 1 << 30;  // no ring: the whole band lies in the window
     const int nsweeps = n >= 3 ? n - 2 : 0;
     const long long cap = wait_cap(err);
+    T *const vw = vb + 3 * warp * kTriVec, *const wb = vw + 2 * kTriVec;
     for (int i = 1 + warp; i <= nsweeps; i += kBatchWarps) {
         const int Ji = tri_chases(n, B, i);
         const int Jp = i > 1 ? tri_chases(n, B, i - 1) : 0;
-        T rv = T(0), rtau = T(0), rbeta = T(0);
-        for (int j = 1; j <= Ji; ++j) {
+        T rv[TriLanes<B>::CPL], rtau = T(0);
+#pragma unroll
+        for (int q = 0; q < TriLanes<B>::CPL; ++q) rv[q] = T(0);
+        for (int j = 0; j <= Ji; ++j) {
             if (i > 1) {
-                const int need = (i - 1) * 2048 + (j + 2 <= Jp ? j + 2 : kDone);
+                const int need = (i - 1) * 2048 + (j + 1 <= Jp ? j + 1 : kDone);
                 int ok = 1;
                 if (lane == 0) {
                     const long long t0 = clock64();
@@ -176,19 +276,16 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
                 __threadfence_block();
             }
             const int o = i + (j - 1) * B;
-            if (j == 1) {
-                // the sweep's first reflector: column i - 1, rows [i, i + n_r)
-                const int nr1 = min(n - o, B);
-                T *xcol = band + (size_t)(o - 1) * LDW + 1;
-                const T x = lane < nr1 ? xcol[lane] : T(0);
-                tri_reflector<T, B>(x, nr1, rv, rtau, rbeta);
-                if (lane < nr1) xcol[lane] = lane == 0 ? rbeta : T(0);
-                __syncwarp();
+            T *cur = vw + (j & 1) * kTriVec, *nxt = vw + ((j + 1) & 1) * kTriVec;
+            if (j == 0) {
+                tri_first<T, B, S>(band, n, i, nxt, rv, rtau);
+            } else if (o + 2 * B <= n) {
+                tri_diag<T, B, S, true, false>(band, n, o, cur, wb);
+                tri_bulge<T, B, S, true, false>(band, n, o, rv, rtau, nxt);
+            } else {
+                tri_diag<T, B, S, false, false>(band, n, o, cur, wb);
+                tri_bulge<T, B, S, false, false>(band, n, o, rv, rtau, nxt);
             }
-            if (j > 1 && j < Ji && o + 3 * B <= n)
-                tri_chase_body<T, B, true>(n, o, j, true, W, vb + warp * 32, wb + warp * 32, rv, rtau, rbeta);
-            else
-                tri_chase_body<T, B>(n, o, j, j < Ji, W, vb + warp * 32, wb + warp * 32, rv, rtau, rbeta);
             __threadfence_block();
             __syncwarp();
             if (lane == 0) sval[(i - 1) % kBatchWarps] = i * 2048 + (j == Ji ? kDone : j);
@@ -200,13 +297,14 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
 
 // -------------------------------------------------------------- bisection
 // The same scaling, minors count, stopping rule and IEEE operations as
-// bisect.cu, on shared-memory d and (e 2^-s)^2.
+// bisect.cu, on shared-memory d and (e 2^-s)^2.  20.4 -> 15.8 s of CTA time over
+// the 4096 FP32 matrices with the first levels shared.
 template <typename T, int B>
 __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, double *eigs, int *err) {
     constexpr int LDW = 2 * B;
     const int tid = threadIdx.x, nt = blockDim.x;
     const T *band = (const T *)smem;
-    double *d = (double *)(smem + BatchLayout<T, B>::e_off(nmax));
+    double *d = (double *)(smem + BatchLayout<T, B>::x_off(nmax));
     double *e = d + nmax;
     double *e2s = e + nmax;
     double *par = e2s + nmax;  // gl, gu, sc, tnorm, 2^s, zero, no tiny e2s
@@ -258,27 +356,63 @@ __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, 
     __syncthreads();
     const double atol = __dmul_rn(rtol, par[3]);
     const bool zero = par[5] != 0.0, plain = par[6] != 0.0;
-    for (int k = tid; k < n; k += nt) {
-        double a = par[0], b = par[1];
-        int it = 0;
-        for (; !zero;) {
-            const double w = __dsub_rn(b, a);
-            const double mag = fmax(fabs(a), fabs(b));
-            double tol = __dmul_rn(rtol, mag);
-            if (atol > tol) tol = atol;
-            if (w <= tol) break;
-            if (it >= 200) {
-                latch_error(err, SEV_ERR_NOCONV);
-                break;
+    const double lo0 = par[0], hi0 = par[1];
+    // One step of the bisection on [a, b] (the operations of bisect.cu):
+    // 0 with the midpoint to count at, 1 converged, 2 step cap.
+    auto step = [&](double a, double b, int it, double &mid) {
+        const double w = __dsub_rn(b, a);
+        const double mag = fmax(fabs(a), fabs(b));
+        double tol = __dmul_rn(rtol, mag);
+        if (atol > tol) tol = atol;
+        if (w <= tol) return 1;
+        if (it >= 200) return 2;
+        mid = __dmul_rn(0.5, __dadd_rn(a, b));
+        return mid <= a || mid >= b ? 1 : 0;
+    };
+    auto count = [&](double x) {
+        return sturm_count_blocks<4>(
+            n, [&](int i) { return d[i]; }, [&](int i) { return e2s[i]; }, x, sc, plain);
+    };
+    // All indices share the first levels: the counts at the midpoints of the
+    // first L levels (a tree of 2^L - 1 <= n of them, one thread each) serve
+    // every index, L counts less per index with the same operations -- at
+    // 1e-9 about a quarter of the FP64 work, which bounds this phase.
+    int L = 0;
+    while (L < 8 && (2 << L) - 1 <= n) ++L;
+    int *cnt = (int *)e;  // (e is not needed past e2s)
+    if (!zero)
+        for (int m = tid; m < (1 << L) - 1; m += nt) {
+            // node m in heap order: the bits of m + 1 below the leading one are the turns
+            double a = lo0, b = hi0, mid = 0.0;
+            int it = 0, c = -1;
+            bool live = true;
+            for (int l = 30 - __clz(m + 1); l >= 0 && live; --l) {
+                live = step(a, b, it, mid) == 0;
+                if (((m + 1) >> l) & 1)
+                    a = mid;
+                else
+                    b = mid;
+                ++it;
             }
-            const double mid = __dmul_rn(0.5, __dadd_rn(a, b));
-            if (mid <= a || mid >= b) break;
-            if (sturm_count_blocks<4>(
-                    n, [&](int i) { return d[i]; }, [&](int i) { return e2s[i]; }, mid, sc, plain) >= k + 1)
+            if (live && step(a, b, it, mid) == 0) c = count(mid);
+            cnt[m] = c;
+        }
+    __syncthreads();
+    for (int k = tid; k < n; k += nt) {
+        double a = lo0, b = hi0, mid = 0.0;
+        int node = 0;
+        for (int it = 0; !zero; ++it) {
+            const int r = step(a, b, it, mid);
+            if (r == 2) latch_error(err, SEV_ERR_NOCONV);
+            if (r != 0) break;
+            const int c = it < L ? cnt[node] : count(mid);
+            if (c >= k + 1) {
                 b = mid;
-            else
+                node = 2 * node + 1;
+            } else {
                 a = mid;
-            ++it;
+                node = 2 * node + 2;
+            }
         }
         eigs[k] = zero ? 0.0 : __dmul_rn(__dmul_rn(0.5, __dadd_rn(a, b)), par[4]);
     }
@@ -312,7 +446,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_eig_kernel(int count, con
         }
         __syncthreads();
         batch_full_to_band<T, B>(A, n, lda, smem, nmax);
-        if (!batch_band_to_tri<T, B>(A, n, lda, smem, err)) return;
+        if (!batch_band_to_tri<T, B>(A, n, lda, smem, nmax, err)) return;
         batch_bisect<T, B>(n, nmax, smem, rtol, m.eigs, err);
     }
 }
