@@ -200,9 +200,13 @@ int sev_tridiag_bisect_static(int n, const double *d, const double *e, double rt
  *          for prec, else 16 (SEV_MIXED) or 8 (SEV_FP64).
  * Matrices with n <= 1024 whose path fits one CTA's shared memory run in ONE
  * persistent launch (each CTA takes matrices largest first from a device
- * queue); the others run through sev_eigvalsh one after another on the
- * handle's stream.  Plan creation allocates the descriptor table and
- * reserves the handle's workspace and synchronises; sev_batch_run only
+ * queue); the others run through sev_eigvalsh, those with n <= 4096 up to
+ * eight at a time on streams of the handle's own which start after the work
+ * enqueued so far on the handle's stream and which that stream then waits
+ * for (one after another on the handle's stream with a caller's workspace,
+ * under capture and with per-kernel timing on).  Plan creation allocates the
+ * descriptor table, reserves the workspaces (kept by the handle until
+ * sev_destroy) and synchronises; sev_batch_run only
  * enqueues work (no allocation, no host synchronisation) and may be
  * captured in a CUDA graph when every matrix runs in the batched launch
  * (sev_batch_plan_info reports large_count == 0).  Errors as sev_eigvalsh.

@@ -3,6 +3,7 @@
 // Algorithm 4.3: full-to-band, band-to-band stages b0 -> ... -> 1 (the stage
 // widths come from schedule() below), and bisection on the final
 // tridiagonal.
+#include <cmath>
 #include <cstddef>
 #include <cstdlib>
 #include <cstring>
@@ -257,8 +258,8 @@ static int full_to_band_t(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ld
 // and the band width of one batch, uploads the per-matrix descriptors once
 // and reserves every workspace, so that running it only launches kernels.
 // Matrices whose whole path fits one CTA's shared memory go to the batched
-// kernel (batched.cu), largest first; the others run the single-matrix path
-// one after another on the handle's stream.
+// kernel (batched.cu), largest first; the others run the single-matrix path,
+// side by side on the handle's lanes where that pays.
 struct sev_batch_s {
     int device = 0;
     int prec = SEV_MIXED;
@@ -272,8 +273,10 @@ struct sev_batch_s {
         void *A;
         double *eigs;
         int n, lda;
+        int lane;  // 0: the handle's own stream
     };
     std::vector<Big> big;
+    int lanes = 1;
 };
 
 namespace sev {
@@ -293,6 +296,67 @@ static bool batch_fits(sev_ctx *h, int prec, int b, int n) {
 }
 
 static double batch_rtol(int prec) { return prec == SEV_FP64 ? 1e-14 : 1e-9; }
+
+// Large matrices side by side.  One matrix of a few thousand rows leaves most
+// SMs idle most of the time -- a panel is one cluster of at most 16 CTAs, a band
+// stage a pipeline of some tens -- and is bound by chains of dependent steps,
+// so several run on lanes of their own: eight FP32 matrices of order 1024..3072
+// 136.8 ms one after another, 81.5 on two lanes, 58 on four and on eight; seven of
+// order 1024..1300 62, 40, 25.5 and 18.7; two of order ~1050 17.5 and 9.6.
+// (The kernels of different lanes never wait on one another, and those that wait
+// within one launch make progress on any part of their grid or start as a whole:
+// clusters and cooperative grids.)  A matrix above kLaneMaxN fills the GPU with
+// its own products and updates; it, a caller's workspace, a capture and
+// per-kernel timing take the handle's stream, one matrix after another.
+constexpr int kLanes = 8;
+constexpr int kLaneMaxN = 4096;
+
+static void lanes_destroy(sev_ctx *h) {
+    for (sev_ctx *l : h->lanes) {
+        if (l->ws_own) cudaFree(l->ws_own);
+        if (l->lane_event) cudaEventDestroy(l->lane_event);
+        if (l->stream) cudaStreamDestroy(l->stream);
+        delete l;
+    }
+    h->lanes.clear();
+    if (h->lane_event) cudaEventDestroy(h->lane_event);
+    h->lane_event = nullptr;
+}
+
+// At least `count` lanes besides the handle's own stream; false: not to be had.
+static bool lanes_reserve(sev_ctx *h, int count) {
+    if (!h->lane_event && cudaEventCreateWithFlags(&h->lane_event, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        h->lane_event = nullptr;
+        return false;
+    }
+    while ((int)h->lanes.size() < count) {
+        sev_ctx *l = new (std::nothrow) sev_ctx();
+        if (!l) return false;
+        if (cudaStreamCreateWithFlags(&l->stream, cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&l->lane_event, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            if (l->stream) cudaStreamDestroy(l->stream);
+            delete l;
+            return false;
+        }
+        l->device = h->device;
+        l->sm_count = h->sm_count;
+        l->smem_optin = h->smem_optin;
+        l->d_err = h->d_err;
+        h->lanes.push_back(l);
+    }
+    return true;
+}
+
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
 
 }  // namespace sev
 
@@ -340,6 +404,7 @@ int sev_destroy(sev_handle h) {
         cudaEventDestroy(t.e1);
     }
     for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
+    lanes_destroy(h);
     if (h->ws_own) cudaFree(h->ws_own);
     if (h->h_stage) cudaFree(h->h_stage);
     if (h->d_err) cudaFree(h->d_err);
@@ -535,7 +600,7 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
         if (batch_fits(h, prec, b, n[i]))
             order.push_back(i);
         else
-            P->big.push_back({A[i], eigs[i], n[i], lda[i]});
+            P->big.push_back({A[i], eigs[i], n[i], lda[i], 0});
     }
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return n[x] > n[y]; });
     P->small_count = (int)order.size();
@@ -566,15 +631,17 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
             return rc;
         }
     }
-    // reserve the single-matrix workspace now, so that running the plan allocates nothing
-    size_t need = 0;
-    for (const auto &g : P->big) {
+    auto ws_bytes = [&](const sev_batch_s::Big &g) {
         const int b0 = pick_b0(h, g.n, prec);
         const int bc = b0 > g.n - 1 ? g.n - 1 : b0;
         size_t w = prec == SEV_FP64 ? eig_workspace<double>(h, g.n, bc) : eig_workspace<float>(h, g.n, bc);
         if (prec == SEV_MIXED && !h->ws_ext) w += full_to_band_copy_bytes<float>(h, g.n, bc, (const float *)g.A, g.lda);
-        if (w > need) need = w;
-    }
+        return w;
+    };
+    // reserve the handle's workspace now, so that running the plan allocates
+    // nothing (for all of them: the plan may have to run on one stream)
+    size_t need = 0;
+    for (const auto &g : P->big) need = std::max(need, ws_bytes(g));
     if (need) {
         void *ws = nullptr;
         const int rc = get_workspace(h, need, &ws);
@@ -583,6 +650,28 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
             delete P;
             return rc;
         }
+    }
+    // lanes of the large matrices: largest first, each to the lane with the least
+    // work so far (a reduction's time grows about as n^1.5 at these orders)
+    int spread = 0;
+    for (const auto &g : P->big) spread += g.n <= kLaneMaxN;
+    P->lanes = h->ws_ext ? 1 : std::min(kLanes, std::max(spread, 1));
+    if (P->lanes > 1) {
+        std::stable_sort(P->big.begin(), P->big.end(),
+                         [](const sev_batch_s::Big &x, const sev_batch_s::Big &y) { return x.n > y.n; });
+        std::vector<double> load(P->lanes, 0.0);
+        std::vector<size_t> need(P->lanes, 0);
+        for (auto &g : P->big) {
+            if (g.n <= kLaneMaxN) g.lane = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+            load[g.lane] += (double)g.n * std::sqrt((double)g.n);
+            need[g.lane] = std::max(need[g.lane], ws_bytes(g));
+        }
+        bool ok = lanes_reserve(h, P->lanes - 1);
+        for (int l = 1; l < P->lanes && ok; ++l) {
+            void *ws = nullptr;
+            ok = get_workspace(h->lanes[l - 1], need[l], &ws) == SEV_OK;
+        }
+        if (!ok) P->lanes = 1;
     }
     *plan = P;
     return SEV_OK;
@@ -602,11 +691,36 @@ int sev_batch_run(sev_handle h, sev_batch_plan P) {
                                              batch_rtol(P->prec), P->grid);
         if (rc) return rc;
     }
-    for (const auto &g : P->big) {
-        rc = sev_eigvalsh(h, g.n, g.A, g.lda, 0, P->prec, g.eigs);
-        if (rc) return rc;
+    // (a plan may be run by another handle of its device than the one that made it)
+    const bool serial = h->ws_ext || h->timing || (int)h->lanes.size() < P->lanes - 1 || capturing(h->stream);
+    const int lanes = serial ? 1 : P->lanes;
+    if (lanes == 1) {
+        for (const auto &g : P->big) {
+            rc = sev_eigvalsh(h, g.n, g.A, g.lda, 0, P->prec, g.eigs);
+            if (rc) return rc;
+        }
+        return SEV_OK;
     }
-    return SEV_OK;
+    SEV_CUDA(cudaEventRecord(h->lane_event, h->stream));
+    for (int l = 1; l < lanes; ++l) {
+        sev_ctx *c = h->lanes[l - 1];
+        c->leaf_rows_override = h->leaf_rows_override;
+        c->chase_x3_min_b = h->chase_x3_min_b;
+        c->tuned = h->tuned;
+        SEV_CUDA(cudaStreamWaitEvent(c->stream, h->lane_event, 0));
+    }
+    for (const auto &g : P->big) {
+        rc = sev_eigvalsh(g.lane ? h->lanes[g.lane - 1] : h, g.n, g.A, g.lda, 0, P->prec, g.eigs);
+        if (rc) break;
+    }
+    // whatever happened, the handle's stream continues after all lanes
+    for (int l = 1; l < lanes; ++l) {
+        sev_ctx *c = h->lanes[l - 1];
+        if (cudaEventRecord(c->lane_event, c->stream) != cudaSuccess ||
+            cudaStreamWaitEvent(h->stream, c->lane_event, 0) != cudaSuccess)
+            rc = rc ? rc : SEV_ERR_CUDA;
+    }
+    return rc;
 }
 
 int sev_batch_plan_destroy(sev_batch_plan P) {
