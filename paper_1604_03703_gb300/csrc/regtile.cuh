@@ -339,54 +339,14 @@ __device__ __forceinline__ T reg_house(T (&x)[R], int k, T *vout) {
     return tau;
 }
 
-// Householder QR of the m x nc block held in `a` (m <= 32R, nc <= NW Q;
-// rows >= m and columns >= nc zero), r = min(nc, m - 1) reflectors.  On
-// return column c holds R above and on the diagonal and v_c below it (unit
-// diagonal implicit); taus[c] = tau_c.  vs: 3 x 32R shared scratch.  With
-// Gm and Tm (shared, leading dimension ldg >= r) the compact-WY factor T of
-// the r reflectors is formed on the way (into Tm; Gm receives G = V^T V
-// above its diagonal): every dot product of a reflector with a finished
-// column is an entry of G that the trailing update computes anyway, and
-// column k - 2 of T is formed in step k by an otherwise waiting warp.
-//
-// Step k applies reflector k.  The warp owning column k + 1 first brings
-// that column up to date and forms reflector k + 1 from it (lookahead); it
-// leaves its other columns for the next step, where it applies reflectors
-// k and k + 1 to them back to back while the next owner forms reflector
-// k + 2.  So a step lasts one column update plus one reflector, the owner's
-// share of the trailing update being off the critical path; every column
-// still receives the reflectors in order 0, 1, 2, ... (the same arithmetic
-// as applying them one step at a time).  Reflectors rotate through three
-// buffers: the deferred warp still reads reflector k - 1 in step k while
-// the owner writes k + 1.
-// Barrier of the warps running reg_qr: the whole CTA (BAR = 0) or named
-// barrier BAR over warps 0 .. NW-1 (the rest of the CTA does other work).
-template <int NW, int BAR>
-__device__ __forceinline__ void reg_sync() {
-    if constexpr (BAR == 0)
-        __syncthreads();
-    else
-        asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NW * 32) : "memory");
-}
-
 // The reflector in buffer slot k % 3, restricted to the row blocks it can
-// touch, applied to this warp's columns c with lo < c < nc; with Gm, the
-// dot products with the finished columns are kept as entries of G.
+// touch, applied to this warp's columns c with lo < c < nc.
 template <typename T, int R, int Q, int NW>
 __device__ __forceinline__ void reg_apply_step(T (&a)[Q][R], const RowBlocks<R> &blk, const T *vs, const T *taus,
-                                               int k, int lo, int nc, T *Gm, int ldg) {
+                                               int k, int lo, int nc) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T tk = taus[k];
-    if (tk == T(0)) {
-        if (Gm && lane == 0) {  // T's column k is zero then; no stale value reaches it
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const int c = warp + NW * q;
-                if (c < k) Gm[c + (size_t)k * ldg] = T(0);
-            }
-        }
-        return;
-    }
+    if (tk == T(0)) return;
     const T *v = vs + (k % 3) * (32 * R);
     bool act[R];
     T vr[R];
@@ -406,46 +366,30 @@ __device__ __forceinline__ void reg_apply_step(T (&a)[Q][R], const RowBlocks<R> 
         reg_apply_f32x2<R, Q>(a, vr, act, tk, cm, dq);
     else
         reg_apply<T, R, Q>(a, vr, act, tk, cm, dq);
-    // G(c, k) = v_c^T v_k for this warp's finished columns c < k: the dot
-    // of reflector k with column c (rows >= k hold v_c there)
-    if (Gm && lane == 0) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const int c = warp + NW * q;
-            if (c < k) Gm[c + (size_t)k * ldg] = dq[q];
-        }
-    }
 }
 
-// Column k of the compact-WY factor T (forward, column-wise: Q = I - V T V^T,
-// T upper triangular, r x r) by one warp: T(k, k) = tau_k, for a < k
-// T(a, k) = -tau_k sum_{q = a}^{k-1} T(a, q) G(q, k) with G = V^T V, and
-// zeros below the diagonal.
-template <typename T>
-__device__ __forceinline__ void reg_t_column(int k, int r, const T *taus, const T *Gm, T *Tm, int ldg) {
-    const int lane = threadIdx.x & 31;
-    const T tk = taus[k];
-    for (int a = k + 1 + lane; a < r; a += 32) Tm[a + (size_t)k * ldg] = T(0);
-    for (int a = lane; a <= k; a += 32) {
-        T s0 = 0, s1 = 0;
-        int q = a;
-        for (; q + 1 < k; q += 2) {
-            s0 += Tm[a + (size_t)q * ldg] * Gm[q + (size_t)k * ldg];
-            s1 += Tm[a + (size_t)(q + 1) * ldg] * Gm[q + 1 + (size_t)k * ldg];
-        }
-        if (q < k) s0 += Tm[a + (size_t)q * ldg] * Gm[q + (size_t)k * ldg];
-        Tm[a + (size_t)k * ldg] = a == k ? tk : -tk * (s0 + s1);
-    }
-}
-
-template <typename T, int R, int Q, int NW, int BAR = 0>
-__device__ int reg_qr(T (&a)[Q][R], int m, int nc, int bstack, T *vs, T *taus, T *Gm = nullptr,
-                      T *Tm = nullptr, int ldg = 0) {
+// Householder QR of the m x nc block held in `a` (m <= 32R, nc <= NW Q;
+// rows >= m and columns >= nc zero), r = min(nc, m - 1) reflectors.  On
+// return column c holds R above and on the diagonal and v_c below it (unit
+// diagonal implicit); taus[c] = tau_c.  vs: 3 x 32R shared scratch.
+//
+// Step k applies reflector k.  The warp owning column k + 1 first brings
+// that column up to date and forms reflector k + 1 from it (lookahead); it
+// leaves its other columns for the next step, where it applies reflectors
+// k and k + 1 to them back to back while the next owner forms reflector
+// k + 2.  So a step lasts one column update plus one reflector, the owner's
+// share of the trailing update being off the critical path; every column
+// still receives the reflectors in order 0, 1, 2, ... (the same arithmetic
+// as applying them one step at a time).  Reflectors rotate through three
+// buffers: the deferred warp still reads reflector k - 1 in step k while
+// the owner writes k + 1.
+template <typename T, int R, int Q, int NW>
+__device__ int reg_qr(T (&a)[Q][R], int m, int nc, int bstack, T *vs, T *taus) {
     static_assert(NW >= 2, "reg_qr: the owner of a column and of the next one must differ");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = nc < m - 1 ? nc : m - 1;
     if (r <= 0) {
-        reg_sync<NW, BAR>();
+        __syncthreads();
         return 0;
     }
     const RowBlocks<R> blk(bstack);
@@ -453,7 +397,7 @@ __device__ int reg_qr(T (&a)[Q][R], int m, int nc, int bstack, T *vs, T *taus, T
         const T t0 = reg_house<T, R>(a[0], 0, vs);
         if (lane == 0) taus[0] = t0;
     }
-    reg_sync<NW, BAR>();
+    __syncthreads();
     // k = r: no step, only the last owner's deferred share (reflector r - 1
     // on its columns past r)
     for (int k = 0; k <= r; ++k) {
@@ -494,84 +438,13 @@ __device__ int reg_qr(T (&a)[Q][R], int m, int nc, int bstack, T *vs, T *taus, T
             const bool deferred = k >= 1 && k < nc && (k % NW) == warp;
             const int kend = step ? k : k - 1;
             for (int kk = deferred ? k - 1 : k; kk <= kend; ++kk)
-                reg_apply_step<T, R, Q, NW>(a, blk, vs, taus, kk, k, nc, Gm, ldg);
-            // T's column k - 2 (G(., k - 2) is complete since the last
-            // barrier) by a warp that neither owns column k + 1 nor is
-            // catching up (warp k mod NW): warp (k + 2) mod NW
-            if (Tm && NW >= 3 && step && k >= 2 && warp == (k + 2) % NW) reg_t_column<T>(k - 2, r, taus, Gm, Tm, ldg);
+                reg_apply_step<T, R, Q, NW>(a, blk, vs, taus, kk, k, nc);
         }
         if (step) {
             if (k1 < nc && (k1 % NW) == warp) RTRACE(k, 3);
-            reg_sync<NW, BAR>();
+            __syncthreads();
         }
     }
-    if (Tm) {
-        // the last columns of T (all of them with two warps), in order
-        reg_sync<NW, BAR>();
-        if (warp == 0)
-            for (int k = (NW >= 3 ? (r - 2 > 0 ? r - 2 : 0) : 0); k < r; ++k) {
-                reg_t_column<T>(k, r, taus, Gm, Tm, ldg);
-                __syncwarp();
-            }
-        reg_sync<NW, BAR>();
-    }
-    return r;
-}
-
-// Householder QR of an m x nc block (m <= 32, nc <= Q) held by ONE warp:
-// lane l keeps row l of every column (a[q] = M(l, q)).  No barrier: each
-// step forms reflector k from column k (reg_house; v through the 32-entry
-// scratch vs) and applies it to the later columns, the dot products of all
-// columns summed together (transposing butterfly); the sums for the
-// finished columns are G(q, k) = v_q^T v_k, from which lane a forms row a
-// of the compact-WY factor T (forward, column-wise) in registers:
-// T(a, k) = -tau_k sum_{q = a}^{k-1} T(a, q) G(q, k), T(k, k) = tau_k.  On
-// return column c holds R on and above the diagonal and v_c below; taus[c]
-// and T (r x r, leading dimension ldt, zeros below the diagonal) are in
-// shared memory; returns r = min(nc, m - 1).
-template <typename T, int Q>
-__device__ int warp_qr(T (&a)[Q], int m, int nc, T *vs, T *taus, T *Tm, int ldt) {
-    const int lane = threadIdx.x & 31;
-    int r = nc < m - 1 ? nc : m - 1;
-    if (r < 0) r = 0;
-    T trow[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) trow[q] = T(0);
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        if (k < r) {
-            T x[1] = {a[k]};
-            const T tk = reg_house<T, 1>(x, k, vs);
-            a[k] = x[0];
-            __syncwarp();
-            const T v = vs[lane];
-            __syncwarp();
-            T d[Q];
-#pragma unroll
-            for (int q = 0; q < Q; ++q) d[q] = q == k ? T(0) : v * a[q];
-            if constexpr (sizeof(T) == 4 && (Q == 2 || Q == 4 || Q == 8 || Q == 16)) {
-                warp_sums_x<Q>(d);
-            } else {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
-            }
-#pragma unroll
-            for (int q = k + 1; q < Q; ++q) a[q] = fmat(-tk * d[q], v, a[q]);
-            T sacc = T(0);
-#pragma unroll
-            for (int q = 0; q < k; ++q) sacc = fmat(trow[q], d[q], sacc);
-            trow[k] = lane < k ? -tk * sacc : (lane == k ? tk : T(0));
-            if (lane == 0) taus[k] = tk;
-        }
-    }
-    if (lane < r) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-            if (q < r) Tm[lane + (size_t)q * ldt] = trow[q];
-    }
-    __syncwarp();
     return r;
 }
 
