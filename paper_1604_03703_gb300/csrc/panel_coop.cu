@@ -13,7 +13,7 @@
 // ~1.5-2 us.  Direct columns need neither the way down nor the reconstruction:
 // U, tau and R are the result (the same reflectors: beta = -sgn(alpha) ||x||,
 // tau in [1, 2]).  Measured (GB300): the whole panel step at n = 16384, b = 128
-// (FP32) 276 -> 83 ms per reduction, n = 8192, b = 64 101 -> 19 ms, n = 2048, b =
+// (FP32) 276 -> 66 ms per reduction, n = 8192, b = 64 101 -> 19 ms, n = 2048, b =
 // 64 16.1 -> 4.0 ms; n = 3001, b = 32 in FP64 200 -> 16 ms.
 //
 // One exchange per column.  With x = column k below row k (zero above) and
@@ -31,7 +31,7 @@
 // barrier is needed.  Two sets of words alternate: a CTA sends column k + 1
 // only after it has read all of column k, so whoever has read column k + 1
 // knows that column k's words may be overwritten.  Panels of up to 4096 rows
-// (FP64: 1024) run on one cluster of at most 16 CTAs, the words going from
+// (2048 over 64 columns, FP64 1024) run on one cluster of at most 16 CTAs, the words going from
 // shared memory to shared memory; taller ones on the whole GPU (cooperative
 // launch, at most one CTA per SM) through L2.  Every wait is capped and latches
 // SEV_ERR_TIMEOUT on expiry.
@@ -627,9 +627,13 @@ size_t panel_coop_words(const sev_ctx *h, int b) {
 
 // Rows per CTA (in units of 32) on the whole GPU: the fewest for which the CTAs
 // stay a moderate number -- more rows mean more arithmetic per CTA and column,
-// more CTAs mean more shares to read.  0: the panel does not fit the GPU.
+// more CTAs mean more shares to read.  Over 64 columns (16 column warps, 96
+// registers a thread) 256 rows do not fit the registers: 128 rows as long as the
+// GPU has the CTAs (n = 16384, b = 128: 70.9 ms of panels per reduction against
+// 82.4).  0: the panel does not fit the GPU.
 template <typename T>
-static int coop_rt(const sev_ctx *h, int N) {
+static int coop_rt(const sev_ctx *h, int N, bool wide) {
+    if (wide && N <= 128 * h->sm_count) return 4;
     const int sizes[3] = {2, 4, 8}, room[3] = {sizeof(T) == 4 ? 0 : 96, sizeof(T) == 4 ? 32 : 128, h->sm_count};
     for (int i = 0; i < 3; ++i) {
         const int C = (N + 32 * sizes[i] - 1) / (32 * sizes[i]);
@@ -640,9 +644,11 @@ static int coop_rt(const sev_ctx *h, int N) {
 
 // The same on one cluster, whose CTAs exchange through shared memory (N = 2048,
 // b = 64: 129 us a panel against 165 through L2); 0: not there.  FP64 keeps few rows per
-// CTA (its FP64 pipes bound the column, not the exchange).
+// CTA (its FP64 pipes bound the column, not the exchange).  Over 64 columns 128
+// rows per CTA here too, and taller panels on the whole GPU (70.9 -> 65.9 ms).
 template <typename T>
-static int coop_cl_rt(int N) {
+static int coop_cl_rt(int N, bool wide) {
+    if (wide) return N <= 128 * kCoopClMax ? 4 : 0;
     if (sizeof(T) == 8) return N <= 64 * kCoopClMax ? 2 : 0;
     return N <= 128 * 8 ? 4 : (N <= 256 * kCoopClMax ? 8 : 0);
 }
@@ -650,7 +656,7 @@ static int coop_cl_rt(int N) {
 template <typename T>
 int panel_coop_supported(const sev_ctx *h, int N, int b) {
     if (h->leaf_rows_override > 0) return 0;  // the caller asked for a tree of that leaf size
-    return b >= 1 && b <= (sizeof(T) == 4 ? 128 : 64) && coop_rt<T>(h, N) > 0;
+    return b >= 1 && b <= (sizeof(T) == 4 ? 128 : 64) && coop_rt<T>(h, N, b > 64) > 0;
 }
 
 template <typename T, int RT>
@@ -711,15 +717,18 @@ static int panel_coop_run_cl(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *T
 
 template <typename T, int Q, int NW>
 static int panel_coop_rt(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
+    constexpr bool wide = NW == 16;
     int rc = SEV_ERR_UNSUPPORTED;
     if constexpr (sizeof(T) == 8) {
-        if (coop_cl_rt<T>(N) == 2) rc = panel_coop_run_cl<T, 2, Q, NW>(h, N, b, P, lda, U, Tm);
+        if (coop_cl_rt<T>(N, wide) == 2) rc = panel_coop_run_cl<T, 2, Q, NW>(h, N, b, P, lda, U, Tm);
     } else {
-        if (coop_cl_rt<T>(N) == 4) rc = panel_coop_run_cl<T, 4, Q, NW>(h, N, b, P, lda, U, Tm);
-        if (coop_cl_rt<T>(N) == 8) rc = panel_coop_run_cl<T, 8, Q, NW>(h, N, b, P, lda, U, Tm);
+        if (coop_cl_rt<T>(N, wide) == 4) rc = panel_coop_run_cl<T, 4, Q, NW>(h, N, b, P, lda, U, Tm);
+        if constexpr (!wide) {
+            if (coop_cl_rt<T>(N, wide) == 8) rc = panel_coop_run_cl<T, 8, Q, NW>(h, N, b, P, lda, U, Tm);
+        }
     }
     if (rc != SEV_ERR_UNSUPPORTED) return rc;
-    switch (coop_rt<T>(h, N)) {
+    switch (coop_rt<T>(h, N, wide)) {
         case 2:
             if constexpr (sizeof(T) == 8) return panel_coop_run<T, 2, Q, NW>(h, N, b, P, lda, U, Tm, comm, tag0);
             return SEV_ERR_UNSUPPORTED;

@@ -42,7 +42,8 @@ def test_panel_fp64_vs_oracle(H, orc, n, b):
     np.testing.assert_allclose(np.tril(got), np.tril(ref), atol=20 * n * EPS64 * np.linalg.norm(A), rtol=0)
 
 
-@pytest.mark.parametrize("n,b", [(257, 128), (400, 127), (513, 100), (300, 33), (1200, 96), (4300, 64), (90, 8), (70, 3)])
+@pytest.mark.parametrize("n,b", [(257, 128), (400, 127), (513, 100), (300, 33), (1200, 96), (2300, 128), (4300, 64), (90, 8),
+                                 (70, 3)])
 def test_panel_fp32_keeps_the_spectrum(H, n, b):
     """Backward stable similarities: ||E||_2 <= 4 n eps32 ||A||_2 (the bound of
     the other FP32 full-to-band test)."""
