@@ -45,7 +45,7 @@
 // then forms the reflector, with T's recurrence in between.
 // Measured (GB300): 64 -> 16 at n = 8192, FP32: 48.1 -> 14.9 ms; 128 -> 32 and
 // 32 -> 16 together at n = 16384: 200 -> 80 ms; 32 -> 16 at n = 3001, FP64: 95.5
-// -> 28.1 ms; 32 -> 16 -> 8 -> 4 -> 2 at n = 512, FP64: 67.0 -> 17.2 ms.
+// -> 19.8 ms; 32 -> 16 -> 8 -> 4 -> 2 at n = 512, FP64: 67.0 -> 14.8 ms.
 #pragma once
 #include "regtile.cuh"
 
@@ -412,7 +412,7 @@ __device__ __forceinline__ void step_make_set(int w, const T (&a)[Q][RT], int m,
 // --------------------------------------------------------------- the kernel
 template <typename T>
 struct StepArgs {
-    int n, ldab, b, h, nsweeps, slots;
+    int n, ldab, b, h, nsweeps, slots, sms;
     T *AB;
     int *flags;  // kStepFlags per sweep
     int *ctr;    // sweep counters of the roles
@@ -471,7 +471,9 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
     using SM = StepSmem<T, RT, Q>;
     constexpr int TN = RT == 1 ? 1 : (RT == 2 ? 2 : 4);   // columns per tile of the thin products
     constexpr int DN = RT == 1 ? 1 : 2;
-    const int role = MULTI ? (int)(blockIdx.x & 3) : (int)(threadIdx.x >> 7);
+    // (FP64: an SM's second block in another role than its first: a chain beside a C2 half)
+    const int turn = sizeof(T) == 8 ? 2 * (int)(blockIdx.x / P.sms) : 0;
+    const int role = MULTI ? ((int)blockIdx.x + turn) & 3 : (int)(threadIdx.x >> 7);
     StepGroup g;
     g.nt = MULTI ? kStepThreadsMulti : kStepThreadsRole;
     g.tid = MULTI ? (int)threadIdx.x : (int)(threadIdx.x & 127);
@@ -821,6 +823,14 @@ int launch_step(sev_ctx *hd, int n, T *AB, int ldab, int b, int h, void *ws, siz
     int groups = hd->sm_count * per_sm / (MULTI ? 4 : 1);
     const int most = MULTI ? step_slots(n, b, h) : step_num_steps(n, b, h, 1) / 2 + 4;
     if (groups > most) groups = most;
+    // The steps of a wide FP64 band keep an SM's FP64 pipes busy, and a second CTA on
+    // the SM stretches its step: one CTA per SM until more than twice as many sweeps
+    // could run (32 -> 16 at n = 3001 23.5 -> 19.8 ms, 64 -> 16 at 8192 102 -> 90),
+    // above that all of them, the second CTA of an SM in another role than the
+    // first (32 -> 16 at n = 6000: 57.3 ms with one CTA per SM, 55.7 with two of the
+    // same role, 49.7).  Narrow bands lose by it (4 -> 2 at n = 512).
+    P.sms = hd->sm_count < 8 ? 4 : hd->sm_count & ~3;
+    if (MULTI && sizeof(T) == 8 && b >= 32 && groups > P.sms / 4 && most <= P.sms / 2) groups = P.sms / 4;
     if (groups > P.nsweeps) groups = P.nsweeps;
     if (groups < 1) groups = 1;
     P.slots = groups;

@@ -37,7 +37,8 @@ def reduce(H, A, b, h, dtype, pad=0):
 
 CASES64 = [(130, 4, 2), (131, 8, 2), (97, 8, 4), (150, 6, 3), (100, 9, 3), (77, 12, 4), (203, 16, 8), (161, 32, 16),
            (170, 32, 4), (33, 32, 16), (34, 32, 16), (65, 32, 16), (66, 32, 8), (301, 64, 16), (129, 64, 32),
-           (193, 64, 2), (300, 96, 32), (385, 128, 16), (400, 128, 8), (60, 20, 10)]
+           (193, 64, 2), (300, 96, 32), (385, 128, 16), (400, 128, 8), (60, 20, 10),
+           (400, 4, 2), (620, 4, 2)]  # (more sweeps at once than one CTA per SM)
 
 
 @pytest.mark.parametrize("n,b,h", CASES64)
@@ -48,6 +49,17 @@ def test_band_step_fp64_vs_oracle(H, orc, n, b, h):
     A, got = reduce(H, A, b, h, torch.float64, pad=n % 2)
     ref = orc.band_to_band(A, b, h)
     np.testing.assert_allclose(np.tril(got), np.tril(ref), atol=20 * n * EPS64 * np.linalg.norm(A), rtol=0)
+
+
+def test_band_step_fp64_one_cta_per_sm(H):
+    """A wide FP64 band whose sweeps are limited to one CTA per SM."""
+    import torch
+
+    n, b, h = 2400, 32, 16
+    A = I.random_band(n, b, 13850)
+    A, got = reduce(H, A, b, h, torch.float64)
+    lam = np.linalg.eigvalsh(A)
+    assert np.abs(np.linalg.eigvalsh(got) - lam).max() <= 20 * n * EPS64 * np.abs(lam).max()
 
 
 @pytest.mark.parametrize("n,b,h", [(900, 32, 16), (901, 32, 8), (700, 64, 16), (701, 64, 8), (515, 128, 32), (513, 128, 64),
