@@ -40,11 +40,13 @@
 // QR (step_qr): four warps, lane = row, columns dealt to the warps; one barrier
 // and one set of warp sums per column: with x the current column below its
 // diagonal entry and v = e + x / (alpha - beta), every warp sums x^T a for its
-// columns and x^T x at once, before the scalars are known.  ~0.5K cycles per
-// column in FP32 against ~2.8K for an owner warp that first updates its column,
-// then forms the reflector, with T's recurrence in between.
+// columns and x^T x at once, before the scalars are known.  ~0.9K cycles per
+// column in FP32 (1.1K at b = 128; FP64 4.8K, its pipe) against ~2.8K for an owner
+// warp that first updates its column, then forms the reflector, with T's
+// recurrence in between.  A step of 128 -> 32: 45% of it the QR, then U T, M (U T)
+// and the loads.
 // Measured (GB300): 64 -> 16 at n = 8192, FP32: 48.1 -> 14.9 ms; 128 -> 32 and
-// 32 -> 16 together at n = 16384: 200 -> 80 ms; 32 -> 16 at n = 3001, FP64: 95.5
+// 32 -> 16 together at n = 16384: 200 -> 72 ms; 32 -> 16 at n = 3001, FP64: 95.5
 // -> 19.8 ms; 32 -> 16 -> 8 -> 4 -> 2 at n = 512, FP64: 67.0 -> 14.8 ms.
 #pragma once
 #include "regtile.cuh"
@@ -247,6 +249,10 @@ __device__ __forceinline__ T step_sums(T (&d)[Q]) {  // sum of value lane >> (5 
 template <typename T, int RT, int Q>
 __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs, T *G, T *tau, T *red, int bar) {
     constexpr int LDG = 4 * Q + 4;
+    // two columns per FMA, selects on a column replaced by branches: fewer
+    // instructions where they bound the step (128 -> 32 at n = 16384, FP32 49.0 -> 45.6
+    // ms, 32 -> 16 at 8191 12.4 -> 11.6); 64 -> 16 and FP64 are 1% faster without
+    constexpr bool PACK = sizeof(T) == 4 && RT != 2;
     const int lane = threadIdx.x & 31;
     const int r = m - 1 < h ? (m - 1 > 0 ? m - 1 : 0) : h;
     // the largest entry: x is held times its power of two, so that no square or
@@ -290,11 +296,28 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
             const T x = xk[lane + 32 * t];  // rows < k are zero
             xr[t] = lane + 32 * t == k ? T(0) : x;
         }
+        if constexpr (PACK) {
+            float2 dd[Q / 2];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            d[q] = T(0);
+            for (int p = 0; p < Q / 2; ++p) dd[p] = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int t = 0; t < RT; ++t) d[q] = fmat(xr[t], a[q][t], d[q]);
+            for (int t = 0; t < RT; ++t) {
+                const float2 xx = make_float2(xr[t], xr[t]);
+#pragma unroll
+                for (int p = 0; p < Q / 2; ++p) dd[p] = ffma2(xx, make_float2(a[2 * p][t], a[2 * p + 1][t]), dd[p]);
+            }
+#pragma unroll
+            for (int p = 0; p < Q / 2; ++p) {
+                d[2 * p] = dd[p].x;
+                d[2 * p + 1] = dd[p].y;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                d[q] = T(0);
+#pragma unroll
+                for (int t = 0; t < RT; ++t) d[q] = fmat(xr[t], a[q][t], d[q]);
+            }
         }
         T tk = T(0), beta = T(0), inv = T(0), s[Q];
         if constexpr (sizeof(T) == 4) {
@@ -333,24 +356,59 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
             ms[q] = c > k ? -tk * s[q] : T(0);
             if (c < k && lane == 0) G[c * LDG + k] = s[q];
         }
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-#pragma unroll
-            for (int t = 0; t < RT; ++t) {
-                const int g = lane + 32 * t;
-                const T u = fmat(ms[q], v[t], a[q][t]);
-                a[q][t] = w + 4 * q == k ? (g > k ? v[t] : (g == k && tk != T(0) ? beta : a[q][t])) : u;
-            }
         const int k1 = k + 1;
-        if (k1 < r && (k1 & 3) == w) {
-            T *xn = xs + (k1 & 1) * (32 * RT);
-            const unsigned pick = 1u << (k1 >> 2);
+        if constexpr (PACK) {
 #pragma unroll
             for (int t = 0; t < RT; ++t) {
-                T x = a[0][t];
+                const float2 vv = make_float2(v[t], v[t]);
 #pragma unroll
-                for (int q = 1; q < Q; ++q) x = (pick >> q) & 1 ? a[q][t] : x;
-                xn[lane + 32 * t] = lane + 32 * t >= k1 ? x * scale : T(0);
+                for (int p = 0; p < Q / 2; ++p) {
+                    const float2 u = ffma2(make_float2(ms[2 * p], ms[2 * p + 1]), vv, make_float2(a[2 * p][t], a[2 * p + 1][t]));
+                    a[2 * p][t] = u.x;
+                    a[2 * p + 1][t] = u.y;
+                }
+            }
+            if (k1 < r && (k1 & 3) == w) {
+                T *xn = xs + (k1 & 1) * (32 * RT);
+                const unsigned pick = 1u << (k1 >> 2);
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if ((pick >> q) & 1) {
+#pragma unroll
+                        for (int t = 0; t < RT; ++t) xn[lane + 32 * t] = lane + 32 * t >= k1 ? a[q][t] * scale : T(0);
+                    }
+            }
+            if ((k & 3) == w) {
+                const unsigned pick = 1u << (k >> 2);
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if ((pick >> q) & 1) {
+#pragma unroll
+                        for (int t = 0; t < RT; ++t) {
+                            const int g = lane + 32 * t;
+                            a[q][t] = g > k ? v[t] : (g == k && tk != T(0) ? beta : a[q][t]);
+                        }
+                    }
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+#pragma unroll
+                for (int t = 0; t < RT; ++t) {
+                    const int g = lane + 32 * t;
+                    const T u = fmat(ms[q], v[t], a[q][t]);
+                    a[q][t] = w + 4 * q == k ? (g > k ? v[t] : (g == k && tk != T(0) ? beta : a[q][t])) : u;
+                }
+            if (k1 < r && (k1 & 3) == w) {
+                T *xn = xs + (k1 & 1) * (32 * RT);
+                const unsigned pick = 1u << (k1 >> 2);
+#pragma unroll
+                for (int t = 0; t < RT; ++t) {
+                    T x = a[0][t];
+#pragma unroll
+                    for (int q = 1; q < Q; ++q) x = (pick >> q) & 1 ? a[q][t] : x;
+                    xn[lane + 32 * t] = lane + 32 * t >= k1 ? x * scale : T(0);
+                }
             }
         }
         if (w == 0 && lane == 0) tau[k] = tk;
@@ -391,10 +449,22 @@ __device__ __forceinline__ void step_make_set(int w, const T (&a)[Q][RT], int m,
             const T mine = tau[k] * acc[k / LPR];
             const T val = LPR == 1 ? mine : __shfl_sync(0xffffffffu, mine, lane % RPW + RPW * (k % LPR));
             if (g == k % LPR) acc[k / LPR] = val;
+            // (columns c >= r take whatever G holds there; they are dropped below)
+            if constexpr (LPR == 1) {
 #pragma unroll
-            for (int i = k / LPR; i < HPL; ++i) {
-                const int c = g + LPR * i;
-                if (c > k) acc[i] = fmat(-val, c < r ? G[k * LDG + c] : T(0), acc[i]);
+                for (int c4 = (k + 1) & ~3; c4 < HPL; c4 += 4) {
+                    T gv[4];
+                    vec_ld<T, 4>(G + k * LDG + c4, gv);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (c4 + u > k) acc[c4 + u] = fmat(-val, gv[u], acc[c4 + u]);
+                }
+            } else {
+#pragma unroll
+                for (int i = k / LPR; i < HPL; ++i) {
+                    const int c = g + LPR * i;
+                    if (c > k) acc[i] = fmat(-val, G[k * LDG + c], acc[i]);
+                }
             }
         }
     }
@@ -459,8 +529,15 @@ struct StepGroup {
     }
 };
 
+// Two CTAs per SM (more sweeps at once: 64 -> 16 at n = 8192 15.0 ms, with one 16.2)
+// where the block in registers leaves room for it.
 template <typename T, int RT, int Q, bool MULTI>
-__global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRole)
+constexpr int step_min_blocks() {
+    return MULTI ? (RT * Q * sizeof(T) <= 64 ? 2 : 1) : (RT == 1 ? 2 : 1);
+}
+
+template <typename T, int RT, int Q, bool MULTI>
+__global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRole, step_min_blocks<T, RT, Q, MULTI>())
     band_step_kernel(StepArgs<T> P) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ volatile int s_abort, s_sweep;
@@ -500,7 +577,7 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
     };
     // rows [0, m) x all b columns of M of the step at r0 into Ms, rows up to b4 zeroed
     auto load_m = [&](int r0, int m) {
-        constexpr int U = RT == 4 ? 4 : 8;
+        constexpr int U = 8;
         for (int c0 = warp; c0 < b; c0 += nw * U) {
             T v[U][RT];
 #pragma unroll
