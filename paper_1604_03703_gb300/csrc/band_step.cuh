@@ -631,10 +631,13 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                 if (!MULTI && role == 2) st_release(mine + 3, j);
             }
         };
-        // set j produced by role 0 is in this role's shared memory
-        auto need_set = [&](int j) {
+        // set j produced by role 0 is in this role's shared memory; ld > 0: and the
+        // role with the other half of C2 has read M of step ld
+        auto need_set = [&](int j, int ld = 0) {
             if constexpr (MULTI) {
-                if (!g.sync_ok(g.tid == 0 && g.flag_failed(mine + 6, j))) return false;
+                const bool failed = (g.tid == 0 && g.flag_failed(mine + 6, j)) ||
+                                    (g.tid == 32 && g.flag_failed(mine + 2 + (role ^ 1), ld));
+                if (!g.sync_ok(failed)) return false;
                 const float4 *src = (const float4 *)ring_of(s, j);
                 float4 *dst = (float4 *)sets;
                 batched_copy<float4, 4>(
@@ -824,6 +827,19 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                     make_w(U0, m, b);
                     g.sync();
                     const bool next = j < J;
+                    // M is written back once every role that needs all of it has read it:
+                    // role 0 before it makes set j + 1, in the last step before it is
+                    // complete; the other half's role as its flag says
+                    if (!next) {
+                        bool failed = false;
+                        if constexpr (MULTI) {
+                            if (g.tid == 0) failed = g.flag_failed(mine, j);
+                            if (g.tid == 32) failed = g.flag_failed(mine + 2 + (role ^ 1), j);
+                        } else if (g.tid == 0) {
+                            failed = g.local_failed(&s_done[0], j);
+                        }
+                        if (!g.sync_ok(failed)) break;
+                    }
                     grp_outer<T, 4, TN, false, false>(
                         g.tid, g.nt, m, nc, h, Ws, ldb, U0 + c_lo, ldb, (const T *)nullptr, 0, (const T *)nullptr, 0,
                         [&](int a, int c, T v) {
@@ -833,7 +849,7 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                         });
                     g.sync();
                     if (next) {
-                        if (!need_set(j + 1)) break;
+                        if (!need_set(j + 1, j)) break;
                         have = true;
                         const T *U1 = set_of(j + 1), *UTc = U1 + ldb * D.h4;
                         grp_dot<T, 2, DN>(g.tid, g.nt, D.h4, nc, D.b4, UTc, ldb, Ms + c_lo * ldb, ldb,
