@@ -174,6 +174,8 @@ def kernel_model(name, n, b0, elem, sched=None):
     band stages b -> h (k = b/h): each of the n/h sweeps reads and writes the
     2b stored diagonals of the columns it passes, ~2 s 2b (n - ih) bytes, so
     2 s k n^2 bytes per stage; the b -> 1 stage is k = b.
+    panel QR: per column the products of x with all b columns and the update of
+    all b columns, 4 N b^2 flops per panel.
     tree-QR nodes: 2(2b)b^2 - (2/3)b^3 flops per stacked-triangle QR (the
     dense count; the kernel skips the structural zeros); leaves of at most
     256 rows, so ceil(N/256) - 1 nodes per panel.
@@ -199,6 +201,8 @@ def kernel_model(name, n, b0, elem, sched=None):
                 continue
             tot += 2.0 * elem * (b // h) * float(n) ** 2
         return tot, "byte", "hbm"
+    if name == "panel_coop":
+        return sum(4.0 * N * b0 * b0 for N in Ns), "flop", "alu"
     if name == "tsqr_node_qr":
         nodes = sum(max(-(-N // 256) - 1, 0) for N in Ns)
         return nodes * (4.0 * b0 ** 3 - 2.0 * b0 ** 3 / 3.0), "flop", "alu"
@@ -213,12 +217,7 @@ def kernel_model(name, n, b0, elem, sched=None):
 # kernel, taken by ncu at this benchmark's configuration (n = 16384, b0 = 128,
 # the schedule named) for the kernel as it is built now; a kernel or schedule
 # absent here reports null.
-MEASURED_TRAFFIC = {
-    "band_chase": {"schedule": [128, 32, 8, 1], "bytes_per_step": 16848640 + 5070080 + 5244672 + 1515776,
-                   "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the two band_chase launches of one "
-                           "eigvalsh (128 -> 32 on clusters: 21.9 MB; 32 -> 8: 6.8 MB), 1 pass, full size: the 16 MB "
-                           "band is read about once and stays in L2"},
-}
+MEASURED_TRAFFIC = {}
 
 
 def roofline(name, amount, unit, bound, ms_per_step, peaks, clocks, elem):

@@ -137,9 +137,8 @@ int sev_full_to_band(sev_handle handle, int n, void *A, int lda, int b, int prec
  * Band-to-band reduction b -> h (Algorithm 4.2) in place on packed band
  * storage.  Requires h >= 1, h < b, b % h == 0, ldab >= 2b.  Entries of AB
  * at distance > b from the diagonal must be zero on entry; on return the
- * band has half-bandwidth h and entries beyond it are zero.  Chases run as a
- * persistent wavefront in which chase (i, j) starts once chase (i-1, j+2)
- * and (i, j-1) are complete.
+ * band has half-bandwidth h and entries beyond it are zero.  Sweeps run as
+ * a persistent pipeline, sweep i two steps behind sweep i - 1.
  */
 int sev_band_to_band(sev_handle handle, int n, void *AB, int ldab, int b, int h, int prec);
 
