@@ -306,7 +306,8 @@ __device__ __forceinline__ T reg_house(T (&x)[R], int k, T *vout) {
         const double ssq = warp_sum(s0 + s1);
         const double al = (double)alpha;
         double td, bd, id;
-        if ((ssq != 0.0 && ssq < 1e-280) || !(ssq < 1e300) || fabs(al) > 1e150 || (al != 0.0 && fabs(al) < 1e-140)) {
+        if ((ssq < 1e-280 && (ssq != 0.0 || al == 0.0)) || !(ssq < 1e300) || fabs(al) > 1e150 ||
+            (al != 0.0 && fabs(al) < 1e-140)) {
             // rare: rescale by an exact power of two so the squares neither
             // overflow nor underflow
             double amax = fabs(al);
@@ -314,20 +315,18 @@ __device__ __forceinline__ T reg_house(T (&x)[R], int k, T *vout) {
             for (int t = 0; t < R; ++t)
                 if (lane + 32 * t > k) amax = fmax(amax, fabs((double)x[t]));
             amax = warp_max(amax);
-            int e2;
-            frexp(amax, &e2);
-            const double sc = ldexp(1.0, -e2);
+            const double sc = pow2i(-house_scale_exp((unsigned)__double2hiint(amax)));
             double a2 = 0.0;
 #pragma unroll
             for (int t = 0; t < R; ++t)
                 if (lane + 32 * t > k) {
                     const double y = (double)x[t] * sc;
                     a2 = fma(y, y, a2);
+                    x[t] = (T)y;  // id belongs to the scaled column (without the scale it may overflow)
                 }
             a2 = warp_sum(a2);
             house_scalars(al * sc, a2, &td, &bd, &id);
             bd /= sc;
-            id *= sc;
         } else {
             house_scalars(al, ssq, &td, &bd, &id);
         }
