@@ -271,25 +271,37 @@ __device__ __forceinline__ T reg_house(T (&x)[R], int k, T *vout) {
     const T alpha = __shfl_sync(0xffffffffu, rsel<R>(x, k >> 5), k & 31);
     T tau, beta, inv;
     if constexpr (sizeof(T) == 4) {
-        F2 a0{0.f, 0.f}, a1{0.f, 0.f};
-#pragma unroll
-        for (int t = 0; t < R; ++t) {
-            const int row = lane + 32 * t;
-            if (row > k) {
-                if (t & 1)
-                    f2_add_sq(a1, (float)x[t]);
-                else
-                    f2_add_sq(a0, (float)x[t]);
-            }
-        }
         RTRACE(k, 4);
-        const F2 acc = warp_sum_f2(f2_add(a0, a1));
+        F2 acc;
+        float sc = 1.f;
+#pragma unroll 1
+        for (;;) {
+            F2 a0{0.f, 0.f}, a1{0.f, 0.f};
+#pragma unroll
+            for (int t = 0; t < R; ++t) {
+                const int row = lane + 32 * t;
+                if (row > k) {
+                    if (t & 1)
+                        f2_add_sq(a1, (float)x[t]);
+                    else
+                        f2_add_sq(a0, (float)x[t]);
+                }
+            }
+            acc = warp_sum_f2(f2_add(a0, a1));
+            if (sc != 1.f) break;
+            const float s = fmaf((float)alpha, (float)alpha, acc.hi);
+            if (!house_f2_needs_scale(s)) break;
+            sc = house_f2_scale(s);
+#pragma unroll
+            for (int t = 0; t < R; ++t)
+                if (lane + 32 * t > k) x[t] = (T)((float)x[t] * sc);
+        }
         RTRACE(k, 5);
         float tf, bf, iv;
-        house_scalars_f2((float)alpha, acc, &tf, &bf, &iv);
+        house_scalars_f2((float)alpha * sc, acc, &tf, &bf, &iv);
         RTRACE(k, 6);
         tau = (T)tf;
-        beta = (T)bf;
+        beta = (T)(sc == 1.f ? bf : bf / sc);
         inv = (T)iv;
     } else {
         double s0 = 0.0, s1 = 0.0;

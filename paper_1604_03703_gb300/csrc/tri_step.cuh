@@ -42,16 +42,29 @@ __device__ __forceinline__ T tri_sum_row(T s) {
     return s;
 }
 
-// tri_house for an FP64 column whose squares leave FP64's range, or a zero one:
-// the column is held times a power of two.  Beside larger entries an inexact tau
+// tri_house for a column whose squares leave the range of its type, or a zero
+// one: the column is held times a power of two.  Beside larger entries an inexact tau
 // would spoil these, and in a matrix of that scale the column is not
 // negligible.  A function of its own: rare, and its registers stay out of the
-// steps (the test for it costs 0.3% of a solve: n = 3001 108.6 -> 109.0 ms).
+// steps (the test for it costs 0.3% of a solve: n = 3001 108.6 -> 108.9 ms
+// in FP64, 8191 rows of width 32 in FP32 43.3 ms as before).
+template <typename T>
 struct TriHouse {
-    double v, tau, beta;
+    T v, tau, beta;
 };
 template <int B>
-__device__ __noinline__ TriHouse tri_house_scaled(double x, int r, int nr) {
+__device__ __noinline__ TriHouse<float> tri_house_scaled(float x, int r, int nr, float sc) {
+    const float y = x * sc;
+    const F2 acc = warp_sum_f2<B>(two_prod(y, y));
+    TriHouse<float> h;
+    float inv;
+    house_scalars_f2s(__shfl_sync(0xffffffffu, y, 0), acc, &h.tau, &h.beta, &inv);
+    h.beta /= sc;
+    h.v = r == 0 ? 1.f : (r < nr ? y * inv : 0.f);
+    return h;
+}
+template <int B>
+__device__ __noinline__ TriHouse<double> tri_house_scaled(double x, int r, int nr) {
     const unsigned hi = r < nr ? (unsigned)__double2hiint(x) & 0x7fffffffu : 0u;
     const int e = house_scale_exp(__reduce_max_sync(0xffffffffu, hi));
     const double y = x * pow2i(-e);
@@ -59,7 +72,7 @@ __device__ __noinline__ TriHouse tri_house_scaled(double x, int r, int nr) {
     double a = rest ? y * y : 0.0;
 #pragma unroll
     for (int off = B / 2; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-    TriHouse h;
+    TriHouse<double> h;
     double inv;
     house_scalars(__shfl_sync(0xffffffffu, y, 0), a, &h.tau, &h.beta, &inv);
     h.beta *= pow2i(e);
@@ -76,17 +89,21 @@ __device__ __forceinline__ void tri_house(T x, int r, int nr, T &v, T &tau, T &b
     if constexpr (sizeof(T) == 4) {
         const F2 acc = warp_sum_f2<B>(two_prod((float)x, (float)x));  // alpha^2 included
         float tf, bf, inf;
-        house_scalars_f2s(__shfl_sync(0xffffffffu, (float)x, 0), acc, &tf, &bf, &inf);
+        house_scalars_f2s_core(__shfl_sync(0xffffffffu, (float)x, 0), acc, &tf, &bf, &inf);
         tau = (T)tf;
         beta = (T)bf;
         v = r == 0 ? T(1) : (rest ? x * (T)inf : T(0));
+        if (house_f2_needs_scale(acc.hi)) {  // (the same in every lane; asked here the test is off the chain)
+            const TriHouse<float> h = tri_house_scaled<B>((float)x, r, nr, house_f2_scale(acc.hi));
+            tau = (T)h.tau, beta = (T)h.beta, v = (T)h.v;
+        }
     } else {
         double a = rest ? (double)x * (double)x : 0.0;
 #pragma unroll
         for (int off = B / 2; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
         const double alpha = (double)__shfl_sync(0xffffffffu, x, 0), s = fma(alpha, alpha, a);
         if (house_needs_scale(s)) {  // (the same in every lane)
-            const TriHouse h = tri_house_scaled<B>((double)x, r, nr);
+            const TriHouse<double> h = tri_house_scaled<B>((double)x, r, nr);
             tau = (T)h.tau, beta = (T)h.beta, v = (T)h.v;
             return;
         }

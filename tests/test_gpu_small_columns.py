@@ -10,8 +10,10 @@ from paper_1604_03703_gb300 import inputs as I
 pytestmark = pytest.mark.gpu
 EPS = {"float64": 2.0**-52, "float32": 2.0**-23}
 # norms whose squares are normal, subnormal, zero
-TINY = {"float64": [1e-140, 1e-150, 1e-153, 1e-155, 1e-157, 1e-160, 1e-170, 1e-300, 1e-310]}
-SCALES = {"float64": [1e-157, 1e-170, 1e-250, 1e160, 1e250]}
+TINY = {"float64": [1e-140, 1e-150, 1e-153, 1e-155, 1e-157, 1e-160, 1e-170, 1e-300, 1e-310],
+        "float32": [1e-17, 1e-19, 1e-20, 1e-21, 1e-22, 1e-24, 1e-30, 1e-40]}
+SCALES = {"float64": [1e-157, 1e-170, 1e-250, 1e160, 1e250],
+          "float32": [1e-20, 1e-22, 1e-25, 1e-30, 1e20, 1e25, 1e30]}
 
 
 @pytest.fixture(scope="module")
