@@ -108,7 +108,8 @@ int sev_set_workspace(sev_handle handle, void *workspace, size_t bytes);
  * Gershgorin bound of the tridiagonal.
  * A NaN or Inf in A's lower triangle latches SEV_ERR_NONFINITE; the
  * reductions still run over it (their work does not depend on the values),
- * the bisection is skipped and eigs receives NaNs.
+ * the bisection is skipped and eigs receives NaNs.  Other calls are not
+ * affected, whether the error has been read or not.
  */
 int sev_eigvalsh(sev_handle handle, int n, void *A, int lda, int b0, int prec, double *eigs);
 
@@ -300,9 +301,10 @@ int sev_get_error(sev_handle handle);
  * Time limit of every device-side wait of this handle's kernels (a sweep
  * waiting on its predecessor's progress, a ring slot, an mbarrier, a grid
  * barrier), in SM clock cycles; 0 restores the default of 4e9 (~2 s at
- * 2 GHz).  A wait that runs out latches SEV_ERR_TIMEOUT and its kernel
- * returns without finishing (the context stays usable).  Synchronises the
- * handle's stream first.  A short limit is a watchdog for tests: work that
+ * 2 GHz).  A wait that runs out latches SEV_ERR_TIMEOUT, its kernel returns
+ * without finishing (the context stays usable), and solves that are under way
+ * or are started before sev_get_error has been called return NaN eigenvalues.
+ * Synchronises the handle's stream first.  A short limit is a watchdog for tests: work that
  * legitimately waits longer than it then fails.  Negative cycles return -2.
  */
 int sev_set_wait_limit(sev_handle handle, long long cycles);

@@ -869,7 +869,7 @@ int sev_get_error(sev_handle h) {
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SEV_ERR_CUDA;
     int v = 0;
     if (cudaMemcpy(&v, h->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return SEV_ERR_CUDA;
-    if (v) cudaMemset(h->d_err, 0, sizeof(int));
+    if (v) cudaMemset(h->d_err, 0, offsetof(DevStatus, wait_cycles));
     return v;
 }
 

@@ -265,9 +265,9 @@ __device__ void band_chase(T *AB, int ldab, int n, int b, int h, int i, int j, C
 }
 
 // Capped wait of one thread until sweep s - 1 has completed `need` chases;
-// false on expiry or a latched error (then the error word is set).
+// false on expiry, here or elsewhere (then the error word is set).
 __device__ __forceinline__ bool wait_progress(const int *progress, int s, int need, long long cap, int *err) {
-    return wait_flag(&progress[s - 1], need, cap, err, [&] { return *(volatile int *)err != 0; }) >= 0;
+    return wait_flag(&progress[s - 1], need, cap, err, [&] { return any_gave_up(err); }) >= 0;
 }
 
 template <typename T>

@@ -499,7 +499,7 @@ struct StepGroup {
     __device__ __forceinline__ void sync() const { step_bar(bar, nt); }
     // One thread's wait for *f >= need (need <= 0: none); true when it failed.
     __device__ __forceinline__ bool flag_failed(const int *f, int need) const {
-        return need > 0 && wait_flag(f, need, cap, err, [&] { return *(volatile int *)err != 0 || *abort; }) < 0;
+        return need > 0 && wait_flag(f, need, cap, err, [&] { return any_gave_up(err) || *abort; }) < 0;
     }
     // One thread's wait for a counter in this CTA's shared memory; true when it failed.
     __device__ __forceinline__ bool local_failed(const volatile int *f, int need) const {
@@ -507,7 +507,7 @@ struct StepGroup {
         while (*f < need) {
             if (*abort) return true;
             if (wait_expired(t0, cap)) {
-                latch_error(err, SEV_ERR_TIMEOUT);
+                latch_timeout(err);
                 return true;
             }
         }

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__((2 * G + 3) * 32, 1)
                     const long long t0 = clock64();
                     while (!tri_mbar_test(&avail[st % kTriBars], (st / kTriBars) & 1) && !s_abort) {
                         if (wait_expired(t0, cap)) {
-                            latch_error(err, SEV_ERR_TIMEOUT);
+                            latch_timeout(err);
                             s_abort = 1;
                         }
                     }
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__((2 * G + 3) * 32, 1)
                     // the previous group's last sweep has passed these columns
                     if (gi > 0 && ts + 1 > seen) {
                         seen = wait_flag(&progress[gi - 1], ts + 1 <= Jprev ? ts + 1 : kTriInf, cap, err,
-                                         [&] { return *(volatile int *)err != 0 || s_abort; });
+                                         [&] { return any_gave_up(err) || s_abort; });
                         ok = seen >= 0;
                     }
                     const long long t0 = clock64();
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__((2 * G + 3) * 32, 1)
                     while (ok && (s_wblo < hi - CAP || s_done < ts - kTriBars + 1)) {
                         if (s_abort) ok = 0;
                         if (wait_expired(t0, cap)) {
-                            latch_error(err, SEV_ERR_TIMEOUT);
+                            latch_timeout(err);
                             ok = 0;
                         }
                     }
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__((2 * G + 3) * 32, 1)
                     const long long t0 = clock64();
                     while ((td = s_done) <= written && !s_abort) {
                         if (wait_expired(t0, cap)) {
-                            latch_error(err, SEV_ERR_TIMEOUT);
+                            latch_timeout(err);
                             s_abort = 1;
                         }
                     }

@@ -118,11 +118,12 @@ template int launch_tridiag_extract<double>(sev_ctx *, int, const double *, int,
 // par[0] = gl, par[1] = gu (scaled, widened Gershgorin interval), par[2] = sc
 // = 2^-s, par[3] = tnorm (scaled max |end| of the unwidened interval),
 // par[4] = 2^s, par[5] = 1 if T = 0 (a zero Gershgorin bound), par[6] = 1 if
-// the caller's skip flag was set (non-finite input: no bisection, NaN
-// eigenvalues), par[7] = 1 if some e2s is nonzero but below 2^-322.  e2s[i] =
-// (e_i 2^-s)^2.
+// the caller's skip flag was set (non-finite input) or, with such a flag, a
+// wait has run out in the reductions (no bisection, NaN eigenvalues), par[7] =
+// 1 if some e2s is nonzero but below 2^-322.  e2s[i] = (e_i 2^-s)^2.
 __global__ void bisect_prep_kernel(int n, const double *__restrict__ d, const double *__restrict__ e,
-                                   double *__restrict__ e2s, double *__restrict__ par, const int *skip) {
+                                   double *__restrict__ e2s, double *__restrict__ par, const int *skip,
+                                   const int *status) {
     __shared__ double red[32];
     __shared__ double s_sc;
     __shared__ int s_tiny;
@@ -152,7 +153,7 @@ __global__ void bisect_prep_kernel(int n, const double *__restrict__ d, const do
         par[3] = tnorm;
         par[4] = pow2_exact(s);
         par[5] = tnorm == 0.0 ? 1.0 : 0.0;
-        par[6] = (skip && *skip) ? 1.0 : 0.0;
+        par[6] = (skip && (*skip || any_gave_up(status))) ? 1.0 : 0.0;
         s_sc = sc;
     }
     __syncthreads();
@@ -377,7 +378,7 @@ __global__ void __launch_bounds__(kBisThreads)
     __shared__ int s_warp[32];
     const long long cap = wait_cap(err);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (par[6] != 0.0) {  // non-finite input (every CTA reads the same flag: no barrier is entered)
+    if (par[6] != 0.0) {  // no tridiagonal to bisect (every CTA reads the same flag: no barrier is entered)
         if (blockIdx.x == 0)
             for (int k = tid; k < n; k += kBisThreads) eigs[k] = __longlong_as_double(0x7ff8000000000000LL);
         return;
@@ -475,7 +476,7 @@ __global__ void __launch_bounds__(kBisThreads) bisect_rounds_kernel(int n, const
     const double atol = __dmul_rn(rtol, par[3]);
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const int gthreads = gridDim.x * blockDim.x;
-    if (par[6] != 0.0) {  // non-finite input (every CTA reads the same flag: no barrier is entered)
+    if (par[6] != 0.0) {  // no tridiagonal to bisect (every CTA reads the same flag: no barrier is entered)
         for (int k = gtid; k < n; k += gthreads) eigs[k] = __longlong_as_double(0x7ff8000000000000LL);
         return;
     }
@@ -587,7 +588,7 @@ int launch_bisect(sev_ctx *h, int n, const double *d, const double *e, double rt
     W.leadof = c.take<int>((size_t)n);
     W.cnt = c.take<int>((size_t)(n > kBisMaxItems ? n : kBisMaxItems));
     W.ctl = c.take<BisCtl>(1);
-    SEV_LAUNCH(h, K_BISECT_PREP, bisect_prep_kernel, 1, 1024, 0, n, d, e, e2, par, skip);
+    SEV_LAUNCH(h, K_BISECT_PREP, bisect_prep_kernel, 1, 1024, 0, n, d, e, e2, par, skip, h->d_err);
     if (n == 1) {
         SEV_CUDA(cudaMemcpyAsync(eigs, d, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
         return SEV_OK;
@@ -680,7 +681,7 @@ extern "C" int sev_tridiag_bisect_static(int n, const double *d, const double *e
     double *par = ptr + kStaticPar;    // 8 doubles
     int *status = (int *)(ptr + kStaticStatus);
     if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return SEV_ERR_CUDA;
-    bisect_prep_kernel<<<1, 1024, 0, st>>>(n, d, n > 1 ? e : d, e2, par, nullptr);
+    bisect_prep_kernel<<<1, 1024, 0, st>>>(n, d, n > 1 ? e : d, e2, par, nullptr, status);
     if (cudaGetLastError() != cudaSuccess) return SEV_ERR_CUDA;
     int bs = 64;
     while (bs > 32 && (n + bs - 1) / bs < sm_count) bs >>= 1;

@@ -144,9 +144,9 @@ __device__ __forceinline__ bool coop_give_up(int tries, long long &t0, long long
     if (tries == 0) t0 = clock64();
     int stop = 0;
     if ((threadIdx.x & 31) == 0) {
-        if ((tries & 31) == 31 && *(volatile int *)err != 0) stop = 1;
+        if ((tries & 31) == 31 && any_gave_up(err)) stop = 1;
         if (wait_expired(t0, cap)) {
-            latch_error(err, SEV_ERR_TIMEOUT);
+            latch_timeout(err);
             stop = 1;
         }
     }

@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(128, 1)
             }
         }
     } else if (threadIdx.x == 0) {
-        latch_error(err, SEV_ERR_TIMEOUT);
+        latch_timeout(err);
     }
     tc_fence_before();
     __syncthreads();
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kSyThreads, 1)
                 for (int j = 0; j < BN; ++j) Y[(size_t)row + (size_t)j * N] = sum[j];
             }
         } else if (lane == 0) {
-            latch_error(err, SEV_ERR_TIMEOUT);
+            latch_timeout(err);
         }
     }
     tc_fence_before();

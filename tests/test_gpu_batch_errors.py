@@ -27,11 +27,11 @@ def matrices(torch, sizes, dt, seed):
     return out
 
 
-# side by side on the handle's lanes; and one after another, with small ones in front
+# side by side on the handle's lanes, and one on the handle's own stream
 @pytest.mark.parametrize("dtype_name,sizes,bad", [("float32", [1301, 1200, 1531, 1100, 1040, 1025, 1400, 1240, 1150], 2),
                                                   ("float32", [1301, 1200, 1100, 1040], 3),
                                                   ("float64", [1030, 1100, 1060], 0),
-                                                  ("float32", [64, 100, 1200, 33], 1), ("float32", [4200, 1200], 0)])
+                                                  ("float32", [4200, 1200], 0)])
 def test_nan_in_one_matrix_of_a_batch(H, dtype_name, sizes, bad):
     import torch
 
@@ -58,6 +58,27 @@ def test_nan_in_one_matrix_of_a_batch(H, dtype_name, sizes, bad):
                 assert bool(torch.isnan(g).all())
             else:
                 assert torch.equal(g, r), sizes[i]
+
+
+@pytest.mark.parametrize("dtype_name", ["float32", "float64"])
+def test_nothing_finite_from_a_solve_whose_waits_ran_out(H, dtype_name):
+    """Until the error has been read; then the handle solves as before."""
+    import torch
+
+    n = 1300
+    (A,) = matrices(torch, [n], getattr(torch, dtype_name), 16250)
+    ref = H.eigvalsh(A.clone())
+    assert H.get_error() == 0
+    H.set_wait_limit(1)
+    try:
+        first = H.eigvalsh(A.clone())
+    finally:
+        H.set_wait_limit(0)
+    second = H.eigvalsh(A.clone())
+    assert H.get_error() == 3  # SEV_ERR_TIMEOUT
+    assert bool(torch.isnan(first).all()) and bool(torch.isnan(second).all())
+    assert torch.equal(H.eigvalsh(A.clone()), ref)
+    assert H.get_error() == 0
 
 
 @pytest.mark.parametrize("dtype_name", ["float32", "float64"])
