@@ -295,6 +295,13 @@ __device__ bool batch_band_to_tri(const T *A, int n, int lda, unsigned char *sme
     return s_fail == 0;
 }
 
+// A matrix that holds a NaN or an Inf has no eigenvalues to find: as in the
+// single-matrix path the error is latched and they are NaN.
+__device__ __forceinline__ void batch_nonfinite(int n, double *eigs, int *err) {
+    if (threadIdx.x == 0) latch_error(err, SEV_ERR_NONFINITE);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) eigs[k] = __longlong_as_double(0x7ff8000000000000LL);
+}
+
 // -------------------------------------------------------------- bisection
 // The same scaling, minors count, stopping rule and IEEE operations as
 // bisect.cu, on shared-memory d and (e 2^-s)^2.  20.4 -> 15.8 s of CTA time over
@@ -315,20 +322,25 @@ __device__ void batch_bisect(int n, int nmax, unsigned char *smem, double rtol, 
     }
     __syncthreads();
     double lo = INFINITY, hi = -INFINITY;
+    bool bad = false;  // an entry that the reductions left non-finite (fmin and fmax would pass over a NaN)
     for (int i = tid; i < n; i += nt) {
         double r = 0.0;
         if (i > 0) r = __dadd_rn(r, fabs(e[i - 1]));
         if (i + 1 < n) r = __dadd_rn(r, fabs(e[i]));
+        bad |= !isfinite(__dadd_rn(fabs(d[i]), r));
         lo = fmin(lo, __dsub_rn(d[i], r));
         hi = fmax(hi, __dadd_rn(d[i], r));
+    }
+    if (__syncthreads_or(bad)) {
+        batch_nonfinite(n, eigs, err);
+        return;
     }
     lo = -block_max(-lo, red);
     hi = block_max(hi, red);
     if (tid == 0) {
         double tnorm = fmax(fabs(lo), fabs(hi));
-        if (!isfinite(tnorm)) latch_error(err, SEV_ERR_NONFINITE);
         int s = 0;
-        if (tnorm > 0.0 && isfinite(tnorm)) (void)frexp(tnorm, &s);
+        if (tnorm > 0.0) (void)frexp(tnorm, &s);
         const double sc = pow2_exact(-s);
         lo = __dmul_rn(lo, sc);
         hi = __dmul_rn(hi, sc);
@@ -436,15 +448,26 @@ __global__ void __launch_bounds__(kBatchThreads) batch_eig_kernel(int count, con
         const int n = m.n, lda = m.lda;
         if (n <= 0) continue;
         if (n == 1) {
-            if (threadIdx.x == 0) m.eigs[0] = (double)A[0];
+            if (threadIdx.x == 0) {
+                m.eigs[0] = (double)A[0];
+                if (!isfinite(A[0])) latch_error(err, SEV_ERR_NONFINITE);
+            }
             continue;
         }
         // mirror the lower triangle: the panel products read all of A22
+        bool bad = false;
         for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
             const int i = idx % n, j = idx / n;
-            if (i < j) A[i + (size_t)j * lda] = A[j + (size_t)i * lda];
+            if (i <= j) {
+                const T v = A[j + (size_t)i * lda];
+                bad |= !isfinite(v);
+                A[i + (size_t)j * lda] = v;
+            }
         }
-        __syncthreads();
+        if (__syncthreads_or(bad)) {
+            batch_nonfinite(n, m.eigs, err);
+            continue;
+        }
         batch_full_to_band<T, B>(A, n, lda, smem, nmax);
         if (!batch_band_to_tri<T, B>(A, n, lda, smem, nmax, err)) return;
         batch_bisect<T, B>(n, nmax, smem, rtol, m.eigs, err);

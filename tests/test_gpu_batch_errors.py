@@ -31,7 +31,9 @@ def matrices(torch, sizes, dt, seed):
 @pytest.mark.parametrize("dtype_name,sizes,bad", [("float32", [1301, 1200, 1531, 1100, 1040, 1025, 1400, 1240, 1150], 2),
                                                   ("float32", [1301, 1200, 1100, 1040], 3),
                                                   ("float64", [1030, 1100, 1060], 0),
-                                                  ("float32", [4200, 1200], 0)])
+                                                  ("float32", [4200, 1200], 0),
+                                                  # in the batched launch
+                                                  ("float32", [64, 100, 1200, 33], 1), ("float64", [64, 100, 33], 2)])
 def test_nan_in_one_matrix_of_a_batch(H, dtype_name, sizes, bad):
     import torch
 
@@ -58,6 +60,31 @@ def test_nan_in_one_matrix_of_a_batch(H, dtype_name, sizes, bad):
                 assert bool(torch.isnan(g).all())
             else:
                 assert torch.equal(g, r), sizes[i]
+
+
+@pytest.mark.parametrize("b", [4, 8, 16])
+@pytest.mark.parametrize("n,i,j,value", [(1, 0, 0, "nan"), (2, 0, 0, "inf"), (2, 1, 0, "nan"), (5, 4, 4, "-inf"),
+                                         (40, 39, 0, "nan"), (200, 199, 199, "nan"), (200, 0, 0, "inf"), (200, 101, 100, "nan")])
+def test_nonfinite_entry_of_a_small_matrix(H, n, i, j, value, b):
+    """Latched, and no eigenvalue is finite (n = 1: the entry itself)."""
+    import torch
+
+    (A,) = matrices(torch, [n], torch.float32, 16260)
+    A[i, j] = A[j, i] = float(value)
+    got = H.eigvalsh_batched([A], b)[0]
+    assert H.get_error() == 1  # SEV_ERR_NONFINITE
+    assert not bool(torch.isfinite(got).any())
+
+
+def test_overflow_inside_the_reduction_is_not_silent(H):
+    """Finite entries whose products overflow FP32."""
+    import torch
+
+    n = 100
+    A = torch.full((n, n), 3e38, device="cuda")
+    got = H.eigvalsh_batched([A], 8)[0]
+    assert H.get_error() == 1  # SEV_ERR_NONFINITE
+    assert bool(torch.isnan(got).all())
 
 
 @pytest.mark.parametrize("dtype_name", ["float32", "float64"])
