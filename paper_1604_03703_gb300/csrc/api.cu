@@ -50,6 +50,14 @@ void timing_end(sev_ctx *h, int kid) {
     if (t.kid == kid) cudaEventRecord(t.e1, h->stream);
 }
 
+cudaError_t allow_smem(const sev_ctx *h, const void *kernel) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(h->smem_optin - a.sharedSizeBytes));
+}
+
 int check_launch(sev_ctx *) {
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SEV_OK : SEV_ERR_CUDA;

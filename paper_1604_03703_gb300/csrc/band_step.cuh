@@ -900,7 +900,7 @@ int launch_step(sev_ctx *hd, int n, T *AB, int ldab, int b, int h, void *ws, siz
     if (smem + 1024 > hd->smem_optin) return SEV_ERR_UNSUPPORTED;
     if (ws_bytes < step_workspace(n, b, h)) return SEV_ERR_WORKSPACE;
     auto kern = band_step_kernel<T, RT, Q, MULTI>;
-    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SEV_CUDA(allow_smem(hd, (const void *)kern));
     const int threads = MULTI ? kStepThreadsMulti : 3 * kStepThreadsRole;
     int per_sm = 0;
     SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));

@@ -322,7 +322,7 @@ static int launch_tri(sev_ctx *h, int n, T *AB, int ldab, int *progress, int *ct
     SEV_CUDA(cudaMemsetAsync(progress, 0, sizeof(int) * (size_t)ngroups, h->stream));
     SEV_CUDA(cudaMemsetAsync(ctr, 0, sizeof(int), h->stream));
     auto kern = band_tri_kernel<T, B, G>;
-    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SEV_CUDA(allow_smem(h, (const void *)kern));
     int per_sm = 0;
     SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (2 * G + 3) * 32, smem));
     if (per_sm < 1) return SEV_ERR_UNSUPPORTED;

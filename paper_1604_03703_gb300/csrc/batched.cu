@@ -494,7 +494,7 @@ static int prepare_batch_b(sev_ctx *h, int count, int nmax, int *grid) {
     const size_t smem = BatchLayout<T, B>::bytes(nmax);
     if (smem > h->smem_optin) return SEV_ERR_UNSUPPORTED;
     auto kern = batch_eig_kernel<T, B>;
-    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SEV_CUDA(allow_smem(h, (const void *)kern));
     int per_sm = 0;
     SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBatchThreads, smem));
     if (per_sm < 1) return SEV_ERR_UNSUPPORTED;

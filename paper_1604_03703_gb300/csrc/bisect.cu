@@ -603,7 +603,7 @@ int launch_bisect(sev_ctx *h, int n, const double *d, const double *e, double rt
     const void *kern = small ? (const void *)bisect_small_kernel : (const void *)bisect_rounds_kernel;
     const size_t smem = small ? bis_small_smem(n) : 0;
     if (small)
-        SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bis_small_smem(kBisSmallN)));
+        SEV_CUDA(allow_smem(h, (const void *)kern));
     int per_sm = 0;
     SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBisThreads, smem));
     if (per_sm < 1) return SEV_ERR_UNSUPPORTED;

@@ -496,8 +496,7 @@ template <typename T>
 int panel_finish_single_leaf(sev_ctx *h, int N, int b, const T *U, const T *tau, const int *nref, const T *R, T *Tm,
                              T *P, int lda) {
     const size_t s_fin = sizeof(T) * 2 * (size_t)(b + 1) * b;
-    SEV_CUDA(cudaFuncSetAttribute(single_leaf_finish_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)s_fin));
+    SEV_CUDA(allow_smem(h, (const void *)single_leaf_finish_kernel<T>));
     SEV_LAUNCH(h, K_RECON_LU, single_leaf_finish_kernel<T>, 1, kThreads, s_fin, N, b, U, N, tau, nref, R, Tm, P, lda);
     return SEV_OK;
 }
@@ -505,7 +504,7 @@ int panel_finish_single_leaf(sev_ctx *h, int N, int b, const T *U, const T *tau,
 template <typename T>
 int panel_form_u2(sev_ctx *h, int N, int b, const T *Q, const T *Winv, T *U, T *P, int lda) {
     const size_t s_u2 = sizeof(T) * (size_t)(b + 1) * b;
-    SEV_CUDA(cudaFuncSetAttribute(recon_u2_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_u2));
+    SEV_CUDA(allow_smem(h, (const void *)recon_u2_kernel<T>));
     const int g2 = (N - b + 63) / 64;
     if (g2 > 0) SEV_LAUNCH(h, K_RECON_U2, recon_u2_kernel<T>, g2, kThreads, s_u2, N, b, Q, N, Winv, U, N, P, lda);
     return SEV_OK;
@@ -540,14 +539,13 @@ int panel_factor(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, void *ws)
         return SEV_ERR_UNSUPPORTED;
 
     const size_t s_leaf = smem_leaf_qr<T>(r_leaf, b);
-    SEV_CUDA(cudaFuncSetAttribute(tsqr_leaf_qr_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_leaf));
+    SEV_CUDA(allow_smem(h, (const void *)tsqr_leaf_qr_kernel<T>));
     if (plan.L == 1) {
         // single leaf: Householder QR of the whole panel gives (U, T) directly
         SEV_LAUNCH(h, K_TSQR_LEAF, tsqr_leaf_qr_kernel<T>, 1, kThreads, s_leaf, P, lda, N, b, r_leaf, 1, U, N, B.tau,
                    B.nref, B.Rbuf, B.Tbuf);
         const size_t s_fin = sizeof(T) * 2 * (size_t)(b + 1) * b;
-        SEV_CUDA(cudaFuncSetAttribute(single_leaf_finish_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)s_fin));
+        SEV_CUDA(allow_smem(h, (const void *)single_leaf_finish_kernel<T>));
         SEV_LAUNCH(h, K_RECON_LU, single_leaf_finish_kernel<T>, 1, kThreads, s_fin, N, b, U, N, B.tau, B.nref, B.Rbuf,
                    Tm, P, lda);
         return SEV_OK;
@@ -556,7 +554,7 @@ int panel_factor(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, void *ws)
                B.Yleaf, N, B.tau, B.nref, B.Rbuf, B.Tbuf);
     // up the tree
     const size_t s_node = smem_node_qr<T>(F, b);
-    SEV_CUDA(cudaFuncSetAttribute(tsqr_node_qr_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_node));
+    SEV_CUDA(allow_smem(h, (const void *)tsqr_node_qr_kernel<T>));
     for (int lev = 1; lev < plan.nlev; ++lev) {
         // internal-node Y slots are indexed by the node's position in its level
         // level by level; reuse one slot array per level (levels run in order
@@ -567,8 +565,7 @@ int panel_factor(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, void *ws)
     }
     // down the tree
     const size_t s_napply = smem_node_apply<T>(F, b, cs);
-    SEV_CUDA(
-        cudaFuncSetAttribute(tsqr_node_apply_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_napply));
+    SEV_CUDA(allow_smem(h, (const void *)tsqr_node_apply_kernel<T>));
     for (int lev = plan.nlev - 1; lev >= 1; --lev) {
         T *Ylev = B.Ynode + (size_t)(plan.off[lev] - plan.L) * plan.ynode_stride;
         dim3 grid(plan.cnt[lev], cs);
@@ -577,17 +574,16 @@ int panel_factor(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, void *ws)
                    lev == plan.nlev - 1 ? 1 : 0, B.Tbuf);
     }
     const size_t s_lapply = smem_leaf_apply<T>(r_leaf, b, cs);
-    SEV_CUDA(
-        cudaFuncSetAttribute(tsqr_leaf_apply_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_lapply));
+    SEV_CUDA(allow_smem(h, (const void *)tsqr_leaf_apply_kernel<T>));
     SEV_LAUNCH(h, K_TSQR_LEAF_Q, tsqr_leaf_apply_kernel<T>, dim3(plan.L, cs), kThreads, s_lapply, N, b, r_leaf, plan.L,
                cs, B.Yleaf, N, B.tau, B.nref, B.Zbuf, B.Q, N, B.Tbuf);
     // reconstruction
     const T *Rroot = B.Rbuf + (size_t)(plan.total - 1) * b * b;
     const size_t s_lu = sizeof(T) * (3 * (size_t)(b + 1) * b + b);
-    SEV_CUDA(cudaFuncSetAttribute(recon_lu_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_lu));
+    SEV_CUDA(allow_smem(h, (const void *)recon_lu_kernel<T>));
     SEV_LAUNCH(h, K_RECON_LU, recon_lu_kernel<T>, 1, kThreads, s_lu, b, B.Q, N, Rroot, U, N, Tm, B.Winv, P, lda);
     const size_t s_u2 = sizeof(T) * (size_t)(b + 1) * b;
-    SEV_CUDA(cudaFuncSetAttribute(recon_u2_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_u2));
+    SEV_CUDA(allow_smem(h, (const void *)recon_u2_kernel<T>));
     const int g2 = (N - b + 63) / 64;
     if (g2 > 0)
         SEV_LAUNCH(h, K_RECON_U2, recon_u2_kernel<T>, g2, kThreads, s_u2, N, b, B.Q, N, B.Winv, U, N, P, lda);

@@ -668,7 +668,7 @@ template <typename T, int RT, int Q, int NW>
 static int panel_coop_run(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, unsigned long long *comm, unsigned tag0) {
     const size_t smem = coop_smem<T, RT>(b);
     auto kern = panel_coop_kernel<T, RT, Q, NW, false>;
-    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SEV_CUDA(allow_smem(h, (const void *)kern));
     const int C = (N + 32 * RT - 1) / (32 * RT);
     int cmax = coop_cmax(h);
     void *args[] = {(void *)&P,    (void *)&lda,  (void *)&N,    (void *)&b,   (void *)&U,
@@ -686,7 +686,7 @@ static int panel_coop_run_cl(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *T
     const size_t smem = coop_smem<T, RT>(b) + 8 * CoopComm<T>::words(b, cmax);
     if (smem > h->smem_optin) return SEV_ERR_UNSUPPORTED;
     auto kern = panel_coop_kernel<T, RT, Q, NW, true>;
-    SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SEV_CUDA(allow_smem(h, (const void *)kern));
     SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];

@@ -474,10 +474,8 @@ static int reg_panel_run(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, c
     const int slices_n = (b + kRegWarps * QN - 1) / (kRegWarps * QN);
     const int slices_l = (b + kRegWarps * QL - 1) / (kRegWarps * QL);
     const size_t s_apply = sizeof(T) * ((size_t)32 * R * b + b);
-    SEV_CUDA(cudaFuncSetAttribute(rtsqr_node_apply_kernel<T, R, QN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)s_apply));
-    SEV_CUDA(cudaFuncSetAttribute(rtsqr_leaf_apply_kernel<T, R, QL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)s_apply));
+    SEV_CUDA(allow_smem(h, (const void *)rtsqr_node_apply_kernel<T, R, QN>));
+    SEV_CUDA(allow_smem(h, (const void *)rtsqr_leaf_apply_kernel<T, R, QL>));
     for (int lev = nlev - 1; lev >= 1; --lev) {
         T *Ylev = B.Ynode + (size_t)(off[lev] - L) * ystride;
         SEV_LAUNCH(h, K_TSQR_DOWN, (rtsqr_node_apply_kernel<T, R, QN>), dim3(cnt[lev], slices_n), kRegThreads,
@@ -488,7 +486,7 @@ static int reg_panel_run(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, c
                L, B.Yleaf, N, B.tau, B.nref, B.Zbuf, B.Q, N);
     const T *Rroot = B.Rbuf + (size_t)(off[nlev - 1]) * b * b;
     const size_t s_rec = sizeof(T) * (2 * (size_t)(b + 1) * b + 2 * 32 * RR + 2 * b);
-    SEV_CUDA(cudaFuncSetAttribute(recon_reg_kernel<T, RR, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_rec));
+    SEV_CUDA(allow_smem(h, (const void *)recon_reg_kernel<T, RR, Q>));
     SEV_LAUNCH(h, K_RECON_LU, (recon_reg_kernel<T, RR, Q>), 1, kRegThreads, s_rec, b, B.Q, N, Rroot, U, N, Tm, B.Winv,
                P, lda);
     return panel_form_u2<T>(h, N, b, B.Q, B.Winv, U, P, lda);

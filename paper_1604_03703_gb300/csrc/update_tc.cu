@@ -685,7 +685,7 @@ int tc_syr2k(sev_ctx *h, int N, int b, T *A22, int lda, void *ws) {
         rc = make_map(&mQ, Q, N, K6p);
         if (rc) return rc;
         const size_t smem = (size_t)kTcStages * kTcStageBytes + 1024;
-        SEV_CUDA(cudaFuncSetAttribute(syr2k_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SEV_CUDA(allow_smem(h, (const void *)syr2k_tc_kernel));
         const long nt = (N + 127) / 128;
         SEV_LAUNCH(h, K_SYR2K_TC, syr2k_tc_kernel, (unsigned)(nt * (nt + 1) / 2), 128, smem, mP, mQ, N, K6p / 64,
                    (float *)A22, lda, h->d_err);
@@ -731,7 +731,7 @@ int tc_symm(sev_ctx *h, int N, int b, const T *A22, int lda, const T *U, T *ypar
         S = (nkb + per - 1) / per;  // every split gets at least one K-block
         const size_t smem = (size_t)kSyRaw * kSyRawBytes + (size_t)kSyCvt * sy_cvt_bytes(b) + 1024;
         auto kern = b == 128 ? symm_tc_kernel<128> : (b == 64 ? symm_tc_kernel<64> : symm_tc_kernel<32>);
-        SEV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SEV_CUDA(allow_smem(h, (const void *)kern));
         SEV_LAUNCH(h, K_SYMM, kern, dim3(rb, S), kSyThreads, smem, mAc, mAr, mUh, mUl, (const float *)A22, lda, N, per,
                    (float *)ypart, (size_t)N * b, h->d_err);
         *splits = S;
