@@ -679,6 +679,16 @@ static int panel_coop_run(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm, 
     return SEV_OK;
 }
 
+// Index of a cluster instance (what the kernel needs of an SM differs among them).
+template <typename T, int RT, int Q, int NW>
+constexpr int coop_cl_index() {
+    constexpr int i = sizeof(T) == 8 ? (Q == 8 ? 1 : 0) : (NW == 16 ? 6 : 2 + (RT == 8 ? 2 : 0) + (Q == 8 ? 1 : 0));
+    static_assert(i < kPanelClKernels && (sizeof(T) == 8 ? RT == 2 && NW == 8 : RT == 4 || (RT == 8 && NW == 8)) &&
+                      (Q == 4 || Q == 8) && (NW == 8 || Q == 8),
+                  "one index per instance");
+    return i;
+}
+
 // One cluster of C CTAs; SEV_ERR_UNSUPPORTED where the GPU cannot hold it.
 template <typename T, int RT, int Q, int NW>
 static int panel_coop_run_cl(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *Tm) {
@@ -700,18 +710,26 @@ static int panel_coop_run_cl(sev_ctx *h, int N, int b, T *P, int lda, T *U, T *T
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (C > 8) {
-        // clusters of more than 8 CTAs depend on the GPU's layout: asked once per handle and size
-        signed char &ok = h->cluster_ok[sizeof(T) == 8][C];
+        // clusters of more than 8 CTAs depend on the GPU's layout: asked once per
+        // handle, kernel and size, for the kernel's widest panel
+        signed char &ok = h->cluster_ok[coop_cl_index<T, RT, Q, NW>()][C];
         if (ok == 0) {
             int fit = 0;
+            cfg.dynamicSmemBytes = coop_smem<T, RT>(Q * NW) + 8 * CoopComm<T>::words(Q * NW, cmax);
             ok = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit > 0 ? 1 : -1;
             cudaGetLastError();
+            cfg.dynamicSmemBytes = smem;
         }
         if (ok < 0) return SEV_ERR_UNSUPPORTED;
     }
     timing_begin(h, K_PANEL_COOP);
-    SEV_CUDA(cudaLaunchKernelEx(&cfg, kern, P, lda, N, b, U, Tm, (unsigned long long *)nullptr, cmax, 0u, h->d_err));
+    const cudaError_t e =
+        cudaLaunchKernelEx(&cfg, kern, P, lda, N, b, U, Tm, (unsigned long long *)nullptr, cmax, 0u, h->d_err);
     timing_end(h, K_PANEL_COOP);
+    if (e != cudaSuccess) {  // the whole-GPU kernel serves the panel (or meets the same error)
+        cudaGetLastError();
+        return SEV_ERR_UNSUPPORTED;
+    }
     return SEV_OK;
 }
 
