@@ -99,6 +99,36 @@ int get_workspace(sev_ctx *h, size_t bytes, void **out) {
     return SEV_OK;
 }
 
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+void *get_copy(sev_ctx *h, size_t need, size_t bytes) {
+    if (bytes == 0) return nullptr;
+    if (h->ws_ext) return h->ws_ext_bytes >= need + bytes ? (char *)h->ws_ext + need : nullptr;
+    if (h->copy_own_bytes < bytes) {
+        if (capturing(h->stream)) return nullptr;
+        if (h->copy_own) {
+            cudaStreamSynchronize(h->stream);
+            cudaFree(h->copy_own);
+            h->copy_own = nullptr;
+            h->copy_own_bytes = 0;
+        }
+        if (cudaMalloc(&h->copy_own, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            h->copy_own = nullptr;
+            return nullptr;
+        }
+        h->copy_own_bytes = bytes;
+    }
+    return h->copy_own;
+}
+
 static int default_b0(int n, int prec) {
     if (prec == SEV_FP64) return n >= 4096 ? 64 : 32;
     return n >= 1024 ? 64 : 32;  // 64 -> 16 -> 1 measured best at n = 16384 (1.18 s against 1.51 s for 128)
@@ -198,15 +228,9 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     const int ldab = 2 * b0 > 2 ? 2 * b0 : 2;
     void *ws = nullptr;
     const size_t need = eig_workspace<T>(h, n, b0);
-    // (a caller's workspace of the queried size has no room for the copy; the
-    // reduction then runs on A as it is)
-    size_t copy = full_to_band_copy_bytes<T>(h, n, b0, A, lda);
-    int rc = get_workspace(h, need + copy, &ws);
-    if (rc && copy) {
-        copy = 0;
-        rc = get_workspace(h, need, &ws);
-    }
+    int rc = get_workspace(h, need, &ws);
     if (rc) return rc;
+    T *const copy = (T *)get_copy(h, need, full_to_band_copy_bytes<T>(h, n, b0, A, lda));
     Carver c(ws);
     T *AB = c.take<T>((size_t)ldab * n);
     double *d = c.take<double>((size_t)n);
@@ -218,12 +242,12 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     // (bounded work, no data-dependent control flow) and the bisection,
     // whose step count depends on the data, is skipped (NaN eigenvalues)
     SEV_CUDA(cudaMemsetAsync(nonfinite, 0, sizeof(int), h->stream));
-    T *const work = copy ? (T *)((char *)ws + need) : A;
+    T *const work = copy ? copy : A;
     const int ldw = copy ? copy_ld(n) : lda;
-    rc = launch_check_finite<T>(h, n, A, lda, nonfinite, copy ? work : nullptr, ldw);
+    rc = launch_check_finite<T>(h, n, A, lda, nonfinite, copy, ldw);
     if (rc) return rc;
     if (b0 < n - 1) {
-        rc = launch_full_to_band<T>(h, n, work, ldw, b0, AB, ldab, stage, stage_bytes, copy != 0);
+        rc = launch_full_to_band<T>(h, n, work, ldw, b0, AB, ldab, stage, stage_bytes, copy != nullptr);
     } else {
         rc = launch_band_from_dense<T>(h, n, A, lda, b0, AB, ldab);
     }
@@ -242,19 +266,15 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
 template <typename T>
 static int full_to_band_t(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ldab) {
     const size_t need = full_to_band_workspace<T>(h, n, b);
-    size_t copy = full_to_band_copy_bytes<T>(h, n, b, A, lda);
     void *ws = nullptr;
-    int rc = get_workspace(h, need + copy, &ws);
-    if (rc && copy) {
-        copy = 0;
-        rc = get_workspace(h, need, &ws);
-    }
+    int rc = get_workspace(h, need, &ws);
     if (rc) return rc;
-    T *const work = copy ? (T *)((char *)ws + need) : A;
+    T *const copy = (T *)get_copy(h, need, full_to_band_copy_bytes<T>(h, n, b, A, lda));
+    T *const work = copy ? copy : A;
     const int ldw = copy ? copy_ld(n) : lda;
-    rc = launch_check_finite<T>(h, n, A, lda, nullptr, copy ? work : nullptr, ldw);
+    rc = launch_check_finite<T>(h, n, A, lda, nullptr, copy, ldw);
     if (rc) return rc;
-    rc = launch_full_to_band<T>(h, n, work, ldw, b, AB, ldab, ws, need, copy != 0);
+    rc = launch_full_to_band<T>(h, n, work, ldw, b, AB, ldab, ws, need, copy != nullptr);
     if (rc || !copy) return rc;
     return launch_dense_from_band<T>(h, n, A, lda, b, AB, ldab);
 }
@@ -323,6 +343,7 @@ constexpr int kLaneMaxN = 4096;
 static void lanes_destroy(sev_ctx *h) {
     for (sev_ctx *l : h->lanes) {
         if (l->ws_own) cudaFree(l->ws_own);
+        if (l->copy_own) cudaFree(l->copy_own);
         if (l->lane_event) cudaEventDestroy(l->lane_event);
         if (l->stream) cudaStreamDestroy(l->stream);
         delete l;
@@ -356,15 +377,6 @@ static bool lanes_reserve(sev_ctx *h, int count) {
         h->lanes.push_back(l);
     }
     return true;
-}
-
-static bool capturing(cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-        cudaGetLastError();
-        return true;
-    }
-    return st != cudaStreamCaptureStatusNone;
 }
 
 }  // namespace sev
@@ -415,6 +427,7 @@ int sev_destroy(sev_handle h) {
     for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
     lanes_destroy(h);
     if (h->ws_own) cudaFree(h->ws_own);
+    if (h->copy_own) cudaFree(h->copy_own);
     if (h->h_stage) cudaFree(h->h_stage);
     if (h->d_err) cudaFree(h->d_err);
     delete h;
@@ -643,14 +656,19 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
     auto ws_bytes = [&](const sev_batch_s::Big &g) {
         const int b0 = pick_b0(h, g.n, prec);
         const int bc = b0 > g.n - 1 ? g.n - 1 : b0;
-        size_t w = prec == SEV_FP64 ? eig_workspace<double>(h, g.n, bc) : eig_workspace<float>(h, g.n, bc);
-        if (prec == SEV_MIXED && !h->ws_ext) w += full_to_band_copy_bytes<float>(h, g.n, bc, (const float *)g.A, g.lda);
-        return w;
+        return prec == SEV_FP64 ? eig_workspace<double>(h, g.n, bc) : eig_workspace<float>(h, g.n, bc);
+    };
+    auto copy_bytes = [&](const sev_batch_s::Big &g) {
+        const int b0 = pick_b0(h, g.n, prec);
+        return prec == SEV_FP64 ? 0 : full_to_band_copy_bytes<float>(h, g.n, std::min(b0, g.n - 1), (const float *)g.A, g.lda);
     };
     // reserve the handle's workspace now, so that running the plan allocates
     // nothing (for all of them: the plan may have to run on one stream)
-    size_t need = 0;
-    for (const auto &g : P->big) need = std::max(need, ws_bytes(g));
+    size_t need = 0, copy = 0;
+    for (const auto &g : P->big) {
+        need = std::max(need, ws_bytes(g));
+        copy = std::max(copy, copy_bytes(g));
+    }
     if (need) {
         void *ws = nullptr;
         const int rc = get_workspace(h, need, &ws);
@@ -660,6 +678,7 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
             return rc;
         }
     }
+    if (!h->ws_ext) get_copy(h, 0, copy);
     // lanes of the large matrices: largest first, each to the lane with the least
     // work so far (a reduction's time grows about as n^1.5 at these orders)
     int spread = 0;
@@ -669,16 +688,18 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
         std::stable_sort(P->big.begin(), P->big.end(),
                          [](const sev_batch_s::Big &x, const sev_batch_s::Big &y) { return x.n > y.n; });
         std::vector<double> load(P->lanes, 0.0);
-        std::vector<size_t> need(P->lanes, 0);
+        std::vector<size_t> need(P->lanes, 0), copy(P->lanes, 0);
         for (auto &g : P->big) {
             if (g.n <= kLaneMaxN) g.lane = (int)(std::min_element(load.begin(), load.end()) - load.begin());
             load[g.lane] += (double)g.n * std::sqrt((double)g.n);
             need[g.lane] = std::max(need[g.lane], ws_bytes(g));
+            copy[g.lane] = std::max(copy[g.lane], copy_bytes(g));
         }
         bool ok = lanes_reserve(h, P->lanes - 1);
         for (int l = 1; l < P->lanes && ok; ++l) {
             void *ws = nullptr;
             ok = get_workspace(h->lanes[l - 1], need[l], &ws) == SEV_OK;
+            if (ok) get_copy(h->lanes[l - 1], 0, copy[l]);
         }
         if (!ok) P->lanes = 1;
     }
