@@ -68,7 +68,7 @@ struct ChaseSmem {
     double *red;
     int ldb1, ldh1;
     __device__ ChaseSmem(unsigned char *base, int b, int h) {
-        ldb1 = b + 4;  // a multiple of 4: 16-byte aligned columns for vector loads
+        ldb1 = b + 4;  // 16-byte aligned columns for vector loads where b is a multiple of 4
         ldh1 = h + 1;
         Us = (T *)base;
         UTs = Us + (size_t)ldb1 * h;
@@ -96,12 +96,12 @@ size_t band_smem_bytes(int b, int h) {
 // The qr-row diagonal block X_d (n_r x n_r, mirrored in S.Xs) after U, T
 // and U T are formed: W_d = X_d (U T); S = U^T W_d; Z = T^T S; V_d = -W_d +
 // U Z / 2; X_d += U V_d^T + V_d U^T; the lower triangle written back.
-template <typename T>
+// VEC: 16-byte loads of FP32 operands (b a multiple of 4).
+template <typename T, bool VEC>
 __device__ void chase_diag_update(T *AB, int ldab, int n, int n_r, int nr, int o_qr_r, ChaseSmem<T> &S, int &bad) {
     const int ldb1 = S.ldb1, ldh1 = S.ldh1;
     const int tid = threadIdx.x, nt = blockDim.x;
-    constexpr bool kVec = sizeof(T) == 4;
-    cta_mm<T, 4, 4, false, kVec>(n_r, nr, n_r, T(1), S.Xs, ldb1, S.UTs, ldb1, 0, nullptr, 0, nullptr, 0, T(0), S.Ws,
+    cta_mm<T, 4, 4, false, VEC>(n_r, nr, n_r, T(1), S.Xs, ldb1, S.UTs, ldb1, 0, nullptr, 0, nullptr, 0, T(0), S.Ws,
                                  ldb1);
     __syncthreads();
     cta_gemm<T, true, false>(nr, nr, n_r, T(1), S.Us, ldb1, S.Ws, ldb1, T(0), S.Zs, ldh1);
@@ -114,13 +114,13 @@ __device__ void chase_diag_update(T *AB, int ldab, int n, int n_r, int nr, int o
         S.Z2s[a + (size_t)c * ldh1] = z;
     }
     __syncthreads();
-    cta_mm<T, 4, 4, false, kVec>(n_r, nr, nr, T(0.5), S.Us, ldb1, S.Z2s, ldh1, 0, nullptr, 0, nullptr, 0, T(-1),
+    cta_mm<T, 4, 4, false, VEC>(n_r, nr, nr, T(0.5), S.Us, ldb1, S.Z2s, ldh1, 0, nullptr, 0, nullptr, 0, T(-1),
                                  S.Ws, ldb1);
     __syncthreads();
     const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
     if (n_r >= 64) {
         // X_d += [U V_d] [V_d U]^T on the tiles on or below the diagonal
-        cta_mm<T, 8, 8, true, kVec, true>(n_r, n_r, nr, T(1), S.Us, ldb1, S.Ws, ldb1, nr, S.Ws, ldb1, S.Us, ldb1, T(1),
+        cta_mm<T, 8, 8, true, VEC, true>(n_r, n_r, nr, T(1), S.Us, ldb1, S.Ws, ldb1, nr, S.Ws, ldb1, S.Us, ldb1, T(1),
                                           S.Xs, ldb1);
         __syncthreads();
         // lower triangle, down the columns (band storage: rows of a column contiguous)
@@ -140,7 +140,7 @@ __device__ void chase_diag_update(T *AB, int ldab, int n, int n_r, int nr, int o
 }
 
 // One chase (i, j) performed by the whole CTA, its QR in shared memory.
-template <typename T>
+template <typename T, bool VEC>
 __device__ void band_chase(T *AB, int ldab, int n, int b, int h, int i, int j, ChaseSmem<T> &S, int &bad) {
     const int o_qr_r = (i - 1) * h + (j - 1) * b + h;
     int o_qr_c, o_v, o_up_c, lim;
@@ -187,8 +187,7 @@ __device__ void band_chase(T *AB, int ldab, int n, int b, int h, int i, int j, C
         __syncthreads();
         cta_form_t(n_r, nr, S.Us, ldb1, S.tau, S.Ts, ldh1, S.Zs, ldh1);
     }
-    constexpr bool kVec = sizeof(T) == 4;
-    cta_mm<T, 4, 4, false, kVec>(n_r, nr, nr, T(1), S.Us, ldb1, S.Ts, ldh1, 0, nullptr, 0, nullptr, 0, T(0), S.UTs,
+    cta_mm<T, 4, 4, false, VEC>(n_r, nr, nr, T(1), S.Us, ldb1, S.Ts, ldh1, 0, nullptr, 0, nullptr, 0, T(0), S.UTs,
                                  ldb1);
     __syncthreads();
     // 4. the qr-row diagonal block X_d (n_r x n_r): two-sided update (the
@@ -209,7 +208,7 @@ __device__ void band_chase(T *AB, int ldab, int n, int b, int h, int i, int j, C
         if (r < c) S.Xs[r + (size_t)c * ldb1] = S.Xs[c + (size_t)r * ldb1];
     }
     __syncthreads();
-    chase_diag_update<T>(AB, ldab, n, n_r, nr, o_qr_r, S, bad);
+    chase_diag_update<T, VEC>(AB, ldab, n, n_r, nr, o_qr_r, S, bad);
     __syncthreads();
     // 5. the other rows of W (above: [0, o_v), below: [o_v + n_r, n_c)):
     //    X <- X - (X U T) U^T, in chunks of at most b rows
@@ -232,13 +231,13 @@ __device__ void band_chase(T *AB, int ldab, int n, int b, int h, int i, int j, C
                     [&](int k, T v) { S.Xs[k % rows + (size_t)(k / rows) * ldb1] = v; });
             }
             __syncthreads();
-            cta_mm<T, 4, 4, false, kVec>(rows, nr, n_r, T(1), S.Xs, ldb1, S.UTs, ldb1, 0, nullptr, 0, nullptr, 0, T(0),
+            cta_mm<T, 4, 4, false, VEC>(rows, nr, n_r, T(1), S.Xs, ldb1, S.UTs, ldb1, 0, nullptr, 0, nullptr, 0, T(0),
                                          S.Ws, ldb1);
             __syncthreads();
             // X <- X - W U^T: register-tiled for wide blocks, else folded into the stores
             const bool tiled = n_r >= 64;
             if (tiled) {
-                cta_mm<T, 8, 8, true, kVec>(rows, n_r, nr, T(-1), S.Ws, ldb1, S.Us, ldb1, 0, nullptr, 0, nullptr, 0,
+                cta_mm<T, 8, 8, true, VEC>(rows, n_r, nr, T(-1), S.Ws, ldb1, S.Us, ldb1, 0, nullptr, 0, nullptr, 0,
                                             T(1), S.Xs, ldb1);
                 __syncthreads();
             }
@@ -270,7 +269,7 @@ __device__ __forceinline__ bool wait_progress(const int *progress, int s, int ne
     return wait_flag(&progress[s - 1], need, cap, err, [&] { return any_gave_up(err); }) >= 0;
 }
 
-template <typename T>
+template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) band_chase_kernel(int n, T *AB, int ldab, int b, int h, int nsweeps,
                                                                int *progress, int *sweep_ctr, int *err) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -296,7 +295,7 @@ __global__ void __launch_bounds__(kThreads) band_chase_kernel(int n, T *AB, int 
                 __syncthreads();
                 if (s_abort) return;
             }
-            band_chase<T>(AB, ldab, n, b, h, i, j, S, bad);
+            band_chase<T, VEC>(AB, ldab, n, b, h, i, j, S, bad);
             __syncthreads();
             // the release store orders the CTA's writes (made visible to
             // thread 0 by the barrier above) before the progress flag
@@ -330,7 +329,8 @@ int launch_band_to_band(sev_ctx *hd, int n, T *AB, int ldab, int b, int h, void 
     int *ctr = c.take<int>(1);
     SEV_CUDA(cudaMemsetAsync(progress, 0, sizeof(int) * ((size_t)nsweeps + 1), hd->stream));
     SEV_CUDA(cudaMemsetAsync(ctr, 0, sizeof(int), hd->stream));
-    auto kern = band_chase_kernel<T>;
+    // a width that is no multiple of 4 has columns that 16-byte loads cannot serve
+    auto kern = sizeof(T) == 4 && b % 4 == 0 ? band_chase_kernel<T, sizeof(T) == 4> : band_chase_kernel<T, false>;
     SEV_CUDA(allow_smem(hd, (const void *)kern));
     int per_sm = 0;
     SEV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));

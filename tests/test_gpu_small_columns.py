@@ -118,7 +118,7 @@ def test_eigvalsh_and_batch_at_extreme_scales(H, dt, scale):
 
 @pytest.mark.parametrize("dt,c", cases(TINY))
 def test_tree_panels_with_tiny_couplings(monkeypatch, dt, c):
-    """The tree QR's register leaves (b = 16) and shared-memory ones (b = 12);
+    """The tree QR's register leaves (b = 16, 12) and shared-memory ones (b = 5);
     a column whose leading entry is zero."""
     import torch
 
@@ -127,7 +127,7 @@ def test_tree_panels_with_tiny_couplings(monkeypatch, dt, c):
     monkeypatch.setenv("SEV_LEAF_ROWS", "64")
     h = api.Handle(0)
     n = 200
-    for b in (16, 12):
+    for b in (16, 12, 5):
         for k in (1, b, b + 1):
             A = couple(I.semicircle(n, 17400 + b), [k], c)
             A[b, 0] = A[0, b] = 0.0
