@@ -79,12 +79,12 @@ constexpr int kStepThreadsRole = 128, kStepThreadsMulti = 256;
 template <typename T, int RT, int Q>
 struct StepSmem {
     // elements: role 0: M, W, G, two column buffers, tau, scratch; role 1: X, W, Z;
-    // role 2: M, W, Z
+    // role 2: M, and W, whose place Z takes
     static __host__ __device__ int role0(const StepDims &d) {
         return d.ldb * d.b4 + d.ldb * d.h4 + 4 * Q * (4 * Q + 4) + 2 * 32 * RT + 4 * Q + 16;
     }
     static __host__ __device__ int role1(const StepDims &d) { return d.ldb * d.b4 + d.ldb * d.h4 + d.ldu * d.h4; }
-    static __host__ __device__ int role2(const StepDims &d) { return d.ldb * d.b4 + 2 * d.ldb * d.h4; }
+    static __host__ __device__ int role2(const StepDims &d) { return d.ldb * d.b4 + d.ldb * d.h4; }
     static __host__ __device__ size_t bytes(int b, int h, bool multi) {
         const StepDims d(b, h);
         const int m01 = role0(d) > role1(d) ? role0(d) : role1(d);
@@ -165,7 +165,8 @@ __device__ __forceinline__ void grp_outer(int tid, int nt, int M, int N, int K, 
 }
 
 // f(m, n, sum_k A(k, m) B(k, n)), A[k + m lda], B[k + n ldb] (k contiguous; K a
-// multiple of 4, padded with zeros in A).
+// multiple of 4, padded with zeros in A).  With N odd the last tile reads one
+// column past B -- of the pad or of the buffer behind it -- and drops the result.
 template <typename T, int TM, int TN, typename F>
 __device__ __forceinline__ void grp_dot(int tid, int nt, int M, int N, int K, const T *A, int lda, const T *B, int ldb,
                                         F f) {
@@ -795,7 +796,7 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
             }
         } else {
             // ------------------------- roles 2, 3: the other columns of M, half each
-            T *const Zt = Xtra;
+            T *const Zt = Ws;  // (Z is formed once W has been used)
             const int w2 = b - h;
             int c_lo = h, nc = w2;
             if constexpr (MULTI) {
@@ -807,7 +808,7 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                     nc = w2 - min(half, w2);
                 }
             }
-            bool have = false;  // the set in shared memory is H_j's (MULTI)
+            bool have = false;                // the set in shared memory is H_j's (MULTI)
             for (int j = 1; j <= J; ++j) {
                 const int r0 = i * h + (j - 1) * b, m = min(n - (r0 + b), b);
                 if (i > 1 && !g.wait4(prev, min(j + 1, Jp), min(j + 1, Jp), min(j, Jp), min(j, Jp))) break;
@@ -840,13 +841,25 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                         }
                         if (!g.sync_ok(failed)) break;
                     }
-                    grp_outer<T, 4, TN, false, false>(
-                        g.tid, g.nt, m, nc, h, Ws, ldb, U0 + c_lo, ldb, (const T *)nullptr, 0, (const T *)nullptr, 0,
-                        [&](int a, int c, T v) {
-                            T &x = Ms[a + (c_lo + c) * ldb];
-                            x -= v;
-                            if (!next) AB[(b + a - c_lo - c) + (size_t)(r0 + c_lo + c) * ldab] = x;
-                        });
+                    auto c2 = [&](int a, int c, T v) {  // (columns counted from c_lo)
+                        if (sizeof(T) == 8 && c < 0) return;
+                        T &x = Ms[a + (c_lo + c) * ldb];
+                        x -= v;
+                        if (!next) AB[(b + a - c_lo - c) + (size_t)(r0 + c_lo + c) * ldab] = x;
+                    };
+                    // TN rows of U are read at once, from a multiple of TN on; other
+                    // targets: FP64 starts before c_lo and drops what lies there, FP32 reads
+                    // single rows (starting early costs FP32 128 -> 32 2%, single
+                    // rows FP64 64 -> 16 3%, both without need)
+                    constexpr bool EARLY = sizeof(T) == 8;
+                    const int off = EARLY ? c_lo & (TN - 1) : 0;
+                    if (EARLY || c_lo % TN == 0)
+                        grp_outer<T, 4, TN, false, false>(g.tid, g.nt, m, nc + off, h, Ws, ldb, U0 + c_lo - off, ldb,
+                                                          (const T *)nullptr, 0, (const T *)nullptr, 0,
+                                                          [&](int a, int c, T v) { c2(a, c - off, v); });
+                    else
+                        grp_outer<T, 4, 1, false, false>(g.tid, g.nt, m, nc, h, Ws, ldb, U0 + c_lo, ldb,
+                                                         (const T *)nullptr, 0, (const T *)nullptr, 0, c2);
                     g.sync();
                     if (next) {
                         if (!need_set(j + 1, j)) break;
@@ -869,12 +882,7 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
 }
 
 // -------------------------------------------------------------------- host
-// Thin products read TN columns at once from column h on: h a multiple of TN.
-inline bool step_shape_ok(int b, int h) {
-    if (b < 2 || b > 128 || h > 64) return false;
-    const int tn = b <= 32 ? 1 : (b <= 64 ? 2 : 4);
-    return h % tn == 0;
-}
+inline bool step_shape_ok(int b, int h) { return b >= 2 && b <= 128 && h <= 64; }
 inline int step_rt(int b) { return b <= 32 ? 1 : (b <= 64 ? 2 : 4); }
 inline int step_q(int h) { return h <= 8 ? 2 : (h <= 16 ? 4 : (h <= 32 ? 8 : 16)); }
 

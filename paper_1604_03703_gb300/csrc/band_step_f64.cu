@@ -15,6 +15,7 @@ int launch_band_step(sev_ctx *hd, int n, double *AB, int ldab, int b, int h, voi
     if (rt == 2 && q == 8) return launch_step<double, 2, 8, true>(hd, n, AB, ldab, b, h, ws, ws_bytes);
     if (rt == 4 && q == 2) return launch_step<double, 4, 2, true>(hd, n, AB, ldab, b, h, ws, ws_bytes);
     if (rt == 4 && q == 4) return launch_step<double, 4, 4, true>(hd, n, AB, ldab, b, h, ws, ws_bytes);
+    if (rt == 4 && q == 8) return launch_step<double, 4, 8, true>(hd, n, AB, ldab, b, h, ws, ws_bytes);
     return SEV_ERR_UNSUPPORTED;
 }
 

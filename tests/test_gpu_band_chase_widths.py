@@ -1,6 +1,6 @@
-"""The general band chase at widths and targets that only it takes: FP32 widths
-that are no multiple of 4 (their columns do not suit 16-byte loads), bands over
-128, and the solves that reach them."""
+"""Band reductions at widths that are no multiple of 4 (their columns do not suit
+16-byte loads of FP32 operands), those over 128 in the general chase among
+them, and the solves that go through such widths."""
 import numpy as np
 import pytest
 
