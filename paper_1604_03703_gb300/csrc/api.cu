@@ -333,7 +333,7 @@ static double batch_rtol(int prec) { return prec == SEV_FP64 ? 1e-14 : 1e-9; }
 // order 1024..1300 62, 40, 25.5 and 18.7; two of order ~1050 17.5 and 9.6.
 // (The kernels of different lanes never wait on one another, and those that wait
 // within one launch make progress on any part of their grid or start together:
-// clusters, cooperative grids, the first four blocks of a band stage.)  A matrix
+// clusters and cooperative grids.)  A matrix
 // above kLaneMaxN fills the GPU with its own products and updates; it, a
 // caller's workspace, a capture and per-kernel timing take the handle's stream,
 // one matrix after another.

@@ -31,7 +31,7 @@
 // The same arithmetic per entry in both.  Roles publish their progress per sweep
 // with release stores; every wait is capped.  Each role takes sweeps from a
 // counter of its own in order, so the smallest unfinished sweep is always held
-// by running CTAs (blocks are dispatched in order: one CTA of each role runs).
+// by running CTAs (MULTI: the launch is cooperative, all roles run).
 //
 // T is never formed: with G = U^T U (a by-product of the QR's dot products) the
 // columns of U T follow from (U T) T^{-1} = U, T^{-1} = diag(1/tau) + striu(G),
@@ -941,8 +941,28 @@ int launch_step(sev_ctx *hd, int n, T *AB, int ldab, int b, int h, void *ws, siz
     P.ctr = P.flags + nflags - 8;
     P.ring = (T *)c.take<double>((size_t)step_slots(n, b, h) * kStepSets * StepDims(b, h).set_elems());
     SEV_CUDA(cudaMemsetAsync(P.flags, 0, sizeof(int) * nflags, hd->stream));
-    SEV_LAUNCH(hd, K_BAND_CHASE, kern, MULTI ? 4 * groups : groups, threads, smem, P);
-    return SEV_OK;
+    // The four CTAs of a sweep need one another, so they have to start together: a
+    // cooperative launch.  (Launched freely, some roles of a sweep could hold SMs
+    // while a cooperative grid on another stream -- a panel, a bisection -- held the
+    // rest and waited for these: neither went on until a wait ran out.  Clusters of
+    // four would do as well, but only 36 of them fit at once where 38 sweeps do:
+    // 128 -> 32 at n = 16384 47.0 ms against 45.7, 32 -> 16 at n = 3001 in FP64 24.7
+    // against 19.9, two CTAs of a cluster sharing an SM.)  One CTA per sweep goes on by
+    // itself, whatever part of the grid runs.
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.gridDim = dim3((unsigned)(MULTI ? 4 * groups : groups));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = hd->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = MULTI ? 1 : 0;
+    timing_begin(hd, K_BAND_CHASE);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P);
+    timing_end(hd, K_BAND_CHASE);
+    return e == cudaSuccess ? SEV_OK : SEV_ERR_CUDA;
 }
 
 }  // namespace sev
