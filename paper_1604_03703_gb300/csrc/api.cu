@@ -108,25 +108,25 @@ static bool capturing(cudaStream_t s) {
     return st != cudaStreamCaptureStatusNone;
 }
 
-void *get_copy(sev_ctx *h, size_t need, size_t bytes) {
+void *get_spare(sev_ctx *h, size_t need, size_t bytes) {
     if (bytes == 0) return nullptr;
     if (h->ws_ext) return h->ws_ext_bytes >= need + bytes ? (char *)h->ws_ext + need : nullptr;
-    if (h->copy_own_bytes < bytes) {
+    if (h->spare_own_bytes < bytes) {
         if (capturing(h->stream)) return nullptr;
-        if (h->copy_own) {
+        if (h->spare_own) {
             cudaStreamSynchronize(h->stream);
-            cudaFree(h->copy_own);
-            h->copy_own = nullptr;
-            h->copy_own_bytes = 0;
+            cudaFree(h->spare_own);
+            h->spare_own = nullptr;
+            h->spare_own_bytes = 0;
         }
-        if (cudaMalloc(&h->copy_own, bytes) != cudaSuccess) {
+        if (cudaMalloc(&h->spare_own, bytes) != cudaSuccess) {
             cudaGetLastError();
-            h->copy_own = nullptr;
+            h->spare_own = nullptr;
             return nullptr;
         }
-        h->copy_own_bytes = bytes;
+        h->spare_own_bytes = bytes;
     }
-    return h->copy_own;
+    return h->spare_own;
 }
 
 static int default_b0(int n, int prec) {
@@ -230,7 +230,7 @@ static int eigvalsh_t(sev_ctx *h, int n, T *A, int lda, int b0, double *eigs) {
     const size_t need = eig_workspace<T>(h, n, b0);
     int rc = get_workspace(h, need, &ws);
     if (rc) return rc;
-    T *const copy = (T *)get_copy(h, need, full_to_band_copy_bytes<T>(h, n, b0, A, lda));
+    T *const copy = (T *)get_spare(h, need, full_to_band_copy_bytes<T>(h, n, b0, A, lda));
     Carver c(ws);
     T *AB = c.take<T>((size_t)ldab * n);
     double *d = c.take<double>((size_t)n);
@@ -269,7 +269,7 @@ static int full_to_band_t(sev_ctx *h, int n, T *A, int lda, int b, T *AB, int ld
     void *ws = nullptr;
     int rc = get_workspace(h, need, &ws);
     if (rc) return rc;
-    T *const copy = (T *)get_copy(h, need, full_to_band_copy_bytes<T>(h, n, b, A, lda));
+    T *const copy = (T *)get_spare(h, need, full_to_band_copy_bytes<T>(h, n, b, A, lda));
     T *const work = copy ? copy : A;
     const int ldw = copy ? copy_ld(n) : lda;
     rc = launch_check_finite<T>(h, n, A, lda, nullptr, copy, ldw);
@@ -343,7 +343,7 @@ constexpr int kLaneMaxN = 4096;
 static void lanes_destroy(sev_ctx *h) {
     for (sev_ctx *l : h->lanes) {
         if (l->ws_own) cudaFree(l->ws_own);
-        if (l->copy_own) cudaFree(l->copy_own);
+        if (l->spare_own) cudaFree(l->spare_own);
         if (l->lane_event) cudaEventDestroy(l->lane_event);
         if (l->stream) cudaStreamDestroy(l->stream);
         delete l;
@@ -427,7 +427,7 @@ int sev_destroy(sev_handle h) {
     for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
     lanes_destroy(h);
     if (h->ws_own) cudaFree(h->ws_own);
-    if (h->copy_own) cudaFree(h->copy_own);
+    if (h->spare_own) cudaFree(h->spare_own);
     if (h->h_stage) cudaFree(h->h_stage);
     if (h->d_err) cudaFree(h->d_err);
     delete h;
@@ -557,9 +557,16 @@ int sev_band_to_band(sev_handle h, int n, void *AB, int ldab, int b, int hh, int
     const bool tri = hh == 1 && band_tri_supported(b, prec == SEV_FP64 ? 8 : 4);
     if (!tri && (prec == SEV_FP64 ? band_smem_bytes<double>(b, hh) : band_smem_bytes<float>(b, hh)) > h->smem_optin)
         return SEV_ERR_UNSUPPORTED;
-    const size_t need = tri ? band_tri_workspace(n) : band_workspace(n, b, hh);
+    size_t need = tri ? band_tri_workspace(n) : band_workspace(n, b, hh);
     void *ws = nullptr;
-    int rc = get_workspace(h, need, &ws);
+    const size_t have = h->ws_ext ? h->ws_ext_bytes : h->ws_own_bytes;
+    if (!tri && have < need && have >= band_chase_workspace(n, hh)) {
+        // the workspace at hand serves the general chase: it is not replaced, nor
+        // the call refused, for the exchange buffers of the faster kernel
+        if (!h->ws_ext) ws = get_spare(h, 0, need);
+        if (!ws) need = have;
+    }
+    int rc = ws ? SEV_OK : get_workspace(h, need, &ws);
     if (rc) return rc;
     return prec == SEV_FP64 ? band_stage<double>(h, n, (double *)AB, ldab, b, hh, ws, need)
                             : band_stage<float>(h, n, (float *)AB, ldab, b, hh, ws, need);
@@ -678,7 +685,7 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
             return rc;
         }
     }
-    if (!h->ws_ext) get_copy(h, 0, copy);
+    if (!h->ws_ext) get_spare(h, 0, copy);
     // lanes of the large matrices: largest first, each to the lane with the least
     // work so far (a reduction's time grows about as n^1.5 at these orders)
     int spread = 0;
@@ -699,7 +706,7 @@ int sev_batch_plan_create(sev_handle h, int count, const int *n, const int *lda,
         for (int l = 1; l < P->lanes && ok; ++l) {
             void *ws = nullptr;
             ok = get_workspace(h->lanes[l - 1], need[l], &ws) == SEV_OK;
-            if (ok) get_copy(h->lanes[l - 1], 0, copy[l]);
+            if (ok) get_spare(h->lanes[l - 1], 0, copy[l]);
         }
         if (!ok) P->lanes = 1;
     }

@@ -305,25 +305,31 @@ __global__ void __launch_bounds__(kThreads) band_chase_kernel(int n, T *AB, int 
     if (__syncthreads_or(bad) && threadIdx.x == 0) latch_error(err, SEV_ERR_INTERNAL);
 }
 
-size_t band_workspace(int n, int b, int h) {
+size_t band_chase_workspace(int n, int h) {
     Carver c(nullptr);
     c.take<int>((size_t)band_num_sweeps(n, h) + 1);
     c.take<int>(1);
-    const size_t step = band_step_workspace(n, b, h);
-    return c.bytes() > step ? c.bytes() : step;
+    return c.bytes();
+}
+size_t band_workspace(int n, int b, int h) {
+    const size_t chase = band_chase_workspace(n, h), step = band_step_workspace(n, b, h);
+    return chase > step ? chase : step;
 }
 
 template <typename T>
 int launch_band_to_band(sev_ctx *hd, int n, T *AB, int ldab, int b, int h, void *ws, size_t ws_bytes) {
     const int nsweeps = band_num_sweeps(n, h);
     if (nsweeps <= 0) return SEV_OK;
-    if (ws_bytes < band_workspace(n, b, h)) return SEV_ERR_WORKSPACE;
+    if (ws_bytes < band_chase_workspace(n, h)) return SEV_ERR_WORKSPACE;
     const size_t smem = band_smem_bytes<T>(b, h);
     if (smem > hd->smem_optin) return SEV_ERR_UNSUPPORTED;
-    // bands up to 128: the step kernel; this file's chase serves wider bands
-    // and the shapes the step kernel has no buffers for
-    const int rc = launch_band_step(hd, n, AB, ldab, b, h, ws, ws_bytes);
-    if (rc != SEV_ERR_UNSUPPORTED) return rc;
+    // bands up to 128: the step kernel; this file's chase serves wider bands, the
+    // shapes the step kernel has no buffers for, and a workspace without room
+    // for its exchange buffers
+    if (ws_bytes >= band_workspace(n, b, h)) {
+        const int rc = launch_band_step(hd, n, AB, ldab, b, h, ws, ws_bytes);
+        if (rc != SEV_ERR_UNSUPPORTED) return rc;
+    }
     Carver c(ws);
     int *progress = c.take<int>((size_t)nsweeps + 1);
     int *ctr = c.take<int>(1);
