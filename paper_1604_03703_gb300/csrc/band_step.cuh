@@ -751,6 +751,10 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
             T *const Zs = Xtra;
             for (int j = 1; j <= J; ++j) {
                 const int r0 = i * h + (j - 1) * b, m = min(n - r0, b);
+                // self-check: the step lies in the matrix, and there is a next one if and
+                // only if two rows or more are left for it (every access of all roles is
+                // bounded by the rows that n leaves, so a wrong count touches nothing else)
+                if (g.tid == 0 && (r0 < h || m < 2 || (j < J) != (n - r0 - b >= 2))) latch_error(P.err, SEV_ERR_INTERNAL);
                 if (i > 1 && !g.wait4(prev, 0, min(j + 1, Jp), min(j, Jp), min(j, Jp))) break;
                 // lower triangle, mirrored (zeros past m)
                 constexpr int U = RT == 4 ? 4 : 8;
