@@ -812,7 +812,7 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                     nc = w2 - min(half, w2);
                 }
             }
-            bool have = false;                // the set in shared memory is H_j's (MULTI)
+            bool have = false;  // the set in shared memory is H_j's (MULTI)
             for (int j = 1; j <= J; ++j) {
                 const int r0 = i * h + (j - 1) * b, m = min(n - (r0 + b), b);
                 if (i > 1 && !g.wait4(prev, min(j + 1, Jp), min(j + 1, Jp), min(j, Jp), min(j, Jp))) break;
@@ -845,25 +845,31 @@ __global__ void __launch_bounds__(MULTI ? kStepThreadsMulti : 3 * kStepThreadsRo
                         }
                         if (!g.sync_ok(failed)) break;
                     }
-                    auto c2 = [&](int a, int c, T v) {  // (columns counted from c_lo)
-                        if (sizeof(T) == 8 && c < 0) return;
-                        T &x = Ms[a + (c_lo + c) * ldb];
+                    auto c2 = [&](int a, int c, T v) {
+                        T &x = Ms[a + c * ldb];
                         x -= v;
-                        if (!next) AB[(b + a - c_lo - c) + (size_t)(r0 + c_lo + c) * ldab] = x;
+                        if (!next) AB[(b + a - c) + (size_t)(r0 + c) * ldab] = x;
                     };
                     // TN rows of U are read at once, from a multiple of TN on; other
                     // targets: FP64 starts before c_lo and drops what lies there, FP32 reads
-                    // single rows (starting early costs FP32 128 -> 32 2%, single
-                    // rows FP64 64 -> 16 3%, both without need)
-                    constexpr bool EARLY = sizeof(T) == 8;
-                    const int off = EARLY ? c_lo & (TN - 1) : 0;
-                    if (EARLY || c_lo % TN == 0)
+                    // single rows (starting early costs FP32 128 -> 32 2%, the other branch
+                    // FP64 64 -> 16 3%, both without need)
+                    if constexpr (sizeof(T) == 8) {
+                        const int off = c_lo & (TN - 1);
                         grp_outer<T, 4, TN, false, false>(g.tid, g.nt, m, nc + off, h, Ws, ldb, U0 + c_lo - off, ldb,
                                                           (const T *)nullptr, 0, (const T *)nullptr, 0,
-                                                          [&](int a, int c, T v) { c2(a, c - off, v); });
-                    else
+                                                          [&](int a, int c, T v) {
+                                                              if (c >= off) c2(a, c_lo - off + c, v);
+                                                          });
+                    } else if (c_lo % TN == 0) {
+                        grp_outer<T, 4, TN, false, false>(g.tid, g.nt, m, nc, h, Ws, ldb, U0 + c_lo, ldb,
+                                                          (const T *)nullptr, 0, (const T *)nullptr, 0,
+                                                          [&](int a, int c, T v) { c2(a, c_lo + c, v); });
+                    } else {
                         grp_outer<T, 4, 1, false, false>(g.tid, g.nt, m, nc, h, Ws, ldb, U0 + c_lo, ldb,
-                                                         (const T *)nullptr, 0, (const T *)nullptr, 0, c2);
+                                                         (const T *)nullptr, 0, (const T *)nullptr, 0,
+                                                         [&](int a, int c, T v) { c2(a, c_lo + c, v); });
+                    }
                     g.sync();
                     if (next) {
                         if (!need_set(j + 1, j)) break;
