@@ -219,6 +219,10 @@ def kernel_model(name, n, b0, elem, sched=None):
 # absent here reports null.
 MEASURED_TRAFFIC = {}
 
+# Kernels whose time is the chain of their steps (columns of a panel, steps of a
+# sweep pipeline), with a few per cent of the issue slots and no DRAM traffic.
+LATENCY_BOUND = ("panel_coop", "band_chase", "band_tri")
+
 
 def roofline(name, amount, unit, bound, ms_per_step, peaks, clocks, elem):
     if amount is None or ms_per_step <= 0:
@@ -638,6 +642,8 @@ def run_ours(args):
     roof = roofline(dominant, amount, unit, bound, dom_ms_step, peaks, clk, 4)
     if roof is not None:
         roof["kernel"] = dominant
+        if dominant in LATENCY_BOUND:
+            roof["note"] = "a chain of dependent steps, bound by their latency; the peak is for scale"
         traffic = MEASURED_TRAFFIC.get(dominant) if (n, b0) == (16384, 128) else None
         if traffic and traffic.get("schedule") != list(sched):
             traffic = None

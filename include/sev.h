@@ -6,9 +6,11 @@
  * "A communication-avoiding parallel algorithm for the symmetric eigenvalue
  * problem" (arXiv 1604.03703), on one GPU:
  *
- *   full-to-band    Algorithm 4.1 (tree QR of each panel, Algorithm 3.2;
- *                   compact-WY by Householder reconstruction, Cor. 3.7;
- *                   two-sided trailing update, Eq. 4.1)
+ *   full-to-band    Algorithm 4.1 (QR of each panel with its compact-WY form,
+ *                   by the whole GPU at once; panels that do not fit it take
+ *                   the tree QR of Algorithm 3.2 and the Householder
+ *                   reconstruction of Cor. 3.7; two-sided trailing update,
+ *                   Eq. 4.1)
  *   band-to-band    Algorithm 4.2 (bulge chasing, b -> h), repeated down
  *                   to the tridiagonal as in Algorithm 4.3
  *   tridiag_bisect  eigenvalues of the final tridiagonal by Sturm-count
@@ -122,9 +124,8 @@ int sev_eigvalsh_host(sev_handle handle, int n, const void *A_host, int lda, int
 
 /*
  * Full-to-band reduction (Algorithm 4.1, run right-looking): per panel of b
- * columns, tree QR of the trailing N x b panel (Algorithm 3.2), Householder
- * reconstruction of (U, T) (Cor. 3.7), W = A22 U, V from the V_1 formula,
- * A22 <- A22 + U V^T + V U^T (Eq. 4.1), band block <- S R.
+ * columns, QR of the trailing N x b panel with its (U, T), W = A22 U, V from
+ * the V_1 formula, A22 <- A22 + U V^T + V U^T (Eq. 4.1), band block <- R.
  *   A     device, n x n (lda), lower triangle read; on return A's lower
  *         triangle holds the band matrix (exact zeros below the band).
  *         A NaN or Inf in it latches SEV_ERR_NONFINITE (the reduction still
@@ -139,7 +140,10 @@ int sev_full_to_band(sev_handle handle, int n, void *A, int lda, int b, int prec
  * storage.  Requires h >= 1, h < b, b % h == 0, ldab >= 2b.  Entries of AB
  * at distance > b from the diagonal must be zero on entry; on return the
  * band has half-bandwidth h and entries beyond it are zero.  Sweeps run as
- * a persistent pipeline, sweep i two steps behind sweep i - 1.
+ * a persistent pipeline, sweep i two steps behind sweep i - 1 (three for bands
+ * over 128).  A caller's workspace of a few bytes per sweep is enough; bands of
+ * up to 128 run faster in one with room for the exchange buffers of a sweep
+ * pipeline, which the handle's own has.
  */
 int sev_band_to_band(sev_handle handle, int n, void *AB, int ldab, int b, int h, int prec);
 
@@ -209,14 +213,16 @@ int sev_tridiag_bisect_static(int n, const double *d, const double *e, double rt
  * sev_destroy) and synchronises; sev_batch_run only
  * enqueues work (no allocation, no host synchronisation) and may be
  * captured in a CUDA graph when every matrix runs in the batched launch
- * (sev_batch_plan_info reports large_count == 0).  Errors as sev_eigvalsh.
+ * (sev_batch_plan_info reports large_count == 0).  Errors as sev_eigvalsh: a
+ * matrix with a NaN or Inf gets NaN eigenvalues, the others are not affected.
  */
 typedef struct sev_batch_s *sev_batch_plan;
 int sev_batch_plan_create(sev_handle handle, int count, const int *n, const int *lda, void *const *A,
                           double *const *eigs, int b, int prec, sev_batch_plan *plan);
 int sev_batch_run(sev_handle handle, sev_batch_plan plan);
 int sev_batch_plan_destroy(sev_batch_plan plan);
-/* Band width, number of matrices in the batched launch, number run one by one. */
+/* Band width, number of matrices in the batched launch, number run through
+ * sev_eigvalsh (large_count). */
 int sev_batch_plan_info(sev_batch_plan plan, int *b, int *small_count, int *large_count);
 /* create + run + synchronise + destroy. */
 int sev_eigvalsh_batched(sev_handle handle, int count, const int *n, const int *lda, void *const *A, int b, int prec,

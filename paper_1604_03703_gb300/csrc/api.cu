@@ -129,9 +129,11 @@ void *get_spare(sev_ctx *h, size_t need, size_t bytes) {
     return h->spare_own;
 }
 
+// Widths without a tuned entry.  FP32 at n = 16384: 64 239 ms, 128 266, 32 292; at
+// n = 2048 64 and 32 16.1, 128 22.7; FP64 at n = 3001: 32 109, 64 127.
 static int default_b0(int n, int prec) {
     if (prec == SEV_FP64) return n >= 4096 ? 64 : 32;
-    return n >= 1024 ? 64 : 32;  // 64 -> 16 -> 1 measured best at n = 16384 (1.18 s against 1.51 s for 128)
+    return n >= 1024 ? 64 : 32;
 }
 
 // b0 for a call with b0 = 0: the autotuned width of the order's bucket if
@@ -142,14 +144,18 @@ static int pick_b0(const sev_ctx *h, int n, int prec) {
 }
 
 // Band schedule (Algorithm 4.3; the paper allows a reduction factor k > 2
-// per stage).  Measured on GB300 at n = 16384 (FP32): the one-stage b -> 1
-// kernel is fastest from b = 16 (192 ms, against 366 ms from 32), a
-// 32 -> 16 stage costs 139 ms, 64 -> 16 238 ms and 128 -> 32 372 ms (128 ->
-// 16 607 ms, 128 -> 64 312 ms).  So: a band of width <= 16 the b -> 1
-// kernel supports goes straight to 1; a band of 128 or more first goes to
-// 32; a wider band that 16 divides goes to 16; otherwise to the widest
-// supported width that divides it, or is halved; an odd band finishes with
-// b -> 1.  b0 = 128 gives 128 -> 32 -> 16 -> 1, b0 = 64 gives 64 -> 16 -> 1.
+// per stage): a band of width <= 16 the b -> 1 kernel supports goes straight to
+// 1; a band of 128 or more first goes to 32; a wider band that 16 divides goes
+// to 16; otherwise to the widest supported width that divides it, or is halved;
+// an odd band finishes with b -> 1.  b0 = 128 gives 128 -> 32 -> 16 -> 1, b0 = 64
+// gives 64 -> 16 -> 1.
+//
+// The rule is older than the kernels it now chooses among.  They take, in FP32
+// at n = 16384 (ms): 128 -> 32 45.8, 128 -> 16 49.4, 128 -> 8 69.9, 64 -> 16 33.4,
+// 64 -> 8 43.8, 32 -> 16 27.1, 32 -> 8 32.3, 32 -> 1 110, 16 -> 1 37.0, 8 -> 1 26.2; in
+// FP64 at n = 3001: 32 -> 16 19.9, 32 -> 8 20.2, 16 -> 1 23.3, 8 -> 1 15.4.  So at large
+// orders 128 -> 16 -> 1 is 23 ms (10% of a solve) faster than the rule's path, and 8 in
+// place of 16 gains 7 ms in FP64; sev_autotune finds such paths.
 static int schedule(int b0, int elem, int *out) {
     int k = 0;
     out[k++] = b0;

@@ -45,9 +45,10 @@
 // warp that first updates its column, then forms the reflector, with T's
 // recurrence in between.  A step of 128 -> 32: 45% of it the QR, then U T, M (U T)
 // and the loads.
-// Measured (GB300): 64 -> 16 at n = 8192, FP32: 48.1 -> 14.9 ms; 128 -> 32 and
-// 32 -> 16 together at n = 16384: 200 -> 72 ms; 32 -> 16 at n = 3001, FP64: 95.5
-// -> 19.8 ms; 32 -> 16 -> 8 -> 4 -> 2 at n = 512, FP64: 67.0 -> 14.8 ms.
+// Measured (GB300): 64 -> 16 at n = 8192, FP32: 48.1 -> 13.9 ms; 128 -> 32 and
+// 32 -> 16 together at n = 16384: 200 -> 72 ms; 128 -> 64 at n = 6000 44 -> 21 ms;
+// 32 -> 16 at n = 3001, FP64: 95.5 -> 19.8 ms; 32 -> 16 -> 8 -> 4 -> 2 at n = 512, FP64: 67.0
+// -> 14.8 ms.
 #pragma once
 #include "regtile.cuh"
 
@@ -222,26 +223,6 @@ __device__ __forceinline__ bool step_bar_or(int id, int nt, int stop) {
 }
 
 // ------------------------------------------------------------------- QR
-template <typename T, int Q, int H = Q / 2>
-__device__ __forceinline__ T step_sums(T (&d)[Q]) {  // sum of value lane >> (5 - log2 Q), transposing butterfly
-    const int lane = threadIdx.x & 31;
-    if constexpr (H >= 1) {
-        constexpr int OFF = 16 * 2 * H / Q;
-        const bool up = lane & OFF;
-#pragma unroll
-        for (int j = 0; j < H; ++j) {
-            const T keep = up ? d[j + H] : d[j], send = up ? d[j] : d[j + H];
-            d[j] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
-        }
-        return step_sums<T, Q, H / 2>(d);
-    } else {
-        T s = d[0];
-#pragma unroll
-        for (int o = 16 / Q; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
-        return s;
-    }
-}
-
 // Householder QR of the m x h block held by four warps (warp w, lane l:
 // a[q][t] = row l + 32 t of column w + 4 q; rows >= m and columns >= h zero), r =
 // min(m - 1, h) reflectors.  On return column c holds R on and above the
@@ -325,7 +306,7 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
             F2 p = two_prod((float)xr[0], (float)xr[0]);
 #pragma unroll
             for (int t = 1; t < RT; ++t) p = f2_add(p, two_prod((float)xr[t], (float)xr[t]));
-            const T sd = step_sums<T, Q>(d);
+            const T sd = warp_sums_t<T, Q>(d);
             const F2 ssq = warp_sum_f2(p);
 #pragma unroll
             for (int q = 0; q < Q; ++q) s[q] = __shfl_sync(0xffffffffu, sd, q * (32 / Q));
@@ -338,7 +319,7 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
 #pragma unroll
             for (int t = 1; t < RT; ++t) p = fma((double)xr[t], (double)xr[t], p);
             const double ssq = warp_sum(p);
-            const T sd = step_sums<T, Q>(d);
+            const T sd = warp_sums_t<T, Q>(d);
 #pragma unroll
             for (int q = 0; q < Q; ++q) s[q] = __shfl_sync(0xffffffffu, sd, q * (32 / Q));
             double td = 0.0, bd = 0.0, id = 0.0;

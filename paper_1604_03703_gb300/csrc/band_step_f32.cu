@@ -6,9 +6,9 @@ namespace sev {
 int launch_band_step(sev_ctx *hd, int n, float *AB, int ldab, int b, int h, void *ws, size_t ws_bytes) {
     if (!step_shape_ok(b, h)) return SEV_ERR_UNSUPPORTED;
     const int rt = step_rt(b), q = step_q(h);
-    // One CTA a sweep for narrow bands: 32 -> 16 at n = 8191 12.4 ms against
-    // 15.0 ms on four CTAs (a step's products are short, the exchange through
-    // global memory is not); 64 -> 16 at n = 8192 17.1 against 14.9 ms.
+    // One CTA a sweep for narrow bands: 32 -> 16 at n = 8191 11.5 ms against
+    // 14.4 ms on four CTAs (a step's products are short, the exchange through
+    // global memory is not); 64 -> 16 at n = 8192 16.7 against 13.9 ms.
     if (b < hd->chase_x3_min_b) {
         if (rt == 1 && q == 2) return launch_step<float, 1, 2, false>(hd, n, AB, ldab, b, h, ws, ws_bytes);
         if (rt == 1 && q == 4) return launch_step<float, 1, 4, false>(hd, n, AB, ldab, b, h, ws, ws_bytes);

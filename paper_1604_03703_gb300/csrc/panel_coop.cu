@@ -117,28 +117,6 @@ struct CoopComm {
     static __host__ __device__ size_t words(int b, int cmax) { return 2 * set_words(b, cmax) + ssq_words(cmax); }
 };
 
-// Warp sums of Q per-lane values by a transposing butterfly; the lane gets
-// the sum of value lane >> (5 - log2 Q).
-template <typename T, int Q, int H = Q / 2>
-__device__ __forceinline__ T warp_sums_t(T (&d)[Q]) {
-    const int lane = threadIdx.x & 31;
-    if constexpr (H >= 1) {
-        constexpr int OFF = 16 * 2 * H / Q;  // H = Q/2: 16, Q/4: 8, ...
-        const bool up = lane & OFF;
-#pragma unroll
-        for (int j = 0; j < H; ++j) {
-            const T keep = up ? d[j + H] : d[j], send = up ? d[j] : d[j + H];
-            d[j] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
-        }
-        return warp_sums_t<T, Q, H / 2>(d);
-    } else {
-        T s = d[0];
-#pragma unroll
-        for (int o = 16 / Q; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
-        return s;
-    }
-}
-
 // A failed try of a polling loop: true when the wait has to be given up.
 __device__ __forceinline__ bool coop_give_up(int tries, long long &t0, long long cap, int *err) {
     if (tries == 0) t0 = clock64();

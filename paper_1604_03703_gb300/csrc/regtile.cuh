@@ -180,6 +180,28 @@ __device__ __forceinline__ void warp_sums_x(float (&d)[Q]) {
     }
 }
 
+// Warp sums of Q per-lane values by a transposing butterfly; the lane gets
+// the sum of value lane >> (5 - log2 Q).
+template <typename T, int Q, int H = Q / 2>
+__device__ __forceinline__ T warp_sums_t(T (&d)[Q]) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (H >= 1) {
+        constexpr int OFF = 16 * 2 * H / Q;  // H = Q/2: 16, Q/4: 8, ...
+        const bool up = lane & OFF;
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            const T keep = up ? d[j + H] : d[j], send = up ? d[j] : d[j + H];
+            d[j] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+        }
+        return warp_sums_t<T, Q, H / 2>(d);
+    } else {
+        T s = d[0];
+#pragma unroll
+        for (int o = 16 / Q; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    }
+}
+
 // reg_apply for FP32 tiles of 2, 4, 8 or 16 columns per warp: the dot products
 // and the updates two columns per instruction (ffma2), the column sums by
 // warp_sums_x.

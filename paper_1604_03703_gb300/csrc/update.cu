@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) symm_kernel(int N, int b, const T *__rest
 // whichever orientation is contiguous (columns below the diagonal block,
 // rows -- A(m, k) = A(k, m) -- above it, transposed into shared memory),
 // and the K range split over blockIdx.z with per-split partial tiles
-// (summed in a fixed order by symm_reduce_kernel) so that every SM has work.
+// (summed in a fixed order by uty_kernel) so that every SM has work.
 // Needs lda % 4 == 0 and a 16-byte-aligned A22.
 constexpr int SBM = 128, SBN = 64, SBK = 16;
 
