@@ -43,11 +43,11 @@ __device__ __forceinline__ T tri_sum_row(T s) {
 }
 
 // tri_house for a column whose squares leave the range of its type, or a zero
-// one: the column is held times a power of two.  Beside larger entries an inexact tau
-// would spoil these, and in a matrix of that scale the column is not
+// one: the column is held times a power of two.  Beside larger entries an
+// inexact tau would spoil these, and in a matrix of that scale the column is not
 // negligible.  A function of its own: rare, and its registers stay out of the
-// steps (the test for it costs 0.3% of a solve: n = 3001 108.6 -> 108.9 ms
-// in FP64, 8191 rows of width 32 in FP32 43.3 ms as before).
+// steps.  (The test for it costs FP64 1-2% of the stage -- 16 -> 1 at n = 3001
+// 23.0 -> 23.2 ms -- and FP32 nothing.)
 template <typename T>
 struct TriHouse {
     T v, tau, beta;
