@@ -276,7 +276,10 @@ static double pow2(int k) /* exact 2^k for -1022 <= k <= 1023 */
  * scaled off-diagonal; each step is u = e2s_{i-1} p_{i-1} followed by
  * p_{i+1} = fma(d_i - x, p_i, -u).  A minor equal to zero takes the sign
  * opposite to its predecessor (it counts as a change, as a zero pivot does
- * under the pivmin rule).  Whenever |p_i| leaves [2^-256, 2^256] the pair
+ * under the pivmin rule).  Two zero minors in a row mean that T splits (e is zero
+ * or negligible) behind a block that is singular at x: all further minors of
+ * the whole vanish, and the count goes on with the minors of the rest, 1, t, ...
+ * Whenever |p_i| leaves [2^-256, 2^256] the pair
  * (p_{i-1}, p_i) is rescaled by the power of two 2^k, k = clamp(-exponent,
  * -512, 512), bringing p_i to [1, 2): signs are unchanged and nothing
  * overflows for a scaled matrix (|d_i - x| <= 2, e2s <= 1).
@@ -290,6 +293,11 @@ int orc_sturm_minors(int n, const double *d, const double *e2s, double sc, doubl
         double t = fma(d[i], sc, -x);
         double u = e2s[i - 1] * a;
         double p = fma(t, b, -u);
+        if (p == 0.0 && b == 0.0) {
+            p = t;
+            b = 1.0;
+            neg = 0;
+        }
         int pn = (p < 0.0) || (p == 0.0 && !neg);
         c += pn != neg;
         neg = pn;

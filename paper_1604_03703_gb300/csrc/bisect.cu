@@ -10,7 +10,8 @@
 // the division-free form of the LDL^T pivot count: per step one FMA on the
 // dependence chain (instead of a ~1000-cycle FP64 division), the pair
 // (p_{i-1}, p_i) rescaled by a power of two when |p_i| leaves
-// [2^-256, 2^256], a zero minor counted as a sign change.  Every FP64
+// [2^-256, 2^256], a zero minor counted as a sign change, the recurrence begun
+// anew after two of them in a row (T splits behind a singular block).  Every FP64
 // operation is written with an explicit round-to-nearest intrinsic so no
 // multiply-add is contracted: the result is the exact IEEE evaluation of the
 // recurrence in the order written.

@@ -14,13 +14,22 @@ __device__ __forceinline__ double pow2_exact(int k) {  // 2^k, -1022 <= k <= 102
 // One step of the minors recurrence with t = d_i sc - x: u = e_{i-1}^2 a,
 // p = t b - u; sign, zero test and exponent from the bits (integer work, so
 // the FP64 pipe sees only the three operations), rescaling by a power of two
-// when |p| leaves [2^-256, 2^256].
+// when |p| leaves [2^-256, 2^256].  Two zero minors in a row: T splits here (e is
+// zero, or negligible) behind a block that is singular at x, all further
+// minors of the whole would vanish, and the count goes on with those of the
+// rest by itself (1, t, ...).
 __device__ __forceinline__ void sturm_step(double di, double e2i, double x, double sc, double &a, double &b,
                                            bool &neg, int &c) {
     const double t = __fma_rn(di, sc, -x);
     const double u = __dmul_rn(e2i, a);
-    const double p = __fma_rn(t, b, -u);
-    const long long pb = __double_as_longlong(p);
+    double p = __fma_rn(t, b, -u);
+    long long pb = __double_as_longlong(p);
+    if (((pb | __double_as_longlong(b)) << 1) == 0) {
+        p = t;
+        pb = __double_as_longlong(p);
+        b = 1.0;
+        neg = false;
+    }
     const bool zero = (pb << 1) == 0;
     const bool pn = zero ? !neg : pb < 0;
     c += pn != neg;
@@ -51,7 +60,8 @@ __device__ __forceinline__ void sturm_step(double di, double e2i, double x, doub
 // than 2^2 a step, so nothing overflows.  `plain` says that no nonzero e_i^2
 // is below 2^-322; then u does not underflow while every |p| of the block and
 // before it is >= 2^-700.  A block with a smaller |p| (or p = 0, whose sign is
-// defined by its predecessor) is run again step by step from where it began.
+// defined by its predecessor, and behind which T may split) is run again step by
+// step from where it began.
 // Blocks of 8 in the single-matrix kernels (16384 eigenvalues at 1e-14: U = 4
 // 79.2 ms, 8 76.5, 16 spills; 118.3 with the branch in every step), of 4 in the
 // batched kernel, whose other phases need the registers.
