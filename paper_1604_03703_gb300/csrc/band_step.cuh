@@ -237,8 +237,10 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
     constexpr bool PACK = sizeof(T) == 4 && RT != 2;
     const int lane = threadIdx.x & 31;
     const int r = m - 1 < h ? (m - 1 > 0 ? m - 1 : 0) : h;
-    // the largest entry: x is held times its power of two, so that no square or
-    // product that matters over- or underflows
+    // the largest entry: the block is held times its power of two, so that no
+    // square or product that matters over- or underflows.  (All of it, not x alone:
+    // x may be 1e-140 of it, x^T a is multiplied by 1 / (alpha - beta) afterwards,
+    // and with a at 1e-190 as it came x^T a had underflowed before.)
     T mx = T(0);
 #pragma unroll
     for (int q = 0; q < Q; ++q)
@@ -264,9 +266,13 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
         scale = pow2i(-e);
         unscale = pow2i(e);
     }
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int t = 0; t < RT; ++t) a[q][t] *= scale;
     if (w == 0) {
 #pragma unroll
-        for (int t = 0; t < RT; ++t) xs[lane + 32 * t] = a[0][t] * scale;
+        for (int t = 0; t < RT; ++t) xs[lane + 32 * t] = a[0][t];
     }
     step_bar(bar, 128);
     for (int k = 0; k < r; ++k) {
@@ -326,7 +332,6 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
             if (fma((double)alpha, (double)alpha, ssq) >= 1e-280) house_scalars((double)alpha, ssq, &td, &bd, &id);
             tk = (T)td, beta = (T)bd, inv = (T)id;
         }
-        beta *= unscale;
         T v[RT], ms[Q];
 #pragma unroll
         for (int t = 0; t < RT; ++t) v[t] = lane + 32 * t == k ? T(1) : xr[t] * inv;
@@ -357,7 +362,7 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
                 for (int q = 0; q < Q; ++q)
                     if ((pick >> q) & 1) {
 #pragma unroll
-                        for (int t = 0; t < RT; ++t) xn[lane + 32 * t] = lane + 32 * t >= k1 ? a[q][t] * scale : T(0);
+                        for (int t = 0; t < RT; ++t) xn[lane + 32 * t] = lane + 32 * t >= k1 ? a[q][t] : T(0);
                     }
             }
             if ((k & 3) == w) {
@@ -389,13 +394,18 @@ __device__ __forceinline__ int step_qr(int w, T (&a)[Q][RT], int m, int h, T *xs
                     T x = a[0][t];
 #pragma unroll
                     for (int q = 1; q < Q; ++q) x = (pick >> q) & 1 ? a[q][t] : x;
-                    xn[lane + 32 * t] = lane + 32 * t >= k1 ? x * scale : T(0);
+                    xn[lane + 32 * t] = lane + 32 * t >= k1 ? x : T(0);
                 }
             }
         }
         if (w == 0 && lane == 0) tau[k] = tk;
         step_bar(bar, 128);
     }
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int t = 0; t < RT; ++t)
+            if (lane + 32 * t <= w + 4 * q) a[q][t] *= unscale;
     return r;
 }
 

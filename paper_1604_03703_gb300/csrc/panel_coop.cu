@@ -22,8 +22,10 @@
 // x^T x and of x^T a_j for ALL columns j before tau and beta are known; for
 // finished columns j < k the same expression is G(j, k) = v_j^T v_k, from
 // which the last CTA forms the compact-WY factor T while it waits for the
-// next exchange.  x is held times the power of two of the panel's largest
-// entry (exact); x^T x of FP32 data is summed error-free in pairs of floats.
+// next exchange.  The panel is held times the power of two of its largest entry
+// (exact; not x alone: x may be 1e-140 of it, and x^T a_j must not underflow before
+// it is divided by alpha - beta); x^T x of FP32 data is summed error-free in pairs
+// of floats.
 //
 // Exchange.  Every value travels as one 8-byte word (FP64: two) holding the
 // 32 bits and a tag (panel and column), stored and polled with single 8-byte
@@ -224,12 +226,12 @@ __device__ __forceinline__ bool coop_poll_pairs(const unsigned long long *p, int
 
 template <typename T, int RT>
 struct CoopSmem {
-    T xs[2][32 * RT];          // scale times column k below row k
+    T xs[2][32 * RT];          // column k below row k
     T sd[kCoopMaxB], sr[kCoopMaxB];  // x^T a_j and row k of the column being formed
     T gs[kCoopMaxB];           // G(j, k), j < k (last CTA)
     T part[16 * 32];           // partial sums of a column of T (last CTA)
     T tau[kCoopMaxB];
-    T sc[4];                   // tau, beta, 1 / (scale (alpha - beta)) of the column; the panel's scale
+    T sc[4];                   // tau, beta, 1 / (alpha - beta) of the column; the panel's scale
     int abort;
 };
 
@@ -318,8 +320,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
     if (threadIdx.x == 0) S.abort = 0;
     if (lastc)
         for (int i = threadIdx.x; i < b * b; i += blockDim.x) Ts[i] = T(0);
-    // The panel's largest entry: x is held times its power of two, so that no
-    // square or product that matters over- or underflows.
+    // The panel's largest entry: the panel is held times its power of two, so that
+    // no square or product that matters over- or underflows.
     {
         double m = 0.0;
         if (warp < NW) {
@@ -358,9 +360,15 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
     __syncthreads();
     const T scale = S.sc[3], unscale = T(1) / scale;
     bool alive = !S.abort;
+    if (warp < NW) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int t = 0; t < RT; ++t) a[q][t] *= scale;
+    }
     if (warp == 0) {
 #pragma unroll
-        for (int t = 0; t < RT; ++t) S.xs[0][lane + 32 * t] = row0 + lane + 32 * t > 0 ? a[0][t] * scale : T(0);
+        for (int t = 0; t < RT; ++t) S.xs[0][lane + 32 * t] = row0 + lane + 32 * t > 0 ? a[0][t] : T(0);
     }
     __syncthreads();
 
@@ -452,7 +460,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                                                           const F2 v{__uint_as_float(hi), __uint_as_float(lo)};
                                                           acc = first ? v : f2_add(acc, v);
                                                       });
-                alpha = __shfl_sync(0xffffffffu, alpha, 0) * (float)scale;
+                alpha = __shfl_sync(0xffffffffu, alpha, 0);
                 acc = warp_sum_f2(acc);
                 float tau = 0.f, beta = 0.f, inv = 0.f;
                 // a column 1e-16 times smaller than the panel's largest entry is a
@@ -460,7 +468,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                 if (fmaf(alpha, alpha, acc.hi) >= 1e-32f) house_scalars_f2(alpha, acc, &tau, &beta, &inv);
                 if (lane == 0) {
                     S.sc[0] = (T)tau;
-                    S.sc[1] = (T)(beta * (float)unscale);
+                    S.sc[1] = (T)beta;
                     S.sc[2] = (T)inv;
                     S.tau[k] = (T)tau;
                 }
@@ -481,14 +489,13 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                                                        });
                 acc = warp_sum(acc);
                 alpha = __shfl_sync(0xffffffffu, alpha, 0);
-                const double as = alpha * (double)scale;
                 double tau = 0.0, beta = 0.0, inv = 0.0;
                 // a column 1e-140 times smaller than the panel's largest entry is a
                 // zero column (its square could not be told from underflow)
-                if (fma(as, as, acc) >= 1e-280) house_scalars(as, acc, &tau, &beta, &inv);
+                if (fma(alpha, alpha, acc) >= 1e-280) house_scalars(alpha, acc, &tau, &beta, &inv);
                 if (lane == 0) {
                     S.sc[0] = (T)tau;
-                    S.sc[1] = (T)(beta * (double)unscale);
+                    S.sc[1] = (T)beta;
                     S.sc[2] = (T)inv;
                     S.tau[k] = (T)tau;
                 }
@@ -554,7 +561,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                     if ((pick >> q) & 1) {
 #pragma unroll
                         for (int t = 0; t < RT; ++t)
-                            xn[lane + 32 * t] = row0 + lane + 32 * t > k1 ? a[q][t] * scale : T(0);
+                            xn[lane + 32 * t] = row0 + lane + 32 * t > k1 ? a[q][t] : T(0);
                     }
             }
         } else if (lastc && k >= 1) {
@@ -588,7 +595,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                 T v = T(0);
                 if (j < nref) v = g < j ? T(0) : (g == j ? T(1) : a[q][t]);
                 U[(size_t)g + (size_t)j * N] = v;
-                P[(size_t)g + (size_t)j * ldp] = g <= j ? a[q][t] : T(0);
+                P[(size_t)g + (size_t)j * ldp] = g <= j ? a[q][t] * unscale : T(0);
             }
     }
 }

@@ -138,3 +138,74 @@ def test_tree_panels_with_tiny_couplings(monkeypatch, dt, c):
             assert np.all(np.isfinite(band)), (b, k)
             assert np.abs(np.linalg.eigvalsh(band) - np.linalg.eigvalsh(A)).max() <= bound(n, dt, A), (b, k)
     h.close()
+
+
+# a matrix far from order one whose columns are far smaller still: x^T a of a block
+# that is not held scaled underflows before 1 / (alpha - beta) brings it back
+BOTH = [("float64", 1e-170, 1e-130), ("float64", 1e-190, 1e-120), ("float64", 1e-190, 1e-135), ("float64", 1e-230, 1e-75),
+        ("float64", 1e200, 1e-135), ("float32", 1e-22, 1e-14), ("float32", 1e-26, 1e-12), ("float32", 1e-30, 1e-7), ("float32", 1e25, 1e-14)]
+
+
+@pytest.mark.parametrize("b,h", [(8, 2), (32, 16), (64, 16), (64, 32), (96, 32), (128, 16)])
+@pytest.mark.parametrize("dt,scale,c", BOTH)
+def test_band_steps_with_both(H, dt, scale, c, b, h):
+    import torch
+
+    n = 3 * b + 20
+    A = couple(I.random_band(n, b, 17500 + b + h), [1, h, h + 1, b, b + 3, 2 * b + 1], c) * scale
+    AB = torch.from_numpy(np.ascontiguousarray(I.dense_to_band(A, 2 * b).T)).to(getattr(torch, dt)).cuda()
+    A = I.band_to_dense(AB.double().cpu().numpy().T) / scale
+    H.band_to_band(AB, b, h)
+    H.raise_device_error()
+    G = I.band_to_dense(AB.double().cpu().numpy().T) / scale
+    assert np.abs(np.linalg.eigvalsh(G) - np.linalg.eigvalsh(A)).max() <= bound(n, dt, A)
+
+
+@pytest.mark.parametrize("n,b", [(90, 8), (300, 32), (300, 64), (1300, 16), (2300, 64)])
+@pytest.mark.parametrize("dt,scale,c", BOTH)
+def test_panels_with_both(H, dt, scale, c, n, b):
+    """One cluster and the whole GPU (FP64 over 1024 rows)."""
+    import torch
+
+    if n == 2300 and dt == "float64":
+        pytest.skip("an order is enough")
+    A = couple(I.semicircle(n, 17600 + n), [1, b, b + 1, 2 * b + 5, n - 3], c) * scale
+    t = torch.from_numpy(A).to(getattr(torch, dt))
+    A = t.double().numpy() / scale
+    G = I.band_to_dense(H.full_to_band(t.cuda(), b).double().cpu().numpy().T) / scale
+    H.raise_device_error()
+    assert np.abs(np.linalg.eigvalsh(G) - np.linalg.eigvalsh(A)).max() <= bound(n, dt, A)
+
+
+@pytest.mark.parametrize("n,b,h", [(816, 110, 22), (700, 64, 16), (600, 32, 16), (800, 128, 16), (500, 16, 4), (900, 48, 24)])
+@pytest.mark.parametrize("k", [-540, -600, -634, -680])
+def test_sparse_bands_far_below_one(H, k, n, b, h):
+    """Few entries: the columns left by earlier sweeps are rounding errors of rounding
+    errors, 2^-53, 2^-106, ... of their block, down to the end of the range."""
+    import torch
+
+    for seed in range(4):
+        r = I.rng(19000 + 10 * b + seed)
+        A = np.where(r.random((n, n)) < 0.03, r.standard_normal((n, n)), 0.0)
+        A = np.tril(A) + np.tril(A, -1).T
+        i, j = np.indices(A.shape)
+        A[np.abs(i - j) > b] = 0.0
+        AB = torch.from_numpy(np.ascontiguousarray(I.dense_to_band(A * 2.0**k, 2 * b).T)).cuda()
+        H.band_to_band(AB, b, h)
+        H.raise_device_error()
+        G = I.band_to_dense(AB.cpu().numpy().T) / 2.0**k
+        assert np.abs(np.linalg.eigvalsh(G) - np.linalg.eigvalsh(A)).max() <= bound(n, "float64", A), seed
+
+
+@pytest.mark.parametrize("n,b", [(300, 32), (816, 64), (1300, 16)])
+@pytest.mark.parametrize("k", [-540, -600, -634, -680])
+def test_sparse_matrices_far_below_one(H, k, n, b):
+    import torch
+
+    for seed in range(3):
+        r = I.rng(19100 + 10 * b + seed)
+        A = np.where(r.random((n, n)) < 2.0 / n, r.standard_normal((n, n)), 0.0)
+        A = np.tril(A) + np.tril(A, -1).T
+        G = I.band_to_dense(H.full_to_band(torch.from_numpy(A * 2.0**k).cuda(), b).cpu().numpy().T) / 2.0**k
+        H.raise_device_error()
+        assert np.abs(np.linalg.eigvalsh(G) - np.linalg.eigvalsh(A)).max() <= bound(n, "float64", A), seed
